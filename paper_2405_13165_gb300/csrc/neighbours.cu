@@ -270,9 +270,9 @@ __global__ void k_clear_cells(const GridDev *g, int32_t *cell_start, int32_t *ce
                               int32_t *n_ucell) {
   if (!g->ok) return;
   const long long nc = g->ncells;
-  // occupied cells, overflow cells, and the work tickets of the mask and fill kernels
+  // cell counts, overflow items, the work tickets and the mask pool's counter
   if (blockIdx.x == 0 && threadIdx.x == 0)
-    n_ucell[0] = n_ucell[1] = n_ucell[2] = n_ucell[3] = n_ucell[4] = 0;
+    for (int k = 0; k < 8; ++k) n_ucell[k] = 0;
   for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < nc;
        k += (long long)gridDim.x * blockDim.x) {
     cell_start[k] = INT_MAX;
@@ -415,19 +415,20 @@ constexpr int kNbrThreads = 128;
 constexpr int kNbrSmemBytes = 32768;
 
 // Warp-per-particle count / fill (ballot compaction), for the occupied cells
-// listed in sel[0 .. *n_sel): the cells whose 27-cell candidate union does not
-// fit the shared-memory tile of the mask kernel below.
+// listed in sel[0 .. *n_sel): the work items (a cell, or a part of its particles)
+// that the mask kernel below cannot hold.
 struct CloudGrids;
+__device__ __forceinline__ void item_part(int P, int split, int c, int *p0, int *np);
 __device__ __forceinline__ void cell_runs(int key, const CloudGrids &cg,
                                           const int32_t *cell_start, const int32_t *cell_end,
                                           int r, int *lo_out, int *len_out);
 
 template <typename T, bool FILL>
 __global__ void __launch_bounds__(kNbrThreads) k_nbr(
-    CloudGrids cg, const int32_t *ucell, const int32_t *sel, const int32_t *n_sel,
-    const vec4_t<T> *spos, const int32_t *svals, const int32_t *cell_start,
-    const int32_t *cell_end, int32_t *counts, const long long *row_ptr, int32_t *col,
-    long long cap_nnz, int64_t n) {
+    CloudGrids cg, const int32_t *ucell, const int32_t *n_ucell, int split, const int32_t *sel,
+    const int32_t *n_sel, const vec4_t<T> *spos, const int32_t *svals,
+    const int32_t *cell_start, const int32_t *cell_end, int32_t *counts,
+    const long long *row_ptr, int32_t *col, long long cap_nnz, int64_t n) {
   using V = vec4_t<T>;
   constexpr int CAP = kNbrSmemBytes / sizeof(V);
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -439,9 +440,12 @@ __global__ void __launch_bounds__(kNbrThreads) k_nbr(
   const unsigned lt = (1u << lane) - 1u;
   const int nu = *n_sel;
   for (int cs = blockIdx.x; cs < nu; cs += gridDim.x) {
-    const int cb = sel[cs];
-    const int key = ucell[2 * cb], s0 = ucell[2 * cb + 1];
-    const int s1 = cell_end[key];
+    const int cb = cell_slot(sel[cs] / split, n_ucell[0], n);
+    const int key = ucell[2 * cb];
+    int s0 = ucell[2 * cb + 1], part, np;
+    item_part(cell_end[key] - s0, split, sel[cs] % split, &part, &np);
+    s0 += part;
+    const int s1 = s0 + np;
     if (threadIdx.x < 9)
       cell_runs(key, cg, cell_start, cell_end, threadIdx.x, &r_lo[threadIdx.x], &r_len[threadIdx.x]);
     __syncthreads();
@@ -498,42 +502,63 @@ __global__ void k_check_nnz(const long long *row_ptr, int64_t n, long long cap_n
 // ------------------------------------------------ warp-per-cell mask path
 // Every particle of a cell shares the candidate set "27 cells around it",
 // which is 9 runs of consecutive sorted positions (3 x-adjacent cells each).
-// Each warp takes occupied cells from a device work queue (an atomic ticket
-// per cell) and handles its cell alone, with warp-level synchronisation only:
-// a film cell (a dozen particles, ~4 candidate words) and a 3D cell (~40
-// particles, ~37 words) then cost the warp in proportion to their work, and
-// no block waits at a barrier for its slowest thread.  The candidates are
-// staged in windows of kWinWords words (32 candidates each) in the warp's part
-// of shared memory; the warp's lanes take (word, particle) items of the window
-// (consecutive lanes, consecutive particles of one word: the candidate reads
-// are broadcasts), test 32 candidates against the particle and write one bit
-// per candidate (word-major mask[w * stride + p], coalesced) plus the row
-// length.  The fill kernel turns the bits back into column indices, so the
-// distance tests run once.
+// Each warp takes work items -- an occupied cell, or one of `split` parts of
+// its particles -- from a device work queue (an atomic ticket per item) and
+// handles its item alone, with warp-level synchronisation only: a film cell (a
+// dozen particles, ~4 candidate words) and a 3D cell (~40 particles, ~37
+// words) then cost the warp in proportion to their work, and no block waits at
+// a barrier for its slowest thread.  The candidates are staged in windows of
+// kWinWords words (32 candidates each) in the warp's part of shared memory;
+// the warp's lanes take (word, particle) pairs of the window (consecutive
+// lanes, consecutive particles of one word: the candidate reads are
+// broadcasts), test 32 candidates against the particle and write one bit per
+// candidate plus the row length.  The fill kernel turns the bits back into
+// column indices, so the distance tests run once.
+//
+// The test is one packed dot product.  With u = (x - x_ref) sc, x_ref a particle
+// of the item's cell and sc the power of two that takes the cell edge c into
+// [1/2, 1),
+//   |u_j - u_i|^2 - (h_i + h_j)^2 / 4
+//     = (|u_j|^2 - h_j^2/4) + (|u_i|^2 - h_i^2/4) - 2 u_i.u_j - (h_i/2) h_j,
+// a sum and four fused multiply-adds per candidate (two candidates per packed
+// FP32 instruction) on staged (u_j, h_j, |u_j|^2 - h_j^2/4), against eleven
+// operations for the difference form; its sign is the bit (a funnel shift).
+// FP32 evaluates it to 1.3e-5 (|u_i| <= 1, |u_j| <= 2 per axis, partial sums up
+// to 28: ten roundings of at most 2^-24 each, and 1.3e-6 from the rounded
+// u), so a value within kBand of zero is decided by the FP64 definition on the
+// original positions instead -- for FP64 clouds too, whose tests all ran on
+// the FP64 pipe before.  One word in 5000 needs that.
+//
+// The bits of an item go to a pool, nwords x P words from an atomic counter
+// (pool_words in all, kMaskWords per particle of the context's capacity on
+// average): film cells need 4 words per particle, cells of an irregular cloud
+// 60, and only what exceeds the pool takes the warp-per-particle kernel.
 constexpr int kMaskThreads = 128;
 constexpr int kMaskWarps = kMaskThreads / 32;
-constexpr int kMaskMaxP = 256;   // particles of one cell in the mask kernel (else: overflow path)
+constexpr int kMaskMaxP = 256;   // particles of one item in the mask kernel (else: overflow path)
 static_assert(kMaskCap < 65536 && kMaskMaxP % 2 == 0, "two 16-bit hit counts per word");
-// FP32 window: four arrays (x, y, z, h/2) of kWinWords words, two pad floats
-// per word: a float2 read gives two consecutive candidates, and the words that
-// lanes of one warp test sit in different banks.  FP64: double4 records, one
-// pad record per word.
-template <typename T> struct MaskWin;
-template <> struct MaskWin<float> {
-  static constexpr int WORDS = 11;
-  static constexpr int SOA = 32 * WORDS + 2 * WORDS;   // floats per array
-  static constexpr int TILE_BYTES = 4 * SOA * (int)sizeof(float);
-};
-template <> struct MaskWin<double> {
-  static constexpr int WORDS = 5;
-  static constexpr int TILE_BYTES = (32 * WORDS + WORDS) * (int)sizeof(double4_16a);
-};
-template <typename T>
-constexpr int kMaskWarpBytes = MaskWin<T>::TILE_BYTES + (kMaskMaxP / 2) * (int)sizeof(unsigned);
+constexpr int kWinWords = 8;
+constexpr float kBand = 1.6e-5f;
+// A window's words: pairs of candidates as (x0, x1, y0, y1) and (z0, z1, h0, h1)
+// (16 pairs and 16 pad bytes per word, so that words tested by lanes of one warp
+// sit in different banks), and (c0, c1).
+constexpr int kWinA = 68, kWinC = 36;   // floats per word
+constexpr int kWinFloats = kWinWords * (2 * kWinA + kWinC);
+constexpr int kMaskWarpBytes = kWinFloats * (int)sizeof(float) +
+                               (kMaskMaxP / 2) * (int)sizeof(unsigned) + 20 * (int)sizeof(int);
+static_assert(kMaskWarpBytes % 16 == 0, "16-byte aligned windows");
 
 constexpr int kFillThreads = 128;
 constexpr int kFillWarps = kFillThreads / 32;
 constexpr int kFillWinWords = 16;   // candidate words of one fill window
+constexpr int kFillRec = kFillWinWords + 2;   // records of one particle, with pad
+
+// Particles [*p0, *p0 + *np) of the cell that part `c` of `split` holds.
+__device__ __forceinline__ void item_part(int P, int split, int c, int *p0, int *np) {
+  const int q = (P + split - 1) / split;
+  *p0 = min(P, c * q);
+  *np = min(P, *p0 + q) - *p0;
+}
 
 // Rows of the 27-cell neighbourhood of global cell `key`: run r (dz = r/3-1,
 // dy = r%3-1) covers cells key-1..key+1 of that (y, z) row of the key's own
@@ -597,173 +622,220 @@ __device__ __forceinline__ void for_window(int lo, int len, int off, int c0, int
   }
 }
 
-// FP32 test with an explicit band: certainly in / certainly out from FP32,
-// the FP64 definition inside +-1e-5 of the bound.
-__device__ __forceinline__ bool support_test(const float4 &a, const float4 &b) {
-  const float dx = b.x - a.x, dy = b.y - a.y, dz = b.z - a.z;
-  const float d2 = (dx * dx + dy * dy) + dz * dz;
-  const float r = (a.w + b.w) * 0.5f;
-  const float r2 = r * r;
-  if (d2 < r2 * 0.99999f) return true;
-  if (d2 > r2 * 1.00001f) return false;
-  return in_support64(a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w);
+// The power of two that takes the cell edge of the cloud of global cell `key`
+// into [1/2, 1).
+__device__ __forceinline__ double cell_scale(int key, const CloudGrids &cg) {
+  int b0 = 0, b1 = cg.nb;
+  while (b1 - b0 > 1) {
+    const int mid = (b0 + b1) >> 1;
+    if (cg.cell_base[mid] <= key) b0 = mid; else b1 = mid;
+  }
+  int e;
+  frexp(cg.grids[b0].c, &e);
+  return ldexp(1.0, -max(-120, min(120, e)));
 }
-__device__ __forceinline__ bool support_test(const double4_16a &a, const double4_16a &b) {
-  return in_support64(a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w);
+
+// (x - ref) sc in FP32: the subtraction in the input's own type, sc exact.
+__device__ __forceinline__ float4 local_of(const float4 &v, const float4 &r, double sc) {
+  const float s = (float)sc;
+  return make_float4((v.x - r.x) * s, (v.y - r.y) * s, (v.z - r.z) * s, v.w * s);
+}
+__device__ __forceinline__ float4 local_of(const double4_16a &v, const double4_16a &r, double sc) {
+  return make_float4((float)((v.x - r.x) * sc), (float)((v.y - r.y) * sc),
+                     (float)((v.z - r.z) * sc), (float)(v.w * sc));
+}
+// |u|^2 - h^2/4
+__device__ __forceinline__ float local_c(const float4 &u) {
+  return fmaf(u.x, u.x, fmaf(u.y, u.y, fmaf(u.z, u.z, -0.25f * u.w * u.w)));
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
     CloudGrids cg, const int32_t *ucell, int32_t *n_ucell, const vec4_t<T> *spos,
     const int32_t *svals, const int32_t *cell_start, const int32_t *cell_end, int32_t *counts,
-    uint32_t *mask, int64_t stride, int32_t *overflow, int32_t *n_overflow, int64_t n) {
+    uint32_t *mask, long long pool_words, long long *mask_off, int split, int32_t *overflow,
+    int32_t *n_overflow, int64_t n) {
   using V = vec4_t<T>;
-  constexpr int WW = MaskWin<T>::WORDS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  unsigned char *mine = smem_raw + wp * kMaskWarpBytes<T>;
-  V *cand = reinterpret_cast<V *>(mine);
-  float *tx = reinterpret_cast<float *>(mine);
-  float *ty = tx + (sizeof(T) == 4 ? MaskWin<float>::SOA : 0);
-  float *tz = ty + (sizeof(T) == 4 ? MaskWin<float>::SOA : 0);
-  float *th = tz + (sizeof(T) == 4 ? MaskWin<float>::SOA : 0);
+  float *ta = reinterpret_cast<float *>(smem_raw + wp * kMaskWarpBytes);
+  float *tb = ta + kWinWords * kWinA, *tc = tb + kWinWords * kWinA;
   // per-particle hit counts, two 16-bit counts per word (a row has at most
-  // kMaskCap < 65536 candidates)
-  unsigned *cnt = reinterpret_cast<unsigned *>(mine + MaskWin<T>::TILE_BYTES);
+  // kMaskCap < 65536 candidates); the runs' starts and offsets (FP64 retakes)
+  unsigned *cnt = reinterpret_cast<unsigned *>(tc + kWinWords * kWinC);
+  int *run_lo = reinterpret_cast<int *>(cnt + kMaskMaxP / 2), *run_off = run_lo + 10;
   if (!cg.all->ok) return;
+  unsigned long long *pool = reinterpret_cast<unsigned long long *>(n_ucell + 6);
   const int nbig = n_ucell[0], nu = nbig + n_ucell[4];
+  const long long items = (long long)nu * split;
+  // items are handed out one at a time (work ticket n_ucell[2]): a warp that
+  // finishes a light film cell takes the next one at once; the next ticket is
+  // drawn before the present item is worked on
+  int t_next = 0;
+  if (lane == 0) t_next = atomicAdd(n_ucell + 2, 1);
   for (;;) {
-    // cells are handed out one at a time (work ticket n_ucell[2]): a warp that
-    // finishes a light film cell takes the next cell at once
-    int t = 0;
-    if (lane == 0) t = atomicAdd(n_ucell + 2, 1);
-    t = __shfl_sync(0xffffffffu, t, 0);
-    if (t >= nu) break;
-    const int cb = cell_slot(t, nbig, n);
-    const int key = ucell[2 * cb], s0 = ucell[2 * cb + 1];
-    const int P = cell_end[key] - s0;
-    int lo, len, off, total;
-    warp_cell_runs(key, cg, cell_start, cell_end, lane, &lo, &len, &off, &total);
-    if (total > kMaskCap || P > kMaskMaxP) {
-      // too many candidates for the mask words, or particles for the counters:
-      // the warp-per-particle kernel takes the cell
-      if (lane == 0) overflow[atomicAdd(n_overflow, 1)] = cb;
+    const int t = __shfl_sync(0xffffffffu, t_next, 0);
+    if (t >= items) break;
+    if (lane == 0) t_next = atomicAdd(n_ucell + 2, 1);
+    const int cb = cell_slot(t / split, nbig, n);
+    const int key = ucell[2 * cb];
+    int s0 = ucell[2 * cb + 1], p0, P;
+    item_part(cell_end[key] - s0, split, t % split, &p0, &P);
+    s0 += p0;
+    if (P == 0) {
+      if (lane == 0) mask_off[t] = -1;
       continue;
     }
-    for (int q = lane; q < (P + 1) / 2; q += 32) cnt[q] = 0u;
+    int lo, len, off, total;
+    warp_cell_runs(key, cg, cell_start, cell_end, lane, &lo, &len, &off, &total);
     const int nwords = (total + 31) >> 5;
-    for (int w0 = 0; w0 < nwords; w0 += WW) {
-      const int w1 = min(nwords, w0 + WW);
+    long long at = -1;
+    if (lane == 0 && total <= kMaskCap && P <= kMaskMaxP) {
+      const long long need = (long long)nwords * P;
+      at = (long long)atomicAdd(pool, (unsigned long long)need);
+      if (at + need > pool_words) at = -1;
+    }
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (lane == 0) mask_off[t] = at;
+    if (at < 0) {
+      // too many candidates or particles for the counters, or the pool is
+      // used up: the warp-per-particle kernel takes the item
+      if (lane == 0) overflow[atomicAdd(n_overflow, 1)] = t;
+      continue;
+    }
+    const double sc = cell_scale(key, cg);
+    const V ref = ld4(spos + s0);
+    if (lane < 9) {
+      run_lo[lane] = lo;
+      run_off[lane] = off;
+    }
+    for (int q = lane; q < (P + 1) / 2; q += 32) cnt[q] = 0u;
+    const int dw = 32 / P, dq = 32 - dw * P;   // a lane's step of 32 pairs
+    for (int w0 = 0; w0 < nwords; w0 += kWinWords) {
+      const int w1 = min(nwords, w0 + kWinWords);
       __syncwarp();   // the previous window's reads are done
       for_window(lo, len, off, w0 * 32, min(total, w1 * 32), lane, [&](int c, int sp) {
-        const V v = ld4(spos + sp);
-        if constexpr (sizeof(T) == 4) {
-          const int sl = c + 2 * (c >> 5);
-          tx[sl] = v.x;
-          ty[sl] = v.y;
-          tz[sl] = v.z;
-          th[sl] = 0.5f * v.w;   // exact: r = h_i / 2 + h_j / 2 = (h_i + h_j) / 2
-        } else {
-          cand[c + (c >> 5)] = v;
-        }
+        const float4 u = local_of(ld4(spos + sp), ref, sc);
+        const int w = c >> 5, k = c & 31, a = w * kWinA + 2 * (k & ~1) + (k & 1);
+        ta[a] = u.x;
+        ta[a + 2] = u.y;
+        tb[a] = u.z;
+        tb[a + 2] = u.w;
+        tc[w * kWinC + k] = local_c(u);
       });
-      __syncwarp();
-      // one work item = (word, particle); consecutive lanes take consecutive
-      // particles of a word, so small cells still fill the warp
-      const int items = P * (w1 - w0);
-      for (int it = lane; it < items; it += 32) {
-        const int wl = it / P, q = it - wl * P;
-        const int w = w0 + wl;
-        const int base = w << 5;
-        const uint32_t valid = (total - base) >= 32 ? 0xffffffffu : ((1u << (total - base)) - 1u);
-        const V xi = ld4(spos + s0 + q);
-        uint32_t m = 0, band = 0;
-        if constexpr (sizeof(T) == 4) {
-          // two candidates per packed FP32 instruction; the window always
-          // holds 32 * WW slots (plus pads), so reads past `total` stay in it
-          // and are masked off
-          const float hi2 = 0.5f * xi.w;
-          const float2 nx = make_float2(-xi.x, -xi.x), ny = make_float2(-xi.y, -xi.y);
-          const float2 nz = make_float2(-xi.z, -xi.z), hh = make_float2(hi2, hi2);
-          const float2 klo = make_float2(0.99999f, 0.99999f), khi = make_float2(1.00001f, 1.00001f);
-          const int sb = 34 * wl;   // slot of candidate 32 w in the window
-#pragma unroll
-          for (int k = 0; k < 32; k += 2) {
-            const float2 bx = *reinterpret_cast<const float2 *>(tx + sb + k);
-            const float2 by = *reinterpret_cast<const float2 *>(ty + sb + k);
-            const float2 bz = *reinterpret_cast<const float2 *>(tz + sb + k);
-            const float2 bh = *reinterpret_cast<const float2 *>(th + sb + k);
-            const float2 dx = __fadd2_rn(bx, nx), dy = __fadd2_rn(by, ny), dz = __fadd2_rn(bz, nz);
-            float2 d2 = __fmul2_rn(dx, dx);
-            d2 = __ffma2_rn(dy, dy, d2);
-            d2 = __ffma2_rn(dz, dz, d2);
-            const float2 r = __fadd2_rn(bh, hh);
-            const float2 r2 = __fmul2_rn(r, r);
-            const float2 l2 = __fmul2_rn(r2, klo), h2 = __fmul2_rn(r2, khi);
-            m |= (d2.x < l2.x ? 1u : 0u) << k;
-            m |= (d2.y < l2.y ? 1u : 0u) << (k + 1);
-            band |= (d2.x <= h2.x ? 1u : 0u) << k;
-            band |= (d2.y <= h2.y ? 1u : 0u) << (k + 1);
-          }
-          m &= valid;
-          band &= valid & ~m;
-          // pairs within 1e-5 of the bound: the FP64 definition decides
-          while (band) {
-            const int k = __ffs(band) - 1;
-            band &= band - 1;
-            const int sl = sb + k;
-            if (in_support64(xi.x, xi.y, xi.z, xi.w, tx[sl], ty[sl], tz[sl], 2.0f * th[sl]))
-              m |= 1u << k;
-          }
-        } else {
-          const V *cw = cand + 33 * wl;   // slot of candidate 32 w in the window
-          for (int k = 0; k < 32; ++k)
-            if ((valid >> k) & 1u)
-              if (support_test(xi, cw[k])) m |= 1u << k;
+      if (w1 == nwords)   // slots past the last candidate: far away
+        for (int c = total - w0 * 32 + lane; c < (w1 - w0) * 32; c += 32) {
+          const int w = c >> 5, k = c & 31, a = w * kWinA + 2 * (k & ~1) + (k & 1);
+          ta[a] = ta[a + 2] = tb[a] = tb[a + 2] = 0.0f;
+          tc[w * kWinC + k] = 1e30f;
         }
-        mask[(int64_t)w * stride + s0 + q] = m;
+      __syncwarp();
+      int wl = lane / P, q = lane - wl * P;
+      for (; wl < w1 - w0;) {
+        const V xi = ld4(spos + s0 + q);
+        const float4 ui = local_of(xi, ref, sc);
+        const float cc = local_c(ui);
+        const float2 ci = make_float2(cc, cc);
+        const float2 ax = make_float2(-2.0f * ui.x, -2.0f * ui.x);
+        const float2 ay = make_float2(-2.0f * ui.y, -2.0f * ui.y);
+        const float2 az = make_float2(-2.0f * ui.z, -2.0f * ui.z);
+        const float2 ah = make_float2(-0.5f * ui.w, -0.5f * ui.w);
+        const float4 *pa = reinterpret_cast<const float4 *>(ta + wl * kWinA);
+        const float4 *pb = reinterpret_cast<const float4 *>(tb + wl * kWinA);
+        const float2 *pc = reinterpret_cast<const float2 *>(tc + wl * kWinC);
+        uint32_t m = 0;
+        float near = 1e30f;
+#pragma unroll
+        for (int k = 15; k >= 0; --k) {
+          const float4 a = pa[k], b = pb[k];
+          float2 d = __fadd2_rn(pc[k], ci);
+          d = __ffma2_rn(make_float2(a.x, a.y), ax, d);
+          d = __ffma2_rn(make_float2(a.z, a.w), ay, d);
+          d = __ffma2_rn(make_float2(b.x, b.y), az, d);
+          d = __ffma2_rn(make_float2(b.z, b.w), ah, d);
+          m = __funnelshift_l(__float_as_uint(d.y), m, 1);
+          m = __funnelshift_l(__float_as_uint(d.x), m, 1);
+          near = fminf(near, fminf(fabsf(d.x), fabsf(d.y)));
+        }
+        const int w = w0 + wl;
+        if (near <= kBand) {
+          // some candidate lies at the bound: the FP64 definition decides it
+          for (int k = 0; k < min(32, total - 32 * w); ++k) {
+            const int a = 2 * (k & ~1) + (k & 1);
+            const float *fa = ta + wl * kWinA + a, *fb = tb + wl * kWinA + a;
+            float d = tc[wl * kWinC + k] + cc;
+            d = fmaf(fa[0], ax.x, d);
+            d = fmaf(fa[2], ay.x, d);
+            d = fmaf(fb[0], az.x, d);
+            d = fmaf(fb[2], ah.x, d);
+            if (fabsf(d) > kBand) continue;
+            const int c = 32 * w + k;
+            int r = 8;
+            while (r > 0 && run_off[r] > c) --r;
+            const V xj = ld4(spos + run_lo[r] + (c - run_off[r]));
+            const bool hit = in_support64(xi.x, xi.y, xi.z, xi.w, xj.x, xj.y, xj.z, xj.w);
+            m = (m & ~(1u << k)) | ((hit ? 1u : 0u) << k);
+          }
+        }
+        mask[at + (long long)w * P + q] = m;
         atomicAdd(&cnt[q >> 1], (unsigned)__popc(m) << ((q & 1) * 16));
+        wl += dw;
+        q += dq;
+        if (q >= P) {
+          q -= P;
+          ++wl;
+        }
       }
     }
     __syncwarp();
     for (int q = lane; q < P; q += 32)
       counts[svals[s0 + q]] = (int)((cnt[q >> 1] >> ((q & 1) * 16)) & 0xffffu);
-    __syncwarp();   // the counters are read before the next cell clears them
+    __syncwarp();   // the counters are read before the next item clears them
   }
 }
 
-// Fill pass for the mask kernel's cells, also one warp per cell from a work
-// queue.  The cell's particles go in chunks of 32 (lane = particle, its row
-// start and running length in registers); for each window of kFillWinWords
-// candidate words the warp stages the candidates' original indices and the
-// chunk's hit words (coalesced) in its part of shared memory, then expands the
-// chunk's rows one particle at a time: one candidate per lane, ballot-free
-// compaction by popcount into the row, coalesced stores.  Rows come out
-// ascending when the cloud is in cell order (candidates are runs of
-// consecutive sorted positions, ascending).
+// Fill pass for the mask kernel's items, also one warp per item from a work
+// queue.  The item's particles go in chunks of 32; for each window of
+// kFillWinWords candidate words the warp stages the candidates' original
+// indices, and each lane, holding one particle, its hit words (coalesced) with
+// the place in the row where each word's first hit goes; then the chunk's rows
+// are expanded one particle at a time: one candidate per lane, its place from a
+// popcount of the lower hits, coalesced stores.  Only that one popcount per
+// (particle, word) is left in the expansion (a warp's POPC takes 8 cycles of
+// the issuing scheduler's unit, measured; it is what bounds the kernel), and
+// words are walked in groups of four up to the window's last one, so film
+// cells (4 words) do not pay for a 16-word window.  Rows come out ascending when
+// the cloud is in cell order (candidates are runs of consecutive sorted
+// positions, ascending).
 __global__ void __launch_bounds__(kFillThreads) k_nbr_fill(
     CloudGrids cg, const int32_t *ucell, int32_t *n_ucell, const int32_t *svals,
-    const int32_t *cell_start, const int32_t *cell_end, const uint32_t *mask, int64_t stride,
-    const long long *row_ptr, int32_t *col, long long cap_nnz, int64_t n) {
-  __shared__ int32_t cand_v[kFillWarps][kFillWinWords * 32];   // original indices
-  __shared__ uint32_t mw[kFillWarps][kFillWinWords][32];       // hit words of the chunk
+    const int32_t *cell_start, const int32_t *cell_end, const uint32_t *mask,
+    const long long *mask_off, int split, const long long *row_ptr, int32_t *col,
+    long long cap_nnz, int64_t n) {
+  __shared__ int32_t cand_v[kFillWarps][kFillWinWords * 32];         // original indices
+  __shared__ __align__(16) uint2 rec[kFillWarps][32][kFillRec];      // (hit word, place)
   if (!cg.all->ok) return;
   if (row_ptr[n] > cap_nnz) return;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  const unsigned lt = (1u << lane) - 1u;
+  const unsigned lt = (1u << lane) - 1u, bit = 1u << lane;
   int32_t *cv = cand_v[wp];
   const int nbig = n_ucell[0], nu = nbig + n_ucell[4];
+  const long long items = (long long)nu * split;
+  int t_next = 0;
+  if (lane == 0) t_next = atomicAdd(n_ucell + 3, 1);   // work ticket, as in the mask kernel
   for (;;) {
-    int t = 0;
-    if (lane == 0) t = atomicAdd(n_ucell + 3, 1);   // work ticket, as in the mask kernel
-    t = __shfl_sync(0xffffffffu, t, 0);
-    if (t >= nu) break;
-    const int cb = cell_slot(t, nbig, n);
-    const int key = ucell[2 * cb], s0 = ucell[2 * cb + 1];
-    const int P = cell_end[key] - s0;
+    const int t = __shfl_sync(0xffffffffu, t_next, 0);
+    if (t >= items) break;
+    if (lane == 0) t_next = atomicAdd(n_ucell + 3, 1);
+    const long long moff = mask_off[t];
+    if (moff < 0) continue;   // empty, or the overflow path fills it
+    const int cb = cell_slot(t / split, nbig, n);
+    const int key = ucell[2 * cb];
+    int s0 = ucell[2 * cb + 1], part, P;
+    item_part(cell_end[key] - s0, split, t % split, &part, &P);
+    s0 += part;
     int lo, len, off, total;
     warp_cell_runs(key, cg, cell_start, cell_end, lane, &lo, &len, &off, &total);
-    if (total > kMaskCap || P > kMaskMaxP) continue;   // the overflow path fills it
     const int nwords = (total + 31) >> 5;
     for (int p0 = 0; p0 < P; p0 += 32) {
       const int np = min(32, P - p0);
@@ -771,29 +843,33 @@ __global__ void __launch_bounds__(kFillThreads) k_nbr_fill(
       const long long rs = lane < np ? row_ptr[svals[s0 + q]] : 0;
       int at = 0;
       for (int w0 = 0; w0 < nwords; w0 += kFillWinWords) {
-        const int w1 = min(nwords, w0 + kFillWinWords);
+        const int nw = min(nwords - w0, kFillWinWords);
         __syncwarp();   // the previous window's reads are done
-        for_window(lo, len, off, w0 * 32, min(total, w1 * 32), lane,
+        for_window(lo, len, off, w0 * 32, min(total, (w0 + nw) * 32), lane,
                    [&](int c, int sp) { cv[c] = svals[sp]; });
-        for (int w = w0; w < w1; ++w)
-          mw[wp][w - w0][lane] = lane < np ? mask[(int64_t)w * stride + s0 + q] : 0u;
+        for (int ww = 0; ww < ((nw + 3) & ~3); ++ww) {
+          const uint32_t m =
+              lane < np && ww < nw ? mask[moff + (long long)(w0 + ww) * P + q] : 0u;
+          rec[wp][lane][ww] = make_uint2(m, (unsigned)at);
+          at += __popc(m);
+        }
         __syncwarp();
-        // this lane's candidate of every word of the window, in registers (the
-        // window loop is unrolled; words past w1 are empty)
+        // this lane's candidate of every word of the window, in registers
         int32_t cvr[kFillWinWords];
 #pragma unroll
-        for (int ww = 0; ww < kFillWinWords; ++ww)
-          cvr[ww] = w0 + ww < w1 ? cv[ww * 32 + lane] : 0;
+        for (int ww = 0; ww < kFillWinWords; ++ww) cvr[ww] = ww < nw ? cv[ww * 32 + lane] : 0;
         for (int k = 0; k < np; ++k) {
           int32_t *crow = col + __shfl_sync(0xffffffffu, rs, k);
-          int a = __shfl_sync(0xffffffffu, at, k);
+          const uint4 *rk = reinterpret_cast<const uint4 *>(rec[wp][k]);
 #pragma unroll
-          for (int ww = 0; ww < kFillWinWords; ++ww) {
-            const uint32_t word = w0 + ww < w1 ? mw[wp][ww][k] : 0u;
-            if ((word >> lane) & 1u) crow[a + __popc(word & lt)] = cvr[ww];
-            a += __popc(word);
+          for (int g = 0; g < kFillWinWords / 4; ++g) {
+            if (4 * g >= nw) break;
+            const uint4 a = rk[2 * g], b = rk[2 * g + 1];
+            if (a.x & bit) crow[a.y + __popc(a.x & lt)] = cvr[4 * g];
+            if (a.z & bit) crow[a.w + __popc(a.z & lt)] = cvr[4 * g + 1];
+            if (b.x & bit) crow[b.y + __popc(b.x & lt)] = cvr[4 * g + 2];
+            if (b.z & bit) crow[b.w + __popc(b.z & lt)] = cvr[4 * g + 3];
           }
-          if (lane == k) at = a;
         }
       }
     }
@@ -947,15 +1023,17 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
   CloudGrids cg{ctx->d_grids, ctx->cell_base, nb, ctx->d_grid};
   const int nbr_blocks = sms * 8;
   int32_t *n_overflow = ctx->n_ucell + 1;
-  const int64_t stride = ctx->cap_particles;
+  const long long pool_words = (long long)kMaskWords * ctx->cap_particles;
+  // parts per cell: a small cloud has fewer cells than the GPU has warps
+  const int split = n <= kSplitMax ? kSplit : 1;
   MAFP_TIMED(ctx, s, sizeof(T) == 4 ? "k_nbr_mask<float>" : "k_nbr_mask<double>",
-             k_nbr_mask<T><<<sms * 16, kMaskThreads, kMaskWarps * kMaskWarpBytes<T>, s>>>(
-                 cg, ctx->ucell, ctx->n_ucell, spos, vin, ctx->cell_start,
-                 ctx->cell_end, ctx->counts, ctx->nbr_mask, stride, ctx->overflow, n_overflow,
-                 n));
+             k_nbr_mask<T><<<sms * 8, kMaskThreads, kMaskWarps * kMaskWarpBytes, s>>>(
+                 cg, ctx->ucell, ctx->n_ucell, spos, vin, ctx->cell_start, ctx->cell_end,
+                 ctx->counts, ctx->nbr_mask, pool_words, ctx->mask_off, split, ctx->overflow,
+                 n_overflow, n));
   MAFP_TIMED(ctx, s, "k_nbr<T,false>(overflow cells)",
              k_nbr<T, false><<<nbr_blocks, kNbrThreads, kNbrSmemBytes, s>>>(
-      cg, ctx->ucell, ctx->overflow, n_overflow, spos, vin, ctx->cell_start,
+      cg, ctx->ucell, ctx->n_ucell, split, ctx->overflow, n_overflow, spos, vin, ctx->cell_start,
       ctx->cell_end, ctx->counts, nullptr, nullptr, 0, n));
   MAFP_LAUNCH_CHECK(ctx);
   int rc = scan_i32_to_i64(ctx, ctx->counts, reinterpret_cast<long long *>(row_ptr), n, s);
@@ -964,13 +1042,13 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
              k_check_nnz<<<1, 1, 0, s>>>(reinterpret_cast<const long long *>(row_ptr), n, cap_nnz, nnz_dev,
                               ctx->d_status, ctx->d_grid));
   MAFP_TIMED(ctx, s, "k_nbr_fill",
-             k_nbr_fill<<<sms * (2048 / kFillThreads), kFillThreads, 0, s>>>(
+             k_nbr_fill<<<sms * 8, kFillThreads, 0, s>>>(
                  cg, ctx->ucell, ctx->n_ucell, vin, ctx->cell_start, ctx->cell_end,
-                 ctx->nbr_mask, stride, reinterpret_cast<const long long *>(row_ptr), col,
-                 cap_nnz, n));
+                 ctx->nbr_mask, ctx->mask_off, split,
+                 reinterpret_cast<const long long *>(row_ptr), col, cap_nnz, n));
   MAFP_TIMED(ctx, s, "k_nbr<T,true>(overflow cells)",
              k_nbr<T, true><<<nbr_blocks, kNbrThreads, kNbrSmemBytes, s>>>(
-      cg, ctx->ucell, ctx->overflow, n_overflow, spos, vin, ctx->cell_start,
+      cg, ctx->ucell, ctx->n_ucell, split, ctx->overflow, n_overflow, spos, vin, ctx->cell_start,
       ctx->cell_end, ctx->counts, reinterpret_cast<const long long *>(row_ptr), col, cap_nnz, n));
   MAFP_TIMED(ctx, s, "k_rowsort",
              k_rowsort<<<grid_for(n, kSortWarps, sms * 8), kSortWarps * 32, 0, s>>>(
@@ -1015,9 +1093,9 @@ int build_neighbours_batched(mafp_ctx *ctx, int64_t n, int32_t dtype, int32_t nc
 
 void init_kernel_attributes() {
   cudaFuncSetAttribute(k_nbr_mask<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kMaskWarps * kMaskWarpBytes<float>);
+                       kMaskWarps * kMaskWarpBytes);
   cudaFuncSetAttribute(k_nbr_mask<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kMaskWarps * kMaskWarpBytes<double>);
+                       kMaskWarps * kMaskWarpBytes);
   cudaFuncSetAttribute(k_nbr<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        kNbrSmemBytes);
   cudaFuncSetAttribute(k_nbr<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
