@@ -136,7 +136,6 @@ int mafp_create(mafp_ctx **out, const mafp_params *params, int64_t cap_particles
   const int64_t cap = cap_particles;
   ctx->max_tiles = cap / 2048 + 1;
   const int64_t i64_len = std::max<int64_t>(2 * cap + 8, 256 * ctx->max_tiles + 8);
-  const int64_t items = kSplit * std::min(cap, kSplitMax) + cap;
   struct {
     void **p;
     size_t bytes;
@@ -153,8 +152,8 @@ int mafp_create(mafp_ctx **out, const mafp_params *params, int64_t cap_particles
       {(void **)&ctx->n_ucell, sizeof(int32_t) * 8},
       {(void **)&ctx->counts, sizeof(int32_t) * cap},
       {(void **)&ctx->nbr_mask, sizeof(uint32_t) * kMaskWords * cap},
-      {(void **)&ctx->mask_off, sizeof(long long) * items},
-      {(void **)&ctx->overflow, sizeof(int32_t) * items},
+      {(void **)&ctx->cell_table, sizeof(int32_t) * 24 * cap},
+      {(void **)&ctx->overflow, sizeof(int32_t) * cap},
       {(void **)&ctx->scan_tmp, sizeof(long long) * (i64_len / 4096 + 4)},
       {(void **)&ctx->scan_ctr, sizeof(int32_t) * 2},
       {(void **)&ctx->fallback, sizeof(int32_t) * cap},
@@ -194,7 +193,7 @@ int mafp_destroy(mafp_ctx *ctx) {
                   ctx->radix_hist, ctx->cell_start, ctx->cell_end,   ctx->spos,
                   ctx->ucell,     ctx->n_ucell,  ctx->counts,       ctx->scan_tmp,
                   ctx->scan_ctr,
-                  ctx->nbr_mask,  ctx->mask_off, ctx->overflow,
+                  ctx->nbr_mask,  ctx->cell_table, ctx->overflow,
                   ctx->fallback, ctx->d_status,  ctx->d_grid,
                   ctx->remap_i64, ctx->remap_i32, ctx->d_grids,   ctx->cell_base,
                   ctx->cloud_id,  ctx->one_cloud, ctx->cloud_partial};

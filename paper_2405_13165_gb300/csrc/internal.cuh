@@ -9,10 +9,9 @@
 namespace mafp {
 
 constexpr int kMaxRowSort = 2048;   // longest row the in-shared-memory row sort handles
-constexpr int kMaskCap = 32768;     // candidates of one cell in the neighbour mask kernel
 constexpr int kMaskWords = 64;      // hit words per particle of the capacity in the mask pool
-constexpr int kSplit = 8;           // parts per cell in the search of a small cloud
-constexpr int64_t kSplitMax = 131072;   // largest such cloud
+constexpr int64_t kSplitAll = 131072;    // largest cloud whose search splits every cell
+constexpr int64_t kSplitMore = 524288;   // largest one that quarters the costly cells
 constexpr int kMaxClouds = 65536;   // clouds of one batched neighbour build
 
 // Device status block (layout mirrored by mafp_status in the public header).
@@ -63,12 +62,12 @@ struct mafp_ctx {
   int32_t *cell_start, *cell_end;
   void *spos;               // sorted positions, 32 bytes per particle
   int32_t *ucell;           // [2 * cap] occupied cells: key, first sorted position
-  int32_t *n_ucell;         // device counters: cells (front group), overflow items, mask and
+  int32_t *n_ucell;         // device counters: cells (front group), overflow cells, mask and
                             // fill tickets, cells (back group), -, mask pool (64 bits)
   int32_t *counts;          // [cap] row lengths
   uint32_t *nbr_mask;       // [kMaskWords * cap] pool of candidate hit bits
-  long long *mask_off;      // [kSplit * min(cap, kSplitMax) + cap] each work item's place in it
-  int32_t *overflow;        // [as mask_off] work items that the mask kernel cannot hold
+  int32_t *cell_table;      // [24 * cap] search records of the occupied cells
+  int32_t *overflow;        // [cap] occupied cells that the mask kernel cannot hold
   long long *scan_tmp;      // tile states of the one-pass scan, zero between scans
   int32_t *scan_ctr;        // [2] tickets and finished tiles of the scan, zero between scans
   int32_t *fallback;        // [cap] particles re-done in FP64

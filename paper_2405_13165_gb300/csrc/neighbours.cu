@@ -403,7 +403,7 @@ __device__ __forceinline__ bool in_support(const float4 &a, const float4 &b) {
   float r = (a.w + b.w) * 0.5f;
   float r2 = r * r;
   float diff = d2 - r2;
-  if (fabsf(diff) <= 1e-5f * r2)
+  if (!(fabsf(diff) > 1e-5f * r2))   // (also where the squares overflow)
     return in_support64(a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w);
   return diff < 0.0f;
 }
@@ -414,55 +414,43 @@ __device__ __forceinline__ bool in_support(const double4_16a &a, const double4_1
 constexpr int kNbrThreads = 128;
 constexpr int kNbrSmemBytes = 32768;
 
-// Warp-per-particle count / fill (ballot compaction), for the occupied cells
-// listed in sel[0 .. *n_sel): the work items (a cell, or a part of its particles)
-// that the mask kernel below cannot hold.
-struct CloudGrids;
-__device__ __forceinline__ void item_part(int P, int split, int c, int *p0, int *np);
-__device__ __forceinline__ void cell_runs(int key, const CloudGrids &cg,
-                                          const int32_t *cell_start, const int32_t *cell_end,
-                                          int r, int *lo_out, int *len_out);
+// What the search needs of one occupied cell, in the order of the work queue
+// (written by k_cell_table): its particles' sorted positions [s0, s0 + P), the
+// candidates (the particles of the 27 cells around it, as nr non-empty runs of
+// consecutive sorted positions: candidate c of run r, off_r <= c < off_(r+1), is
+// sorted position c + delta_r), the power of two 2^-e that takes the cell edge
+// into [1/2, 1), and where its hit words start in the mask pool (-1: the cell
+// goes to the warp-per-particle kernels).
+constexpr int kCellRec = 24;   // ints per record
+enum { kRecS0 = 0, kRecP = 1, kRecTotal = 2, kRecRuns = 3, kRecPool = 4, kRecRun = 6 };
 
+// Warp-per-particle count / fill (ballot compaction), for the occupied cells
+// listed in sel[0 .. *n_sel): those that the mask kernel below cannot hold.
 template <typename T, bool FILL>
 __global__ void __launch_bounds__(kNbrThreads) k_nbr(
-    CloudGrids cg, const int32_t *ucell, const int32_t *n_ucell, int split, const int32_t *sel,
-    const int32_t *n_sel, const vec4_t<T> *spos, const int32_t *svals,
-    const int32_t *cell_start, const int32_t *cell_end, int32_t *counts,
-    const long long *row_ptr, int32_t *col, long long cap_nnz, int64_t n) {
+    const GridDev *all, const int32_t *table, const int32_t *sel, const int32_t *n_sel,
+    const vec4_t<T> *spos, const int32_t *svals, int32_t *counts, const long long *row_ptr,
+    int32_t *col, long long cap_nnz, int64_t n) {
   using V = vec4_t<T>;
   constexpr int CAP = kNbrSmemBytes / sizeof(V);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V *cand = reinterpret_cast<V *>(smem_raw);
-  __shared__ int r_lo[9], r_len[9], r_off[10];
-  if (!cg.all->ok) return;
+  if (!all->ok) return;
   if (FILL && row_ptr[n] > cap_nnz) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = kNbrThreads / 32;
   const unsigned lt = (1u << lane) - 1u;
   const int nu = *n_sel;
   for (int cs = blockIdx.x; cs < nu; cs += gridDim.x) {
-    const int cb = cell_slot(sel[cs] / split, n_ucell[0], n);
-    const int key = ucell[2 * cb];
-    int s0 = ucell[2 * cb + 1], part, np;
-    item_part(cell_end[key] - s0, split, sel[cs] % split, &part, &np);
-    s0 += part;
-    const int s1 = s0 + np;
-    if (threadIdx.x < 9)
-      cell_runs(key, cg, cell_start, cell_end, threadIdx.x, &r_lo[threadIdx.x], &r_len[threadIdx.x]);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int o = 0;
-      for (int r = 0; r < 9; ++r) {
-        r_off[r] = o;
-        o += r_len[r];
-      }
-      r_off[9] = o;
-    }
-    __syncthreads();
-    const bool staged = r_off[9] <= CAP;
+    const int32_t *rec = table + (long long)sel[cs] * kCellRec;
+    const int s0 = rec[kRecS0], s1 = s0 + rec[kRecP], total = rec[kRecTotal];
+    const int nr = rec[kRecRuns] & 255;
+    const bool staged = total <= CAP;
     if (staged) {
-      for (int r = 0; r < 9; ++r)
-        for (int t = threadIdx.x; t < r_len[r]; t += kNbrThreads)
-          cand[r_off[r] + t] = ld4(spos + r_lo[r] + t);
+      for (int r = 0; r < nr; ++r) {
+        const int off = rec[kRecRun + 2 * r], d = rec[kRecRun + 2 * r + 1];
+        const int end = r + 1 < nr ? rec[kRecRun + 2 * r + 2] : total;
+        for (int c = off + threadIdx.x; c < end; c += kNbrThreads) cand[c] = ld4(spos + c + d);
+      }
     }
     __syncthreads();
     for (int p = s0 + w; p < s1; p += nw) {
@@ -470,17 +458,18 @@ __global__ void __launch_bounds__(kNbrThreads) k_nbr(
       long long base = 0;
       if (FILL) base = row_ptr[svals[p]];
       int cnt = 0;
-      for (int r = 0; r < 9; ++r) {
-        const int len = r_len[r], lo = r_lo[r], off = r_off[r];
-        for (int t0 = 0; t0 < len; t0 += 32) {
-          const int t = t0 + lane;
+      for (int r = 0; r < nr; ++r) {
+        const int off = rec[kRecRun + 2 * r], d = rec[kRecRun + 2 * r + 1];
+        const int end = r + 1 < nr ? rec[kRecRun + 2 * r + 2] : total;
+        for (int c0 = off; c0 < end; c0 += 32) {
+          const int c = c0 + lane;
           bool hit = false;
-          if (t < len) {
-            const V xj = staged ? cand[off + t] : ld4(spos + lo + t);
+          if (c < end) {
+            const V xj = staged ? cand[c] : ld4(spos + c + d);
             hit = in_support(xi, xj);
           }
           const unsigned m = __ballot_sync(0xffffffffu, hit);
-          if (FILL && hit) col[base + cnt + __popc(m & lt)] = svals[lo + t];
+          if (FILL && hit) col[base + cnt + __popc(m & lt)] = svals[c + d];
           cnt += __popc(m);
         }
       }
@@ -501,19 +490,21 @@ __global__ void k_check_nnz(const long long *row_ptr, int64_t n, long long cap_n
 
 // ------------------------------------------------ warp-per-cell mask path
 // Every particle of a cell shares the candidate set "27 cells around it",
-// which is 9 runs of consecutive sorted positions (3 x-adjacent cells each).
-// Each warp takes work items -- an occupied cell, or one of `split` parts of
-// its particles -- from a device work queue (an atomic ticket per item) and
-// handles its item alone, with warp-level synchronisation only: a film cell (a
-// dozen particles, ~4 candidate words) and a 3D cell (~40 particles, ~37
-// words) then cost the warp in proportion to their work, and no block waits at
-// a barrier for its slowest thread.  The candidates are staged in windows of
-// kWinWords words (32 candidates each) in the warp's part of shared memory;
-// the warp's lanes take (word, particle) pairs of the window (consecutive
-// lanes, consecutive particles of one word: the candidate reads are
-// broadcasts), test 32 candidates against the particle and write one bit per
-// candidate plus the row length.  The fill kernel turns the bits back into
-// column indices, so the distance tests run once.
+// which is up to 9 runs of consecutive sorted positions (3 x-adjacent cells
+// each).  k_cell_table writes each cell's runs once, a thread per cell.  The
+// mask and fill kernels then take work items -- a cell, or one of `split` parts
+// of its particles -- from a device work queue and handle each by one warp, with
+// warp-level synchronisation only: a film cell (a dozen particles, ~4 candidate
+// words) and a 3D cell (~40 particles, ~37 words) cost the warp in proportion
+// to their work, and no block waits at a barrier for its slowest thread.  The
+// mask kernel takes the candidates in windows of kWinWords words: a lane holds
+// one candidate of each word in registers, the particles are broadcast one
+// after another from shared memory, and a ballot gives the 32 bits of a
+// (particle, word).  (With the particles in the lanes and the candidates
+// broadcast, 10 floats per two candidates go to every lane: the 128 bytes per
+// cycle that shared memory returns bound that form at 0.29 ms on the 1M jet
+// cloud, whatever the arithmetic; here 5 floats go out per 256 tests.)  The fill
+// kernel turns the bits back into column indices, so the tests run once.
 //
 // The test is one packed dot product.  With u = (x - x_ref) sc, x_ref a particle
 // of the item's cell and sc the power of two that takes the cell edge c into
@@ -521,354 +512,444 @@ __global__ void k_check_nnz(const long long *row_ptr, int64_t n, long long cap_n
 //   |u_j - u_i|^2 - (h_i + h_j)^2 / 4
 //     = (|u_j|^2 - h_j^2/4) + (|u_i|^2 - h_i^2/4) - 2 u_i.u_j - (h_i/2) h_j,
 // a sum and four fused multiply-adds per candidate (two candidates per packed
-// FP32 instruction) on staged (u_j, h_j, |u_j|^2 - h_j^2/4), against eleven
-// operations for the difference form; its sign is the bit (a funnel shift).
+// FP32 instruction), against eleven operations for the difference form; its
+// sign is the bit.
 // FP32 evaluates it to 1.3e-5 (|u_i| <= 1, |u_j| <= 2 per axis, partial sums up
 // to 28: ten roundings of at most 2^-24 each, and 1.3e-6 from the rounded
 // u), so a value within kBand of zero is decided by the FP64 definition on the
 // original positions instead -- for FP64 clouds too, whose tests all ran on
-// the FP64 pipe before.  One word in 5000 needs that.
+// the FP64 pipe before (2138 us against 63 us on the 60k jet cloud).  One word in
+// 5000 needs that.  1M jet cloud: 302 us with candidates and differences from
+// shared memory, 213 us so.
 //
-// The bits of an item go to a pool, nwords x P words from an atomic counter
-// (pool_words in all, kMaskWords per particle of the context's capacity on
-// average): film cells need 4 words per particle, cells of an irregular cloud
-// 60, and only what exceeds the pool takes the warp-per-particle kernel.
+// The bits go to a pool, P rows of nwords (rounded up to 4) per cell (pool_words
+// in all, kMaskWords per particle of the context's capacity on average): film
+// cells need 4 words per particle, cells of an irregular cloud 60, and only what
+// exceeds the pool takes the warp-per-particle kernels.
 constexpr int kMaskThreads = 128;
 constexpr int kMaskWarps = kMaskThreads / 32;
-constexpr int kMaskMaxP = 256;   // particles of one item in the mask kernel (else: overflow path)
-static_assert(kMaskCap < 65536 && kMaskMaxP % 2 == 0, "two 16-bit hit counts per word");
 constexpr int kWinWords = 8;
+constexpr int kMaskBlock = 64;   // particles prepared at a time
 constexpr float kBand = 1.6e-5f;
-// A window's words: pairs of candidates as (x0, x1, y0, y1) and (z0, z1, h0, h1)
-// (16 pairs and 16 pad bytes per word, so that words tested by lanes of one warp
-// sit in different banks), and (c0, c1).
-constexpr int kWinA = 68, kWinC = 36;   // floats per word
-constexpr int kWinFloats = kWinWords * (2 * kWinA + kWinC);
-constexpr int kMaskWarpBytes = kWinFloats * (int)sizeof(float) +
-                               (kMaskMaxP / 2) * (int)sizeof(unsigned) + 20 * (int)sizeof(int);
-static_assert(kMaskWarpBytes % 16 == 0, "16-byte aligned windows");
+// Words of a particle's row in the mask pool.
+__host__ __device__ constexpr int row_words(int total) { return ((total + 127) >> 7) << 2; }
 
 constexpr int kFillThreads = 128;
 constexpr int kFillWarps = kFillThreads / 32;
 constexpr int kFillWinWords = 16;   // candidate words of one fill window
 constexpr int kFillRec = kFillWinWords + 2;   // records of one particle, with pad
-
-// Particles [*p0, *p0 + *np) of the cell that part `c` of `split` holds.
-__device__ __forceinline__ void item_part(int P, int split, int c, int *p0, int *np) {
-  const int q = (P + split - 1) / split;
+// Work items: the cells of the front group in 2^front parts each, then those of
+// the back group in 2^back parts.
+struct Split {
+  int front, back;
+};
+// Particles [*p0, *p0 + *np) of the cell's P that part `c` of 2^log holds.
+__device__ __forceinline__ void item_part(int P, int log, int c, int *p0, int *np) {
+  const int q = (P + (1 << log) - 1) >> log;
   *p0 = min(P, c * q);
   *np = min(P, *p0 + q) - *p0;
 }
 
-// Rows of the 27-cell neighbourhood of global cell `key`: run r (dz = r/3-1,
-// dy = r%3-1) covers cells key-1..key+1 of that (y, z) row of the key's own
-// cloud grid, clipped to that grid.
-__device__ __forceinline__ void cell_runs(int key, const CloudGrids &cg,
-                                          const int32_t *cell_start, const int32_t *cell_end,
-                                          int r, int *lo_out, int *len_out) {
-  int b0 = 0, b1 = cg.nb;   // cloud with cell_base[b] <= key < cell_base[b + 1]
-  while (b1 - b0 > 1) {
-    const int mid = (b0 + b1) >> 1;
-    if (cg.cell_base[mid] <= key) b0 = mid; else b1 = mid;
-  }
-  const GridDev &g = cg.grids[b0];
-  const int local = key - (int)cg.cell_base[b0];
-  const int dx_ = g.dim[0], dy_ = g.dim[1], dz_ = g.dim[2];
-  const int cx = local % dx_, cy = (local / dx_) % dy_, cz = local / (dx_ * dy_);
-  const int ddz = r / 3 - 1, ddy = r % 3 - 1;
-  int lo = INT_MAX, hi = 0;
-  if (cz + ddz >= 0 && cz + ddz < dz_ && cy + ddy >= 0 && cy + ddy < dy_) {
-    const int base = key + ddz * dx_ * dy_ + ddy * dx_;
-    const int k0 = cx > 0 ? base - 1 : base, k1 = cx < dx_ - 1 ? base + 1 : base;
-    for (int k = k0; k <= k1; ++k) {
-      lo = min(lo, cell_start[k]);
-      hi = max(hi, cell_end[k]);
-    }
-  }
-  *lo_out = lo;
-  *len_out = hi > lo ? hi - lo : 0;
-}
-
-// The 9 runs of a cell, one per lane 0..8 (start, length, offset in the
-// cell's candidate list), and the candidate total (every lane).
-__device__ __forceinline__ void warp_cell_runs(int key, const CloudGrids &cg,
-                                               const int32_t *cell_start,
-                                               const int32_t *cell_end, int lane, int *lo,
-                                               int *len, int *off, int *total) {
-  *lo = 0;
-  *len = 0;
-  if (lane < 9) cell_runs(key, cg, cell_start, cell_end, lane, lo, len);
-  int inc = *len;
+// One thread per occupied cell (queue position t): its record.
+__global__ void __launch_bounds__(128) k_cell_table(
+    CloudGrids cg, const int32_t *ucell, int32_t *n_ucell, const int32_t *cell_start,
+    const int32_t *cell_end, int32_t *table, long long pool_words, int32_t *overflow,
+    int64_t n) {
+  if (!cg.all->ok) return;
+  const int lane = threadIdx.x & 31;
+  const int nbig = n_ucell[0], nu = nbig + n_ucell[4];
+  unsigned long long *pool = reinterpret_cast<unsigned long long *>(n_ucell + 6);
+  for (int t0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; t0 < nu;
+       t0 += gridDim.x * blockDim.x) {
+    const int t = t0 + lane;
+    const bool in = t < nu;
+    int rec[kCellRec];
 #pragma unroll
-  for (int o = 1; o < 16; o <<= 1) {
-    const int u = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += u;
+    for (int k = 0; k < kCellRec; ++k) rec[k] = 0;
+    long long need = 0;
+    if (in) {
+      const int cb = cell_slot(t, nbig, n);
+      const int key = ucell[2 * cb], s0 = ucell[2 * cb + 1];
+      int b0 = 0, b1 = cg.nb;   // cloud with cell_base[b] <= key < cell_base[b + 1]
+      while (b1 - b0 > 1) {
+        const int mid = (b0 + b1) >> 1;
+        if (cg.cell_base[mid] <= key) b0 = mid; else b1 = mid;
+      }
+      const GridDev &g = cg.grids[b0];
+      const int local = key - (int)cg.cell_base[b0];
+      const int dx_ = g.dim[0], dy_ = g.dim[1], dz_ = g.dim[2];
+      const int row = local / dx_, cx = local - row * dx_;
+      const int cz = row / dy_, cy = row - cz * dy_;
+      // run r (dz = r/3-1, dy = r%3-1) covers cells key-1..key+1 of that (y, z)
+      // row of the key's own cloud grid, clipped to that grid
+      int lo[9], hi[9];
+#pragma unroll
+      for (int r = 0; r < 9; ++r) {
+        const int ddz = r / 3 - 1, ddy = r % 3 - 1;
+        lo[r] = INT_MAX;
+        hi[r] = 0;
+        if (cz + ddz >= 0 && cz + ddz < dz_ && cy + ddy >= 0 && cy + ddy < dy_) {
+          const int base = key + (ddz * dy_ + ddy) * dx_;
+#pragma unroll
+          for (int a = -1; a <= 1; ++a)
+            if (cx + a >= 0 && cx + a < dx_) {
+              lo[r] = min(lo[r], cell_start[base + a]);
+              hi[r] = max(hi[r], cell_end[base + a]);
+            }
+        }
+      }
+      int total = 0, nr = 0;
+#pragma unroll
+      for (int r = 0; r < 9; ++r)
+        if (hi[r] > lo[r]) {
+#pragma unroll
+          for (int k = 0; k <= r; ++k)   // (static indices: rec stays in registers)
+            if (k == nr) {
+              rec[kRecRun + 2 * k] = total;
+              rec[kRecRun + 2 * k + 1] = lo[r] - total;
+            }
+          total += hi[r] - lo[r];
+          ++nr;
+        }
+      const int P = cell_end[key] - s0;
+      int e;   // edges beyond 2^+-120 leave FP32's range: the warp-per-particle kernels
+      frexp(g.c, &e);
+      rec[kRecS0] = s0;
+      rec[kRecP] = P;
+      rec[kRecTotal] = total;
+      rec[kRecRuns] = nr | ((max(-120, min(120, e)) + 128) << 8);
+      if (abs(e) <= 120) need = (long long)row_words(total) * P;
+    }
+    // the warp's share of the pool, by one atomic
+    long long inc = need;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long u = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += u;
+    }
+    long long base = 0;
+    if (lane == 31) base = (long long)atomicAdd(pool, (unsigned long long)inc);
+    base = __shfl_sync(0xffffffffu, base, 31) + inc - need;
+    if (!in) continue;
+    if (need == 0 || base + need > pool_words) {
+      // an edge out of range, or the pool is used up
+      base = -1;
+      overflow[atomicAdd(n_ucell + 1, 1)] = t;
+    }
+    rec[kRecPool] = (int)(unsigned)(base & 0xffffffffll);
+    rec[kRecPool + 1] = (int)(base >> 32);
+    int4 *out = reinterpret_cast<int4 *>(table + (long long)t * kCellRec);
+#pragma unroll
+    for (int k = 0; k < kCellRec / 4; ++k)
+      out[k] = make_int4(rec[4 * k], rec[4 * k + 1], rec[4 * k + 2], rec[4 * k + 3]);
   }
-  *off = inc - *len;
-  *total = __shfl_sync(0xffffffffu, inc, 8);
 }
 
-// Calls put(c - c0, sorted position of candidate c) for every candidate c of
-// the window [c0, c1), lanes striding over each run's part of the window.
-template <typename F>
-__device__ __forceinline__ void for_window(int lo, int len, int off, int c0, int c1, int lane,
-                                           F &&put) {
-#pragma unroll 1
-  for (int r = 0; r < 9; ++r) {
-    const int rlo = __shfl_sync(0xffffffffu, lo, r), rlen = __shfl_sync(0xffffffffu, len, r);
-    const int roff = __shfl_sync(0xffffffffu, off, r);
-    const int a = max(c0, roff), b = min(c1, roff + rlen);
-    for (int c = a + lane; c < b; c += 32) put(c - c0, rlo + (c - roff));
-  }
-}
+// The work queue as one warp walks it: an atomic ticket per item; the next
+// ticket is drawn and the next item's record loaded (one int per lane) while the
+// present item is worked on.
+struct ItemWalk {
+  const int32_t *table;
+  int32_t *ticket;
+  Split sp;
+  int nfront, items, lane;   // items of the front group, of both
+  int at, ahead;             // present item, next ticket (lane 0)
+  int rec_next;
 
-// The power of two that takes the cell edge of the cloud of global cell `key`
-// into [1/2, 1).
-__device__ __forceinline__ double cell_scale(int key, const CloudGrids &cg) {
-  int b0 = 0, b1 = cg.nb;
-  while (b1 - b0 > 1) {
-    const int mid = (b0 + b1) >> 1;
-    if (cg.cell_base[mid] <= key) b0 = mid; else b1 = mid;
+  __device__ __forceinline__ int load(int item) const {
+    const int cell = item < nfront ? item >> sp.front
+                                   : (nfront >> sp.front) + ((item - nfront) >> sp.back);
+    return item < items && lane < kCellRec ? table[(long long)cell * kCellRec + lane] : 0;
   }
-  int e;
-  frexp(cg.grids[b0].c, &e);
-  return ldexp(1.0, -max(-120, min(120, e)));
+  __device__ __forceinline__ int draw() const { return lane == 0 ? atomicAdd(ticket, 1) : 0; }
+  __device__ __forceinline__ void start(const int32_t *tab, int32_t *tk, int nbig, int nlight,
+                                        Split split, int ln) {
+    table = tab;
+    ticket = tk;
+    sp = split;
+    lane = ln;
+    nfront = nbig << sp.front;
+    items = nfront + (nlight << sp.back);
+    at = __shfl_sync(0xffffffffu, draw(), 0);
+    ahead = draw();
+    rec_next = load(at);
+  }
+  // The present item's record (one int per lane), its first particle's sorted
+  // position and count; false at the end.
+  __device__ __forceinline__ bool next(int *rec, int *s0, int *p0, int *P) {
+    if (at >= items) return false;
+    *rec = rec_next;
+    const bool f = at < nfront;
+    const int log = f ? sp.front : sp.back, part = (f ? at : at - nfront) & ((1 << log) - 1);
+    item_part(__shfl_sync(0xffffffffu, *rec, kRecP), log, part, p0, P);
+    *s0 = __shfl_sync(0xffffffffu, *rec, kRecS0) + *p0;
+    at = __shfl_sync(0xffffffffu, ahead, 0);
+    ahead = draw();
+    rec_next = load(at);
+    return true;
+  }
+};
+
+// Sorted positions of candidates c0 + lane + 32 u, u = 0..3 (those past the
+// last candidate give the last one's); r is the run that holds c0 or an earlier
+// one, moved on to c0's.
+__device__ __forceinline__ void candidates4(int rec, int nr, int total, int c0, int lane, int *r,
+                                            int (&sp)[4]) {
+  while (*r + 1 < nr && __shfl_sync(0xffffffffu, rec, kRecRun + 2 * (*r + 1)) <= c0) ++*r;
+  const int d0 = __shfl_sync(0xffffffffu, rec, kRecRun + 2 * *r + 1);
+  int d[4] = {d0, d0, d0, d0}, c[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) c[u] = min(c0 + lane + 32 * u, total - 1);
+  for (int k = *r + 1; k < nr; ++k) {
+    const int o = __shfl_sync(0xffffffffu, rec, kRecRun + 2 * k);
+    if (o >= c0 + 128) break;
+    const int dk = __shfl_sync(0xffffffffu, rec, kRecRun + 2 * k + 1);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) d[u] = c[u] >= o ? dk : d[u];
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) sp[u] = c[u] + d[u];
 }
 
 // (x - ref) sc in FP32: the subtraction in the input's own type, sc exact.
-__device__ __forceinline__ float4 local_of(const float4 &v, const float4 &r, double sc) {
-  const float s = (float)sc;
-  return make_float4((v.x - r.x) * s, (v.y - r.y) * s, (v.z - r.z) * s, v.w * s);
+__device__ __forceinline__ float4 local_of(const float4 &v, const float4 &r, float sc) {
+  return make_float4((v.x - r.x) * sc, (v.y - r.y) * sc, (v.z - r.z) * sc, v.w * sc);
 }
-__device__ __forceinline__ float4 local_of(const double4_16a &v, const double4_16a &r, double sc) {
-  return make_float4((float)((v.x - r.x) * sc), (float)((v.y - r.y) * sc),
-                     (float)((v.z - r.z) * sc), (float)(v.w * sc));
+__device__ __forceinline__ float4 local_of(const double4_16a &v, const double4_16a &r, float sc) {
+  return make_float4((float)(v.x - r.x) * sc, (float)(v.y - r.y) * sc, (float)(v.z - r.z) * sc,
+                     (float)v.w * sc);
 }
 // |u|^2 - h^2/4
 __device__ __forceinline__ float local_c(const float4 &u) {
   return fmaf(u.x, u.x, fmaf(u.y, u.y, fmaf(u.z, u.z, -0.25f * u.w * u.w)));
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
-    CloudGrids cg, const int32_t *ucell, int32_t *n_ucell, const vec4_t<T> *spos,
-    const int32_t *svals, const int32_t *cell_start, const int32_t *cell_end, int32_t *counts,
-    uint32_t *mask, long long pool_words, long long *mask_off, int split, int32_t *overflow,
-    int32_t *n_overflow, int64_t n) {
-  using V = vec4_t<T>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  float *ta = reinterpret_cast<float *>(smem_raw + wp * kMaskWarpBytes);
-  float *tb = ta + kWinWords * kWinA, *tc = tb + kWinWords * kWinA;
-  // per-particle hit counts, two 16-bit counts per word (a row has at most
-  // kMaskCap < 65536 candidates); the runs' starts and offsets (FP64 retakes)
-  unsigned *cnt = reinterpret_cast<unsigned *>(tc + kWinWords * kWinC);
-  int *run_lo = reinterpret_cast<int *>(cnt + kMaskMaxP / 2), *run_off = run_lo + 10;
-  if (!cg.all->ok) return;
-  unsigned long long *pool = reinterpret_cast<unsigned long long *>(n_ucell + 6);
-  const int nbig = n_ucell[0], nu = nbig + n_ucell[4];
-  const long long items = (long long)nu * split;
-  // items are handed out one at a time (work ticket n_ucell[2]): a warp that
-  // finishes a light film cell takes the next one at once; the next ticket is
-  // drawn before the present item is worked on
-  int t_next = 0;
-  if (lane == 0) t_next = atomicAdd(n_ucell + 2, 1);
-  for (;;) {
-    const int t = __shfl_sync(0xffffffffu, t_next, 0);
-    if (t >= items) break;
-    if (lane == 0) t_next = atomicAdd(n_ucell + 2, 1);
-    const int cb = cell_slot(t / split, nbig, n);
-    const int key = ucell[2 * cb];
-    int s0 = ucell[2 * cb + 1], p0, P;
-    item_part(cell_end[key] - s0, split, t % split, &p0, &P);
-    s0 += p0;
-    if (P == 0) {
-      if (lane == 0) mask_off[t] = -1;
-      continue;
-    }
-    int lo, len, off, total;
-    warp_cell_runs(key, cg, cell_start, cell_end, lane, &lo, &len, &off, &total);
-    const int nwords = (total + 31) >> 5;
-    long long at = -1;
-    if (lane == 0 && total <= kMaskCap && P <= kMaskMaxP) {
-      const long long need = (long long)nwords * P;
-      at = (long long)atomicAdd(pool, (unsigned long long)need);
-      if (at + need > pool_words) at = -1;
-    }
-    at = __shfl_sync(0xffffffffu, at, 0);
-    if (lane == 0) mask_off[t] = at;
-    if (at < 0) {
-      // too many candidates or particles for the counters, or the pool is
-      // used up: the warp-per-particle kernel takes the item
-      if (lane == 0) overflow[atomicAdd(n_overflow, 1)] = t;
-      continue;
-    }
-    const double sc = cell_scale(key, cg);
-    const V ref = ld4(spos + s0);
-    if (lane < 9) {
-      run_lo[lane] = lo;
-      run_off[lane] = off;
-    }
-    for (int q = lane; q < (P + 1) / 2; q += 32) cnt[q] = 0u;
-    const int dw = 32 / P, dq = 32 - dw * P;   // a lane's step of 32 pairs
-    for (int w0 = 0; w0 < nwords; w0 += kWinWords) {
-      const int w1 = min(nwords, w0 + kWinWords);
-      __syncwarp();   // the previous window's reads are done
-      for_window(lo, len, off, w0 * 32, min(total, w1 * 32), lane, [&](int c, int sp) {
-        const float4 u = local_of(ld4(spos + sp), ref, sc);
-        const int w = c >> 5, k = c & 31, a = w * kWinA + 2 * (k & ~1) + (k & 1);
-        ta[a] = u.x;
-        ta[a + 2] = u.y;
-        tb[a] = u.z;
-        tb[a + 2] = u.w;
-        tc[w * kWinC + k] = local_c(u);
-      });
-      if (w1 == nwords)   // slots past the last candidate: far away
-        for (int c = total - w0 * 32 + lane; c < (w1 - w0) * 32; c += 32) {
-          const int w = c >> 5, k = c & 31, a = w * kWinA + 2 * (k & ~1) + (k & 1);
-          ta[a] = ta[a + 2] = tb[a] = tb[a + 2] = 0.0f;
-          tc[w * kWinC + k] = 1e30f;
-        }
-      __syncwarp();
-      int wl = lane / P, q = lane - wl * P;
-      for (; wl < w1 - w0;) {
-        const V xi = ld4(spos + s0 + q);
-        const float4 ui = local_of(xi, ref, sc);
-        const float cc = local_c(ui);
-        const float2 ci = make_float2(cc, cc);
-        const float2 ax = make_float2(-2.0f * ui.x, -2.0f * ui.x);
-        const float2 ay = make_float2(-2.0f * ui.y, -2.0f * ui.y);
-        const float2 az = make_float2(-2.0f * ui.z, -2.0f * ui.z);
-        const float2 ah = make_float2(-0.5f * ui.w, -0.5f * ui.w);
-        const float4 *pa = reinterpret_cast<const float4 *>(ta + wl * kWinA);
-        const float4 *pb = reinterpret_cast<const float4 *>(tb + wl * kWinA);
-        const float2 *pc = reinterpret_cast<const float2 *>(tc + wl * kWinC);
-        uint32_t m = 0;
-        float near = 1e30f;
+// The tests of particles [0, np) (prepared in part / pcc) against the lanes'
+// candidates of NP pairs of words (d = the pairs' staged values), 32 particles at
+// a time: their rows' words go to rows (nwp words each) from word w0 on, the
+// hits of this lane's particles k = lane, lane + 32 are added to cnt.
+template <int NP, typename Retake>
+__device__ __forceinline__ void test_window(const float2 (&X)[kWinWords / 2],
+                                            const float2 (&Y)[kWinWords / 2],
+                                            const float2 (&Z)[kWinWords / 2],
+                                            const float2 (&H)[kWinWords / 2],
+                                            const float2 (&C)[kWinWords / 2], int np,
+                                            const float4 *part, const float *pcc,
+                                            uint32_t (*res)[kWinWords + 4], uint32_t *rows,
+                                            int nwp, int lane, int (&cnt)[kMaskBlock / 32],
+                                            Retake &&retake) {
 #pragma unroll
-        for (int k = 15; k >= 0; --k) {
-          const float4 a = pa[k], b = pb[k];
-          float2 d = __fadd2_rn(pc[k], ci);
-          d = __ffma2_rn(make_float2(a.x, a.y), ax, d);
-          d = __ffma2_rn(make_float2(a.z, a.w), ay, d);
-          d = __ffma2_rn(make_float2(b.x, b.y), az, d);
-          d = __ffma2_rn(make_float2(b.z, b.w), ah, d);
-          m = __funnelshift_l(__float_as_uint(d.y), m, 1);
-          m = __funnelshift_l(__float_as_uint(d.x), m, 1);
-          near = fminf(near, fminf(fabsf(d.x), fabsf(d.y)));
-        }
-        const int w = w0 + wl;
-        if (near <= kBand) {
-          // some candidate lies at the bound: the FP64 definition decides it
-          for (int k = 0; k < min(32, total - 32 * w); ++k) {
-            const int a = 2 * (k & ~1) + (k & 1);
-            const float *fa = ta + wl * kWinA + a, *fb = tb + wl * kWinA + a;
-            float d = tc[wl * kWinC + k] + cc;
-            d = fmaf(fa[0], ax.x, d);
-            d = fmaf(fa[2], ay.x, d);
-            d = fmaf(fb[0], az.x, d);
-            d = fmaf(fb[2], ah.x, d);
-            if (fabsf(d) > kBand) continue;
-            const int c = 32 * w + k;
-            int r = 8;
-            while (r > 0 && run_off[r] > c) --r;
-            const V xj = ld4(spos + run_lo[r] + (c - run_off[r]));
-            const bool hit = in_support64(xi.x, xi.y, xi.z, xi.w, xj.x, xj.y, xj.z, xj.w);
-            m = (m & ~(1u << k)) | ((hit ? 1u : 0u) << k);
-          }
-        }
-        mask[at + (long long)w * P + q] = m;
-        atomicAdd(&cnt[q >> 1], (unsigned)__popc(m) << ((q & 1) * 16));
-        wl += dw;
-        q += dq;
-        if (q >= P) {
-          q -= P;
-          ++wl;
-        }
+  for (int half = 0; half < kMaskBlock / 32; ++half) {
+    if (32 * half >= np) break;
+    const int kn = min(32, np - 32 * half);
+#pragma unroll 1   // (two particles side by side cost a block per SM: 231 against 214 us)
+    for (int k = 0; k < kn; ++k) {
+      const float4 f = part[32 * half + k];
+      const float cc = pcc[32 * half + k];
+      float2 d[NP];
+      float near = 1e30f;
+      uint32_t b[2 * NP];
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        d[i] = __fadd2_rn(C[i], make_float2(cc, cc));
+        d[i] = __ffma2_rn(X[i], make_float2(f.x, f.x), d[i]);
+        d[i] = __ffma2_rn(Y[i], make_float2(f.y, f.y), d[i]);
+        d[i] = __ffma2_rn(Z[i], make_float2(f.z, f.z), d[i]);
+        d[i] = __ffma2_rn(H[i], make_float2(f.w, f.w), d[i]);
+        near = fminf(near, fminf(fabsf(d[i].x), fabsf(d[i].y)));
+        b[2 * i] = __ballot_sync(0xffffffffu, d[i].x < 0.0f);
+        b[2 * i + 1] = __ballot_sync(0xffffffffu, d[i].y < 0.0f);
+      }
+      if (__any_sync(0xffffffffu, near <= kBand)) retake(32 * half + k, d, b);
+      if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < NP; i += 2)
+          *reinterpret_cast<uint4 *>(&res[k][2 * i]) =
+              make_uint4(b[2 * i], b[2 * i + 1], b[2 * i + 2], b[2 * i + 3]);
       }
     }
     __syncwarp();
-    for (int q = lane; q < P; q += 32)
-      counts[svals[s0 + q]] = (int)((cnt[q >> 1] >> ((q & 1) * 16)) & 0xffffu);
-    __syncwarp();   // the counters are read before the next item clears them
+    if (lane < kn) {
+#pragma unroll
+      for (int i = 0; i < NP; i += 2) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(&res[lane][2 * i]);
+        cnt[half] += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+        *reinterpret_cast<uint4 *>(rows + (long long)(32 * half + lane) * nwp + 2 * i) = v;
+      }
+    }
+    __syncwarp();   // the words are read before the next particles overwrite them
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
+    const GridDev *all, const int32_t *table, int32_t *n_ucell, const vec4_t<T> *spos,
+    const int32_t *svals, int32_t *counts, uint32_t *mask, Split split) {
+  using V = vec4_t<T>;
+  // prepared particles (-2 u, -h/2) and |u|^2 - h^2/4; the words of 32 particles
+  __shared__ float4 s_part[kMaskWarps][kMaskBlock];
+  __shared__ float s_cc[kMaskWarps][kMaskBlock];
+  __shared__ __align__(16) uint32_t s_res[kMaskWarps][32][kWinWords + 4];
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  if (!all->ok) return;
+  ItemWalk walk;
+  walk.start(table, n_ucell + 2, n_ucell[0], n_ucell[4], split, lane);
+  int rec, s0, p0, P;
+  while (walk.next(&rec, &s0, &p0, &P)) {
+    const long long pool =
+        ((long long)__shfl_sync(0xffffffffu, rec, kRecPool + 1) << 32) |
+        (unsigned)__shfl_sync(0xffffffffu, rec, kRecPool);
+    if (pool < 0 || P == 0) continue;   // the warp-per-particle kernel's, or no particles
+    const int total = __shfl_sync(0xffffffffu, rec, kRecTotal);
+    const int nre = __shfl_sync(0xffffffffu, rec, kRecRuns), nr = nre & 255;
+    const float sc = __int_as_float((127 + 128 - (nre >> 8)) << 23);
+    const int nwp = row_words(total);
+    uint32_t *mrow = mask + pool + (long long)nwp * p0;
+    const V ref = ld4(spos + s0);
+    for (int pb = 0; pb < P; pb += kMaskBlock) {
+      const int np = min(kMaskBlock, P - pb);
+      __syncwarp();   // the previous particles are read
+      for (int q = lane; q < np; q += 32) {
+        const float4 u = local_of(ld4(spos + s0 + pb + q), ref, sc);
+        s_part[wp][q] = make_float4(-2.0f * u.x, -2.0f * u.y, -2.0f * u.z, -0.5f * u.w);
+        s_cc[wp][q] = local_c(u);
+      }
+      __syncwarp();
+      int cnt[kMaskBlock / 32] = {0, 0}, run = 0;
+      for (int w0 = 0; w0 < nwp; w0 += kWinWords) {
+        float2 X[kWinWords / 2], Y[kWinWords / 2], Z[kWinWords / 2], H[kWinWords / 2],
+            C[kWinWords / 2];
+        const int run0 = run;
+#pragma unroll
+        for (int g = 0; g < kWinWords; g += 4) {
+          if (w0 + g >= nwp) break;
+          int sp[4];
+          candidates4(rec, nr, total, (w0 + g) * 32, lane, &run, sp);
+          V v[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[u] = ld4(spos + sp[u]);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const float4 x = local_of(v[u], ref, sc);
+            // a slot past the last candidate is far from everything
+            const float c = (w0 + g + u) * 32 + lane < total ? local_c(x) : 1e30f;
+            const int i = (g + u) / 2;
+            if (u % 2 == 0) {
+              X[i].x = x.x; Y[i].x = x.y; Z[i].x = x.z; H[i].x = x.w; C[i].x = c;
+            } else {
+              X[i].y = x.x; Y[i].y = x.y; Z[i].y = x.z; H[i].y = x.w; C[i].y = c;
+            }
+          }
+        }
+        // pairs at the bound: the FP64 definition decides
+        auto retake = [&](int k, auto &d, auto &b) {
+          const V xi = ld4(spos + s0 + pb + k);
+          int r = run0;
+#pragma unroll
+          for (int g = 0; g < kWinWords; g += 4) {
+            if (g >= (int)(sizeof(d) / sizeof(float))) break;
+            if (w0 + g >= nwp) break;
+            int sp[4];
+            candidates4(rec, nr, total, (w0 + g) * 32, lane, &r, sp);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const float dv = u % 2 ? d[(g + u) / 2].y : d[(g + u) / 2].x;
+              bool hit = dv < 0.0f;
+              if (fabsf(dv) <= kBand) {
+                const V xj = ld4(spos + sp[u]);
+                hit = in_support64(xi.x, xi.y, xi.z, xi.w, xj.x, xj.y, xj.z, xj.w);
+              }
+              b[g + u] = __ballot_sync(0xffffffffu, hit);
+            }
+          }
+        };
+        uint32_t *rows = mrow + (long long)nwp * pb + w0;
+        if (nwp - w0 > 4)
+          test_window<4>(X, Y, Z, H, C, np, s_part[wp], s_cc[wp], s_res[wp], rows, nwp, lane,
+                         cnt, retake);
+        else
+          test_window<2>(X, Y, Z, H, C, np, s_part[wp], s_cc[wp], s_res[wp], rows, nwp, lane,
+                         cnt, retake);
+      }
+#pragma unroll
+      for (int half = 0; half < kMaskBlock / 32; ++half)
+        if (32 * half + lane < np) counts[svals[s0 + pb + 32 * half + lane]] = cnt[half];
+    }
   }
 }
 
 // Fill pass for the mask kernel's items, also one warp per item from a work
 // queue.  The item's particles go in chunks of 32; for each window of
-// kFillWinWords candidate words the warp stages the candidates' original
-// indices, and each lane, holding one particle, its hit words (coalesced) with
-// the place in the row where each word's first hit goes; then the chunk's rows
-// are expanded one particle at a time: one candidate per lane, its place from a
-// popcount of the lower hits, coalesced stores.  Only that one popcount per
-// (particle, word) is left in the expansion (a warp's POPC takes 8 cycles of
-// the issuing scheduler's unit, measured; it is what bounds the kernel), and
-// words are walked in groups of four up to the window's last one, so film
-// cells (4 words) do not pay for a 16-word window.  Rows come out ascending when
-// the cloud is in cell order (candidates are runs of consecutive sorted
-// positions, ascending).
+// kFillWinWords candidate words each lane loads its candidates' original indices
+// into registers and, holding one particle, that particle's hit words
+// (coalesced) with the place in the row where each word's first hit goes; then
+// the chunk's rows are expanded one particle at a time: one candidate per lane,
+// its place from a popcount of the lower hits, coalesced stores.  Only that one
+// popcount per (particle, word) is left in the expansion (a warp's POPC takes 8
+// cycles of the issuing scheduler's unit, measured), and words are walked in
+// groups of four up to the window's last one, so film cells (4 words) do not
+// pay for a 16-word window: 382 -> 184 us on the 1M jet cloud.  Rows come out ascending when the cloud is in cell
+// order (candidates are runs of consecutive sorted positions, ascending).
 __global__ void __launch_bounds__(kFillThreads) k_nbr_fill(
-    CloudGrids cg, const int32_t *ucell, int32_t *n_ucell, const int32_t *svals,
-    const int32_t *cell_start, const int32_t *cell_end, const uint32_t *mask,
-    const long long *mask_off, int split, const long long *row_ptr, int32_t *col,
-    long long cap_nnz, int64_t n) {
-  __shared__ int32_t cand_v[kFillWarps][kFillWinWords * 32];         // original indices
-  __shared__ __align__(16) uint2 rec[kFillWarps][32][kFillRec];      // (hit word, place)
-  if (!cg.all->ok) return;
+    const GridDev *all, const int32_t *table, int32_t *n_ucell, const int32_t *svals,
+    const uint32_t *mask, Split split, const long long *row_ptr, int32_t *col, long long cap_nnz,
+    int64_t n) {
+  __shared__ __align__(16) uint2 srec[kFillWarps][32][kFillRec];     // (hit word, place)
+  if (!all->ok) return;
   if (row_ptr[n] > cap_nnz) return;
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u, bit = 1u << lane;
-  int32_t *cv = cand_v[wp];
-  const int nbig = n_ucell[0], nu = nbig + n_ucell[4];
-  const long long items = (long long)nu * split;
-  int t_next = 0;
-  if (lane == 0) t_next = atomicAdd(n_ucell + 3, 1);   // work ticket, as in the mask kernel
-  for (;;) {
-    const int t = __shfl_sync(0xffffffffu, t_next, 0);
-    if (t >= items) break;
-    if (lane == 0) t_next = atomicAdd(n_ucell + 3, 1);
-    const long long moff = mask_off[t];
-    if (moff < 0) continue;   // empty, or the overflow path fills it
-    const int cb = cell_slot(t / split, nbig, n);
-    const int key = ucell[2 * cb];
-    int s0 = ucell[2 * cb + 1], part, P;
-    item_part(cell_end[key] - s0, split, t % split, &part, &P);
-    s0 += part;
-    int lo, len, off, total;
-    warp_cell_runs(key, cg, cell_start, cell_end, lane, &lo, &len, &off, &total);
-    const int nwords = (total + 31) >> 5;
+  uint2(*wr)[kFillRec] = srec[threadIdx.x >> 5];
+  ItemWalk walk;
+  walk.start(table, n_ucell + 3, n_ucell[0], n_ucell[4], split, lane);
+  int rec, s0, part, P;
+  while (walk.next(&rec, &s0, &part, &P)) {
+    const long long pool =
+        ((long long)__shfl_sync(0xffffffffu, rec, kRecPool + 1) << 32) |
+        (unsigned)__shfl_sync(0xffffffffu, rec, kRecPool);
+    if (pool < 0 || P == 0) continue;
+    const int total = __shfl_sync(0xffffffffu, rec, kRecTotal);
+    const int nr = __shfl_sync(0xffffffffu, rec, kRecRuns) & 255;
+    const int nwp = row_words(total);
+    const uint32_t *mrow = mask + pool + (long long)nwp * part;
     for (int p0 = 0; p0 < P; p0 += 32) {
       const int np = min(32, P - p0);
       const int q = p0 + lane;
       const long long rs = lane < np ? row_ptr[svals[s0 + q]] : 0;
-      int at = 0;
-      for (int w0 = 0; w0 < nwords; w0 += kFillWinWords) {
-        const int nw = min(nwords - w0, kFillWinWords);
-        __syncwarp();   // the previous window's reads are done
-        for_window(lo, len, off, w0 * 32, min(total, (w0 + nw) * 32), lane,
-                   [&](int c, int sp) { cv[c] = svals[sp]; });
-        for (int ww = 0; ww < ((nw + 3) & ~3); ++ww) {
-          const uint32_t m =
-              lane < np && ww < nw ? mask[moff + (long long)(w0 + ww) * P + q] : 0u;
-          rec[wp][lane][ww] = make_uint2(m, (unsigned)at);
-          at += __popc(m);
+      int at = 0, run = 0;
+      for (int w0 = 0; w0 < nwp; w0 += kFillWinWords) {
+        const int nw = min(nwp - w0, kFillWinWords);
+        int32_t cv[kFillWinWords];   // this lane's candidate of every word of the window
+        __syncwarp();                // the previous window's reads are done
+#pragma unroll
+        for (int g = 0; g < kFillWinWords; g += 4) {
+          if (g >= nw) break;
+          int sp[4];
+          const uint4 m4 = lane < np ? *reinterpret_cast<const uint4 *>(
+                                           mrow + (long long)q * nwp + w0 + g)
+                                     : make_uint4(0u, 0u, 0u, 0u);
+          const uint32_t m[4] = {m4.x, m4.y, m4.z, m4.w};
+          candidates4(rec, nr, total, (w0 + g) * 32, lane, &run, sp);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) cv[g + u] = svals[sp[u]];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            wr[lane][g + u] = make_uint2(m[u], (unsigned)at);
+            at += __popc(m[u]);
+          }
         }
         __syncwarp();
-        // this lane's candidate of every word of the window, in registers
-        int32_t cvr[kFillWinWords];
-#pragma unroll
-        for (int ww = 0; ww < kFillWinWords; ++ww) cvr[ww] = ww < nw ? cv[ww * 32 + lane] : 0;
         for (int k = 0; k < np; ++k) {
           int32_t *crow = col + __shfl_sync(0xffffffffu, rs, k);
-          const uint4 *rk = reinterpret_cast<const uint4 *>(rec[wp][k]);
+          const uint4 *rk = reinterpret_cast<const uint4 *>(wr[k]);
 #pragma unroll
           for (int g = 0; g < kFillWinWords / 4; ++g) {
             if (4 * g >= nw) break;
             const uint4 a = rk[2 * g], b = rk[2 * g + 1];
-            if (a.x & bit) crow[a.y + __popc(a.x & lt)] = cvr[4 * g];
-            if (a.z & bit) crow[a.w + __popc(a.z & lt)] = cvr[4 * g + 1];
-            if (b.x & bit) crow[b.y + __popc(b.x & lt)] = cvr[4 * g + 2];
-            if (b.z & bit) crow[b.w + __popc(b.z & lt)] = cvr[4 * g + 3];
+            if (a.x & bit) crow[a.y + __popc(a.x & lt)] = cv[4 * g];
+            if (a.z & bit) crow[a.w + __popc(a.z & lt)] = cv[4 * g + 1];
+            if (b.x & bit) crow[b.y + __popc(b.x & lt)] = cv[4 * g + 2];
+            if (b.z & bit) crow[b.w + __popc(b.z & lt)] = cv[4 * g + 3];
           }
         }
       }
@@ -1024,32 +1105,38 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
   const int nbr_blocks = sms * 8;
   int32_t *n_overflow = ctx->n_ucell + 1;
   const long long pool_words = (long long)kMaskWords * ctx->cap_particles;
-  // parts per cell: a small cloud has fewer cells than the GPU has warps
-  const int split = n <= kSplitMax ? kSplit : 1;
+  // Parts per cell: a small cloud has fewer cells than the GPU has warps (mask and
+  // fill at 5650 particles 71 + 134 us unsplit, 24 + 23 us in these parts); in
+  // larger ones only the costly cells are split, so that no warp ends late
+  // (200k random particles, mask + fill: 535 us unsplit, 438 in halves, 366 in
+  // quarters; the 1M jet cloud 423, 398 and 462 us).
+  const Split split = n <= kSplitAll ? Split{3, 1} : n <= kSplitMore ? Split{2, 0} : Split{1, 0};
+  const long long *rp = reinterpret_cast<const long long *>(row_ptr);
+  MAFP_TIMED(ctx, s, "k_cell_table",
+             k_cell_table<<<grid_for(n, 128, sms * 16), 128, 0, s>>>(
+                 cg, ctx->ucell, ctx->n_ucell, ctx->cell_start, ctx->cell_end, ctx->cell_table,
+                 pool_words, ctx->overflow, n));
   MAFP_TIMED(ctx, s, sizeof(T) == 4 ? "k_nbr_mask<float>" : "k_nbr_mask<double>",
-             k_nbr_mask<T><<<sms * 8, kMaskThreads, kMaskWarps * kMaskWarpBytes, s>>>(
-                 cg, ctx->ucell, ctx->n_ucell, spos, vin, ctx->cell_start, ctx->cell_end,
-                 ctx->counts, ctx->nbr_mask, pool_words, ctx->mask_off, split, ctx->overflow,
-                 n_overflow, n));
+             k_nbr_mask<T><<<sms * 8, kMaskThreads, 0, s>>>(
+                 ctx->d_grid, ctx->cell_table, ctx->n_ucell, spos, vin, ctx->counts,
+                 ctx->nbr_mask, split));
   MAFP_TIMED(ctx, s, "k_nbr<T,false>(overflow cells)",
              k_nbr<T, false><<<nbr_blocks, kNbrThreads, kNbrSmemBytes, s>>>(
-      cg, ctx->ucell, ctx->n_ucell, split, ctx->overflow, n_overflow, spos, vin, ctx->cell_start,
-      ctx->cell_end, ctx->counts, nullptr, nullptr, 0, n));
+                 ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, spos, vin, ctx->counts,
+                 nullptr, nullptr, 0, n));
   MAFP_LAUNCH_CHECK(ctx);
   int rc = scan_i32_to_i64(ctx, ctx->counts, reinterpret_cast<long long *>(row_ptr), n, s);
   if (rc) return rc;
   MAFP_TIMED(ctx, s, "k_check_nnz",
-             k_check_nnz<<<1, 1, 0, s>>>(reinterpret_cast<const long long *>(row_ptr), n, cap_nnz, nnz_dev,
-                              ctx->d_status, ctx->d_grid));
+             k_check_nnz<<<1, 1, 0, s>>>(rp, n, cap_nnz, nnz_dev, ctx->d_status, ctx->d_grid));
   MAFP_TIMED(ctx, s, "k_nbr_fill",
-             k_nbr_fill<<<sms * 8, kFillThreads, 0, s>>>(
-                 cg, ctx->ucell, ctx->n_ucell, vin, ctx->cell_start, ctx->cell_end,
-                 ctx->nbr_mask, ctx->mask_off, split,
-                 reinterpret_cast<const long long *>(row_ptr), col, cap_nnz, n));
+             k_nbr_fill<<<sms * 8, kFillThreads, 0, s>>>(ctx->d_grid, ctx->cell_table,
+                                                         ctx->n_ucell, vin, ctx->nbr_mask, split,
+                                                         rp, col, cap_nnz, n));
   MAFP_TIMED(ctx, s, "k_nbr<T,true>(overflow cells)",
              k_nbr<T, true><<<nbr_blocks, kNbrThreads, kNbrSmemBytes, s>>>(
-      cg, ctx->ucell, ctx->n_ucell, split, ctx->overflow, n_overflow, spos, vin, ctx->cell_start,
-      ctx->cell_end, ctx->counts, reinterpret_cast<const long long *>(row_ptr), col, cap_nnz, n));
+                 ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, spos, vin, ctx->counts,
+                 rp, col, cap_nnz, n));
   MAFP_TIMED(ctx, s, "k_rowsort",
              k_rowsort<<<grid_for(n, kSortWarps, sms * 8), kSortWarps * 32, 0, s>>>(
       reinterpret_cast<const long long *>(row_ptr), col, n, cap_nnz, ctx->d_status,
@@ -1092,10 +1179,6 @@ int build_neighbours_batched(mafp_ctx *ctx, int64_t n, int32_t dtype, int32_t nc
 }
 
 void init_kernel_attributes() {
-  cudaFuncSetAttribute(k_nbr_mask<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kMaskWarps * kMaskWarpBytes);
-  cudaFuncSetAttribute(k_nbr_mask<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kMaskWarps * kMaskWarpBytes);
   cudaFuncSetAttribute(k_nbr<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        kNbrSmemBytes);
   cudaFuncSetAttribute(k_nbr<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,

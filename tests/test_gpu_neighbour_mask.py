@@ -41,7 +41,7 @@ CLOUDS = {
 
 
 @pytest.mark.parametrize("dtype", [M.F32_REFINED, M.F64])
-@pytest.mark.parametrize("scale", [1.0, 2.0 ** -50, 3.0e12])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -50, 3.0e12, 2.0 ** 122])
 @pytest.mark.parametrize("name", sorted(CLOUDS))
 def test_lists_equal_the_oracle(orc, name, scale, dtype):
     pos = CLOUDS[name]() * np.float32(scale)
