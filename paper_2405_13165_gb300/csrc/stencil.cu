@@ -1,9 +1,9 @@
 // stencil.cu -- GFDM stencils of Eq. GFDM_Definition (Sec. 2.3), order 2.
 //
-// One group of G lanes per particle (G = 32 for 3D rows of ~180 entries, 8 for
-// 2D rows of ~40).  Lanes stride over the row, accumulate the packed moment
-// matrix A = sum_j w_j p_j p_j^T, reduce it with a reduce-scatter of shuffles,
-// factor it (Cholesky) and solve for the four right-hand sides in every lane.
+// One group of G lanes per particle (8 for 3D rows of ~180 entries, 4 for film
+// rows of ~40).  Lanes stride over the row, accumulate the distinct moments of
+// A = sum_j w_j p_j p_j^T, reduce them with a reduce-scatter of shuffles, factor
+// A (Cholesky) and solve for the four right-hand sides, one per lane.
 // FP32 path: one refinement step with the residual b - sum_j c_j p_j of the
 // rounded coefficients; particles whose Cholesky pivots are too small or whose
 // condition estimate exceeds cond_fp64 are queued and redone in FP64.
@@ -12,33 +12,383 @@
 
 namespace mafp {
 
+// Clouds of at most kStFewRows particles take the wide groups (too few rows for
+// the GPU's warps otherwise); of more than kStManyRows, four rounds per warp.
+constexpr int64_t kStFewRows = 16384, kStManyRows = 65536;
+
+// Two warps per block: a block's slot is free again as soon as its two warps'
+// rows are done (1M jet cloud, 3D rows: 847 us against 925 with four warps).
+constexpr int kBuildThreads = 64;
+
 __global__ void k_reset_queue(DevStatus *st) { st->fallback_count = 0; }
 
-// Per-lane cache of (q, w) for the refinement and coefficient passes (FP32
-// path): 176 entries per 3D row, 48 per film row; entries beyond it are
-// gathered and recomputed as in the first pass.
+// Per-lane cache for the passes after the moments.  FP32: (q, w) of two entries
+// together, (q1a, q1b, q2a, q2b) and (q3a, q3b, wa, wb), KC entries per lane (176
+// per 3D row, 40 per film row).  FP64: w alone (its exponential is ~25 of the ~55
+// FP64 operations that the coefficient pass spends on an entry).  Entries beyond
+// it are gathered and recomputed as in the first pass.
 template <typename C, int M, int G>
 struct StCache {
-  static constexpr int KC = sizeof(C) == 4 ? (M == 10 ? 176 : 48) / G : 0;
-  static constexpr int BYTES = (kStThreads / G) * KC * G * (int)sizeof(float4);
-  static constexpr int SMEM = BYTES + (kStThreads / G) * StSmem<M, G>::PER_GROUP * (int)sizeof(C);
+  static constexpr int KC = pad_to((M == 10 ? 176 : 40) / G, 2);
+  static constexpr int BYTES = kBuildThreads * KC * (sizeof(C) == 4 ? (int)sizeof(float4) : 8);
+  static constexpr int SMEM = BYTES + (kBuildThreads / G) * StSmem<M, G>::PER_GROUP * (int)sizeof(C);
 };
 
 // neighbours a lane gathers ahead of use: 4 for 3D rows (long rows, the loads
 // in flight together), 2 for film rows
 template <int M> constexpr int kGatherU = M == 10 ? 4 : 2;
-constexpr int kGatherR = 2;   // the same in the refinement pass (more live registers)
 
-// Process particle i with a group of G lanes.  Returns (through *result)
-//  0 = written, 1 = deficient (zeros written), 2 = queued for FP64.
-template <typename TS, typename C, int M, int G, bool REFINE, bool QUEUE, int KC = 0>
+// ------------------------------------------------------------------ FP32 rows
+// The passes over a row in packed FP32 (two operations per instruction; the FMA
+// pipe retires them at the scalar rate, so what falls is the number of
+// instructions issued).  The refinement and coefficient passes pack two
+// right-hand sides (the coefficients of one entry side by side: lambda_k stays
+// in registers once); the moment pass packs the weights and coordinates of two
+// entries.
+// What bounds it (3D, ncu on 300k particles): ~6000 instructions per round of
+// four rows, 57 % of them FP32; the FMA pipe is busy ~60 % of the time (a packed
+// FMA with three different operands takes 3 cycles of it, measured) at 14 warps
+// per SM, the registers' limit.  Film rows: L1 wavefronts (56 % busy) and issue
+// (53 %).  1M jet cloud, 3D 890 -> 794 us, film 300 -> 252 us; with the launch
+// shapes of a new context (32 and 8 lanes before) 2136 -> 951 us for 440k 3D rows.
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  return __ffma2_rn(a, b, c);
+}
+
+// Monomials p_1.. of two packed coordinate triples (pairs in 2D); p_0 = 1 is implied.
+template <int M>
+__device__ __forceinline__ void basis2(float2 a, float2 b, float2 c, float2 (&p)[M]) {
+  if constexpr (M == 10) {
+    p[1] = a; p[2] = b; p[3] = c;
+    p[4] = mul2(a, a); p[5] = mul2(b, b); p[6] = mul2(c, c);
+    p[7] = mul2(a, b); p[8] = mul2(a, c); p[9] = mul2(b, c);
+  } else {
+    p[1] = a; p[2] = b;
+    p[3] = mul2(a, a); p[4] = mul2(a, b); p[5] = mul2(b, b);
+  }
+}
+
+// Process particle i (FP32) with a group of G lanes; results as stencil_particle.
+template <int M, int G, bool REFINE>
+__device__ __forceinline__ void stencil_row32(int64_t i, const float4 *pos, const uint8_t *model,
+                                              const float4 *frame, const long long *row_ptr,
+                                              const int32_t *col, float4 *coef,
+                                              const StParams<float> &sp, float *sm, int *result,
+                                              float *cond_out, float4 *qw) {
+  constexpr int NA = Basis<M>::NA, NR = Basis<M>::NR, KL = NR - 1;
+  constexpr int VR = pad_to(NR * M, G), VM = pad_to(Moments<M>::N, G);
+  constexpr int KP = StCache<float, M, G>::KC / 2, U = kGatherU<M>;
+  const int lane = threadIdx.x & (G - 1);
+  const unsigned gm = group_mask<G>();
+  const float4 xi = ld4(pos + i);
+  const uint8_t mi = model[i];
+  const float hinv = 1.0f / xi.w, h2inv = hinv * hinv;
+  float t1[3] = {0, 0, 0}, t2[3] = {0, 0, 0};
+  if constexpr (M == 6) {
+    const float4 f1 = ld4(frame + 2 * i), f3 = ld4(frame + 2 * i + 1);
+    t1[0] = f1.x; t1[1] = f1.y; t1[2] = f1.z;
+    t2[0] = f3.y * t1[2] - f3.z * t1[1];
+    t2[1] = f3.z * t1[0] - f3.x * t1[2];
+    t2[2] = f3.x * t1[1] - f3.y * t1[0];
+  }
+  const long long b = row_ptr[i];
+  const int len = (int)(row_ptr[i + 1] - b);
+  col += b;
+  coef += b;
+
+  // U neighbours of the lane (entries e, e + G, ... of the row, their columns
+  // given), gathered before any of them is used; slots past the row end load
+  // particle i itself and are marked invalid, as are neighbours of the other model
+  auto columns = [&](int e, int (&j)[U]) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) j[u] = e + u * G < len ? col[e + u * G] : -1;
+  };
+  auto gather = [&](const int *j, int nu, float4 *x, bool *ok) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (u < nu) {
+        const int jj = j[u] >= 0 ? j[u] : (int)i;
+        x[u] = ld4(pos + jj);
+        ok[u] = j[u] >= 0 && model[jj] == mi;
+      }
+  };
+  // (q, w) of two entries, gathered by the caller; w = 0 where an entry is not one
+  auto locate = [&](const float4 &xa, const float4 &xb, bool oka, bool okb, float2 &qa, float2 &qb,
+                    float2 &qc, float2 &w) {
+    const float2 dx = make_float2(xa.x - xi.x, xb.x - xi.x);
+    const float2 dy = make_float2(xa.y - xi.y, xb.y - xi.y);
+    const float2 dz = make_float2(xa.z - xi.z, xb.z - xi.z);
+    const float2 s2 = mul2(fma2(dz, dz, fma2(dx, dx, mul2(dy, dy))), dup2(h2inv));
+    const float2 e = make_float2(expf(-sp.alpha * s2.x), expf(-sp.alpha * s2.y));
+    w = mul2(add2(e, dup2(-sp.ea)), dup2(sp.inv_den));
+    w.x = oka && s2.x <= 1.0f ? w.x : 0.0f;
+    w.y = okb && s2.y <= 1.0f ? w.y : 0.0f;
+    const float2 hh = dup2(hinv);
+    if constexpr (M == 10) {
+      qa = mul2(dx, hh); qb = mul2(dy, hh); qc = mul2(dz, hh);
+    } else {
+      qa = mul2(fma2(dz, dup2(t1[2]), fma2(dx, dup2(t1[0]), mul2(dy, dup2(t1[1])))), hh);
+      qb = mul2(fma2(dz, dup2(t2[2]), fma2(dx, dup2(t2[0]), mul2(dy, dup2(t2[1])))), hh);
+      qc = qb;
+    }
+  };
+
+  // ---- moments (the distinct ones), summed one entry after another: two packed
+  // entries would take 70 sums and with them the registers of a third of the warps
+  float A[VM];
+#pragma unroll
+  for (int k = 0; k < VM; ++k) A[k] = 0.0f;
+  int cnt = 0, kp = 0;
+  // the columns are loaded a round ahead of their use (the records too: 828
+  // against 805 us in 3D, no difference for film)
+  int js[U];
+  columns(lane, js);
+#pragma unroll 1
+  for (int e0 = lane; e0 < len; e0 += U * G, kp += U / 2) {
+    float4 xs[U];
+    bool oks[U];
+    gather(js, U, xs, oks);
+    columns(e0 + U * G, js);
+#pragma unroll
+    for (int u = 0; u < U; u += 2) {
+      float2 q[3], w;
+      locate(xs[u], xs[u + 1], oks[u], oks[u + 1], q[0], q[1], q[2], w);
+      cnt += (oks[u] ? 1 : 0) + (oks[u + 1] ? 1 : 0);
+      if (kp + u / 2 < KP) {
+        float4 *c = qw + 64 * (kp + u / 2);
+        c[0] = make_float4(q[0].x, q[0].y, q[1].x, q[1].y);
+        c[32] = make_float4(q[2].x, q[2].y, w.x, w.y);
+      }
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          float p[M];
+          const float x = v ? q[0].y : q[0].x, y = v ? q[1].y : q[1].x, z = v ? q[2].y : q[2].x;
+          p[0] = 1.0f; p[1] = x; p[2] = y;
+          if constexpr (M == 10) {
+            p[3] = z;
+            p[4] = x * x; p[5] = y * y; p[6] = z * z; p[7] = x * y; p[8] = x * z; p[9] = y * z;
+          } else {
+            p[3] = x * x; p[4] = x * y; p[5] = y * y;
+          }
+          add_moments<M, float, VM>(A, v ? w.y : w.x, p);
+        }
+    }
+  }
+  reduce_scatter<G, VM>(A);
+  __syncwarp(gm);
+#pragma unroll
+  for (int k = 0; k < VM / G; ++k) sm[lane * (VM / G) + k] = A[k];
+  float L[NA];
+  cnt = group_sum<G>(cnt);
+  __syncwarp(gm);
+  constexpr MomentTable<M> MT = Moments<M>::T;
+#pragma unroll
+  for (int k = 0; k < NA; ++k) L[k] = sm[MT.idx[k]];
+  __syncwarp(gm);
+  float tr = 0;
+#pragma unroll
+  for (int r = 0; r < M; ++r) tr += L[pk(r, r)];
+  float invd[M], pmin, pmax;
+  const bool pd = cholesky<M, float, REFINE && M == 10>(L, invd, sp.piv_tol_rel * tr, pmin, pmax);
+  const bool ok = pd && cnt >= M;
+  const float cond = (pmax / pmin) * (pmax / pmin);
+  float *Ls = sm + StSmem<M, G>::SCR;
+  if (lane == 0) {
+#pragma unroll
+    for (int k = 0; k < NA; ++k) Ls[k] = L[k];
+  }
+  __syncwarp(gm);
+  if (!ok || !(cond <= sp.cond_max)) {
+    if (cnt >= M) {
+      *result = 2;   // FP64 decides
+      return;
+    }
+    for (int e = lane; e < len; e += G) st4(coef + e, make_float4(0, 0, 0, 0));
+    *result = 1;
+    *cond_out = INFINITY;
+    return;
+  }
+  // ---- solve: lane k of the group solves right-hand side k, and k + G where there
+  // are more than lanes (a warp issues one solve for all of its groups' lanes at
+  // once instead of NR in a row; lanes k >= NR repeat one), and the group reads the
+  // solutions back from shared memory, as pairs: right-hand sides (0, 1) and (2, 3)
+  // in 3D, (0, 1) and 2 for film
+  constexpr int NQ = (NR + G - 1) / G;   // solves per lane
+  // res[k M + r] (shared): solve for it and put the solution in its place
+  auto solve_all = [&](auto &&right) {
+    float x[NQ][M];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      float bb[M];
+      const int kq = G >= NR ? lane % NR : (lane + q * G < NR ? lane + q * G : NR - 1);
+#pragma unroll
+      for (int r = 0; r < M; ++r) bb[r] = right(kq, r);
+      chol_solve_s<M, float>(Ls, invd, bb, x[q]);
+    }
+    __syncwarp(gm);   // every lane has its right-hand sides before they are overwritten
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+      if (lane + q * G < NR) {
+#pragma unroll
+        for (int r = 0; r < M; ++r) sm[(lane + q * G) * M + r] = x[q][r];
+      }
+    __syncwarp(gm);
+  };
+  float2 l01[M], l2x[M];   // l2x.y: right-hand side 3, or film's correction of the Laplacian
+  {
+    solve_all([&](int k, int r) { return rhs<M, float>(k, r); });
+#pragma unroll
+    for (int r = 0; r < M; ++r) {
+      l01[r] = make_float2(sm[r], sm[M + r]);
+      l2x[r] = make_float2(sm[2 * M + r], M == 10 ? sm[(NR - 1) * M + r] : 0.0f);
+    }
+    __syncwarp(gm);
+  }
+  // calls body(e, q and w) for the lane's entries in pairs e and e + G (one loop
+  // for cached and uncached entries: the passes' code stays in the instruction
+  // cache)
+  auto for_pairs = [&](auto &&body) {
+#pragma unroll 1
+    for (int e = lane, k = 0; e < len; e += 2 * G, ++k) {
+      float2 q[3], w;
+      if (k < KP) {
+        const float4 *c = qw + 64 * k;
+        const float4 u = c[0], v = c[32];
+        q[0] = make_float2(u.x, u.y);
+        q[1] = make_float2(u.z, u.w);
+        q[2] = make_float2(v.x, v.y);
+        w = make_float2(v.z, v.w);
+      } else {   // beyond the cache: gathered again
+        float4 xs[2];
+        bool oks[2];
+        const int j2[2] = {col[e], e + G < len ? col[e + G] : -1};
+        gather(j2, 2, xs, oks);
+        locate(xs[0], xs[1], oks[0], oks[1], q[0], q[1], q[2], w);
+      }
+      body(e, q[0], q[1], q[2], w);
+    }
+  };
+  // sums p.lambda of the packed right-hand sides (p_0 = 1)
+  auto dots = [&](const float2 (&p)[M], float2 &s01, float2 &s2x) {
+    s01 = l01[0];
+    s2x = l2x[0];
+#pragma unroll
+    for (int r = 1; r < M; ++r) {
+      s01 = fma2(p[r], l01[r], s01);
+      s2x = fma2(p[r], l2x[r], s2x);
+    }
+  };
+  // The Laplacian's refinement correction is kept apart (lo) instead of
+  // being added into lambda: its solution has entries ~100x its coefficients on
+  // one-sided (free-surface, wall) rows, and rounding lambda + d to FP32 would put
+  // back an error A * (rounding of lambda) into the moment conditions, which the
+  // applied Laplacian sees divided by h.  Its coefficients are evaluated as
+  // w (p.lambda + p.lo).
+  float lo[M];
+#pragma unroll
+  for (int r = 0; r < M; ++r) lo[r] = 0.0f;
+  if constexpr (REFINE) {
+    // residual b - sum_j c_j p_j of the coefficients as they will be stored
+    float2 R01[M], R2x[M];
+#pragma unroll
+    for (int r = 0; r < M; ++r) R01[r] = R2x[r] = make_float2(0.0f, 0.0f);
+    for_pairs([&](int, float2 qa, float2 qb, float2 qc, float2 w) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        float2 p[M], s01, s2x;
+        basis2<M>(dup2(u ? qa.y : qa.x), dup2(u ? qb.y : qb.x), dup2(u ? qc.y : qc.x), p);
+        dots(p, s01, s2x);
+        const float2 ww = dup2(u ? w.y : w.x);
+        const float2 c01 = mul2(ww, s01), c2x = mul2(ww, s2x);
+        R01[0] = add2(R01[0], c01);
+        R2x[0] = add2(R2x[0], c2x);
+#pragma unroll
+        for (int r = 1; r < M; ++r) {
+          R01[r] = fma2(c01, p[r], R01[r]);
+          R2x[r] = fma2(c2x, p[r], R2x[r]);
+        }
+      }
+    });
+    float R[VR];
+#pragma unroll
+    for (int k = 0; k < VR; ++k) R[k] = 0.0f;
+#pragma unroll
+    for (int r = 0; r < M; ++r) {
+      R[r] = R01[r].x;
+      R[M + r] = R01[r].y;
+      R[2 * M + r] = R2x[r].x;
+      if (NR == 4) R[(NR - 1) * M + r] = R2x[r].y;
+    }
+    reduce_scatter<G, VR>(R);
+#pragma unroll
+    for (int k = 0; k < VR / G; ++k) sm[lane * (VR / G) + k] = R[k];
+    __syncwarp(gm);
+    {
+      // the corrections
+      solve_all([&](int k, int r) { return rhs<M, float>(k, r) - sm[k * M + r]; });
+#pragma unroll
+      for (int r = 0; r < M; ++r) {
+        l01[r].x += sm[r];
+        l01[r].y += sm[M + r];
+        if (NR == 4) l2x[r].x += sm[2 * M + r];
+        lo[r] = sm[KL * M + r];
+        if (NR == 3) l2x[r].y = lo[r];
+      }
+    }
+    __syncwarp(gm);
+  }
+  // ---- coefficients: w p.lambda_k (+ w p.lo for the Laplacian) with the
+  // operator's scale 1/h or 1/h^2 folded into w (the products are taken onto +0,
+  // so an entry of the other model gets +0 whatever the sign of its sum)
+  const float2 zero = make_float2(0.0f, 0.0f);
+  for_pairs([&](int e, float2 qa, float2 qb, float2 qc, float2 w) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      float2 p[M], s01, s2x;
+      basis2<M>(dup2(u ? qa.y : qa.x), dup2(u ? qb.y : qb.x), dup2(u ? qc.y : qc.x), p);
+      dots(p, s01, s2x);
+      const float wu = u ? w.y : w.x, wg = wu * hinv, wl = wu * h2inv;
+      float4 out;
+      if constexpr (M == 10) {
+        if constexpr (REFINE) {
+          float sl = lo[0];
+#pragma unroll
+          for (int r = 1; r < M; ++r) sl = fmaf(p[r].x, lo[r], sl);
+          s2x.y += sl;
+        }
+        const float2 g = fma2(dup2(wg), s01, zero), gl = fma2(make_float2(wg, wl), s2x, zero);
+        out = make_float4(g.x, g.y, gl.x, gl.y);
+      } else {
+        const float sl = s2x.x + s2x.y;   // (s2x.y = p.lo, zero without refinement)
+        const float2 gxy = fma2(make_float2(t1[0], t1[1]), dup2(s01.x),
+                                mul2(make_float2(t2[0], t2[1]), dup2(s01.y)));
+        const float gz = fmaf(s01.x, t1[2], s01.y * t2[2]);
+        const float2 g = fma2(dup2(wg), gxy, zero);
+        const float2 gl = fma2(make_float2(wg, wl), make_float2(gz, sl), zero);
+        out = make_float4(g.x, g.y, gl.x, gl.y);
+      }
+      if (u == 0 || e + G < len) st4(coef + e + u * G, out);
+    }
+  });
+  *result = 0;
+  *cond_out = cond;
+}
+
+// ------------------------------------------------------------ FP64 arithmetic
+// Process particle i in FP64 (TS storage) with a group of G lanes.  Returns
+// (through *result) 0 = written, 1 = deficient (zeros written).  wc: the lane's
+// cache of KC weights (KC = 0: none), 32 apart.
+template <typename TS, int M, int G, int KC = 0>
 __device__ void stencil_particle(int64_t i, const vec4_t<TS> *pos, const uint8_t *model,
                                  const vec4_t<TS> *frame, const long long *row_ptr,
-                                 const int32_t *col, vec4_t<TS> *coef, const StParams<C> &sp,
-                                 C *sm /* per-group scratch, >= pad_to(NR*M or NA, G) */,
-                                 int *result, float *cond_out, float4 *qw = nullptr) {
+                                 const int32_t *col, vec4_t<TS> *coef,
+                                 const StParams<double> &sp, double *sm, int *result,
+                                 float *cond_out, double *wc = nullptr) {
+  using C = double;
   constexpr int NA = Basis<M>::NA, NR = Basis<M>::NR;
-  constexpr int VA = pad_to(NA, G), VR = pad_to(NR * M, G);
   using V = vec4_t<TS>;
   const int lane = threadIdx.x & (G - 1);
   const unsigned gm = group_mask<G>();
@@ -73,8 +423,7 @@ __device__ void stencil_particle(int64_t i, const vec4_t<TS> *pos, const uint8_t
       w = oks[u] ? w : C(0);   // other model / past the row end: contributes exact zeros
       cnt += oks[u] ? 1 : 0;
       if constexpr (KC > 0) {
-        // keep (q, w) for the later passes: they rebuild p without a gather
-        if (kk + u < KC) qw[(kk + u) * G + lane] = make_float4(p[1], p[2], M == 10 ? p[3] : 0.f, w);
+        if (kk + u < KC) wc[(kk + u) * 32] = w;
       }
       add_moments<M, C, VM>(A, w, p);
     }
@@ -94,7 +443,8 @@ __device__ void stencil_particle(int64_t i, const vec4_t<TS> *pos, const uint8_t
 #pragma unroll
   for (int r = 0; r < M; ++r) tr += L[pk(r, r)];
   C invd[M], pmin, pmax;
-  const bool ok = (cnt >= M) && cholesky<M, C>(L, invd, sp.piv_tol_rel * tr, pmin, pmax);
+  const bool pd = cholesky<M, C>(L, invd, sp.piv_tol_rel * tr, pmin, pmax);
+  const bool ok = pd && cnt >= M;
   const C cond = (pmax / pmin) * (pmax / pmin);
   C *Ls = sm + StSmem<M, G>::SCR;
   if (lane == 0) {
@@ -102,23 +452,13 @@ __device__ void stencil_particle(int64_t i, const vec4_t<TS> *pos, const uint8_t
     for (int k = 0; k < NA; ++k) Ls[k] = L[k];
   }
   __syncwarp(gm);
-  if (!ok || (QUEUE && !(cond <= sp.cond_max))) {
-    // deficient (decided in this precision unless queued) -> zeros
-    if (QUEUE && cnt >= M) {
-      *result = 2;
-      return;
-    }
+  if (!ok) {
     for (long long e = b + lane; e < e1; e += G) st4(coef + e, mk4<TS>(0, 0, 0, 0));
     *result = 1;
     *cond_out = INFINITY;
     return;
   }
-  // entries of this lane, and how many of them the cache holds
-  const int nloc = e1 > b + lane ? (int)((e1 - b - lane + G - 1) / G) : 0;
-  const int ncache = KC > 0 ? min(nloc, KC) : 0;
-  // ---- solve: lane k of the group solves right-hand side k (a warp issues one
-  // solve for all of its groups' lanes at once instead of NR in a row; lanes
-  // k >= NR repeat one) and the group reads the solutions back from shared memory
+  // ---- solve: one right-hand side per lane, as in the FP32 rows
   static_assert(G >= NR, "one lane per right-hand side");
   const int kq = lane % NR;
   C lam[NR][M];
@@ -138,88 +478,10 @@ __device__ void stencil_particle(int64_t i, const vec4_t<TS> *pos, const uint8_t
       for (int r = 0; r < M; ++r) lam[k][r] = sm[k * M + r];
     __syncwarp(gm);
   }
-  // The Laplacian's refinement correction is kept apart (lamlo) instead of
-  // being added into lam: its solution has entries ~100x its coefficients on
-  // one-sided (free-surface, wall) rows, and rounding lam + d to FP32 would put
-  // back an error A * (rounding of lam) into the moment conditions, which the
-  // applied Laplacian sees divided by h.  Its coefficients are evaluated as
-  // w (p.lam + p.lamlo).
-  constexpr int KL = NR - 1;
-  C lamlo[M];
-#pragma unroll
-  for (int r = 0; r < M; ++r) lamlo[r] = C(0);
-  if constexpr (REFINE) {
-    // residual b - sum_j c_j p_j of the coefficients as they will be stored
-    C R[VR];
-#pragma unroll
-    for (int k = 0; k < VR; ++k) R[k] = C(0);
-    for (int q = 0; q < ncache; ++q) {
-      const float4 c4 = qw[q * G + lane];
-      C p[M];
-      basis_from_q<M, C>(c4, p);
-      const C w = c4.w;
-#pragma unroll
-      for (int k = 0; k < NR; ++k) {
-        C s = lam[k][0];   // p_0 = 1
-#pragma unroll
-        for (int r = 1; r < M; ++r) s = fma(p[r], lam[k][r], s);
-        const C c = w * s;
-        R[k * M] += c;
-#pragma unroll
-        for (int r = 1; r < M; ++r) R[k * M + r] = fma(c, p[r], R[k * M + r]);
-      }
-    }
-    for (long long e0 = b + lane + (long long)ncache * G; e0 < e1; e0 += kGatherR * G) {
-      V xs[kGatherR];
-      bool oks[kGatherR];
-      gather_row<kGatherR, G>(e0, e1, i, mi, col, pos, model, xs, oks);
-#pragma unroll
-      for (int u = 0; u < kGatherR; ++u) {
-        C p[M];
-        C w = basis_at<M, C>(xi, xs[u], hinv, t1, t2, sp, p);
-        w = oks[u] ? w : C(0);
-#pragma unroll
-        for (int k = 0; k < NR; ++k) {
-          C s = lam[k][0];   // p_0 = 1
-#pragma unroll
-          for (int r = 1; r < M; ++r) s = fma(p[r], lam[k][r], s);
-          const C c = w * s;
-          R[k * M] += c;
-#pragma unroll
-          for (int r = 1; r < M; ++r) R[k * M + r] = fma(c, p[r], R[k * M + r]);
-        }
-      }
-    }
-    reduce_scatter<G, VR>(R);
-#pragma unroll
-    for (int k = 0; k < VR / G; ++k) sm[lane * (VR / G) + k] = R[k];
-    __syncwarp(gm);
-    {
-      // the corrections, one right-hand side per lane as above
-      C rr[M], d[M];
-#pragma unroll
-      for (int r = 0; r < M; ++r) rr[r] = rhs<M, C>(kq, r) - sm[kq * M + r];
-      __syncwarp(gm);   // every lane has its residual before the corrections overwrite it
-      chol_solve_s<M, C>(Ls, invd, rr, d);
-      if (lane < NR) {
-#pragma unroll
-        for (int r = 0; r < M; ++r) sm[lane * M + r] = d[r];
-      }
-      __syncwarp(gm);
-#pragma unroll
-      for (int k = 0; k < NR; ++k)
-#pragma unroll
-        for (int r = 0; r < M; ++r) {
-          if (k == KL) lamlo[r] = sm[k * M + r];
-          else lam[k][r] += sm[k * M + r];
-        }
-    }
-    __syncwarp(gm);
-  }
   // ---- coefficients
   const C h2inv = hinv * hinv;
-  // the output record of one entry: w p.lambda_k (+ w p.lamlo for the
-  // Laplacian) with the operator's scale 1/h or 1/h^2 folded into w
+  // the output record of one entry: w p.lambda_k with the operator's scale 1/h or
+  // 1/h^2 folded into w
   auto coef_of = [&](const C (&p)[M], C w) -> vec4_t<TS> {
     const C wg = w * hinv, wl = w * h2inv;
     C s[NR];
@@ -228,12 +490,6 @@ __device__ void stencil_particle(int64_t i, const vec4_t<TS> *pos, const uint8_t
       C v = lam[k][0];   // p_0 = 1
 #pragma unroll
       for (int r = 1; r < M; ++r) v = fma(p[r], lam[k][r], v);
-      if (REFINE && k == KL) {
-        C sl = lamlo[0];
-#pragma unroll
-        for (int r = 1; r < M; ++r) sl = fma(p[r], lamlo[r], sl);
-        v += sl;
-      }
       s[k] = v;
     }
     if constexpr (M == 10) {
@@ -245,82 +501,93 @@ __device__ void stencil_particle(int64_t i, const vec4_t<TS> *pos, const uint8_t
       return mk4<TS>(TS(gx), TS(gy), TS(gz), TS(wl * s[2]));
     }
   };
-  auto write_coef = [&](long long e, const C (&p)[M], C w) { st4(coef + e, coef_of(p, w)); };
-  for (int q = 0; q < ncache; ++q) {
-    const float4 c4 = qw[q * G + lane];
-    C p[M];
-    basis_from_q<M, C>(c4, p);
-    if (c4.w != 0.f) write_coef(b + lane + (long long)q * G, p, C(c4.w));
-    else st4(coef + b + lane + (long long)q * G, mk4<TS>(0, 0, 0, 0));
-  }
-  for (long long e0 = b + lane + (long long)ncache * G; e0 < e1; e0 += kGatherU<M> * G) {
+  kk = 0;
+  for (long long e0 = b + lane; e0 < e1; e0 += kGatherU<M> * G, kk += kGatherU<M>) {
     V xs[kGatherU<M>];
     bool oks[kGatherU<M>];
     gather_row<kGatherU<M>, G>(e0, e1, i, mi, col, pos, model, xs, oks);
 #pragma unroll
     for (int u = 0; u < kGatherU<M>; ++u) {
-    const long long e = e0 + (long long)u * G;
-    if (e >= e1) break;
-    vec4_t<TS> out = mk4<TS>(0, 0, 0, 0);
-    if (oks[u]) {
-      C p[M];
-      const C w = basis_at<M, C>(xi, xs[u], hinv, t1, t2, sp, p);
-      out = coef_of(p, w);
-    }
-    st4(coef + e, out);
+      const long long e = e0 + (long long)u * G;
+      if (e >= e1) break;
+      vec4_t<TS> out = mk4<TS>(0, 0, 0, 0);
+      if (oks[u]) {
+        C p[M], w;
+        if (KC > 0 && kk + u < KC) {
+          basis_only<M, C>(xi, xs[u], hinv, t1, t2, p);
+          w = wc[(kk + u) * 32];
+        } else {
+          w = basis_at<M, C>(xi, xs[u], hinv, t1, t2, sp, p);
+        }
+        out = coef_of(p, w);
+      }
+      st4(coef + e, out);
     }
   }
   *result = 0;
   *cond_out = (float)cond;
 }
 
-// Main kernel: every particle of model (M == 10 ? 3D : 2D).
-template <typename TS, typename C, int M, int G, bool REFINE, bool QUEUE>
-__global__ void __launch_bounds__(kStThreads, sizeof(C) == 4 ? (M == 10 ? 4 : 6) : 1) k_stencil(
+// Main kernel: every particle of model (M == 10 ? 3D : 2D).  A warp looks at
+// `rounds` x 32 / G consecutive particles, and its groups share those of its
+// model out, so that a warp of the other model ends at once (a film alone spent
+// 57 us in the 3D kernel when every group tested its own particles one by one)
+// and mixed warps leave no group idle but in their last round.
+template <typename TS, typename C, int M, int G, bool REFINE>
+__global__ void __launch_bounds__(kBuildThreads, sizeof(C) == 4 ? (M == 10 ? 7 : 10) : 1) k_stencil(
     int64_t n, const vec4_t<TS> *pos, const uint8_t *model, const vec4_t<TS> *frame,
     const long long *row_ptr, const int32_t *col, vec4_t<TS> *coef, uint8_t *status,
-    float *cond, StParams<C> sp, DevStatus *st, int32_t *queue) {
-  constexpr int NA = Basis<M>::NA, NR = Basis<M>::NR;
-  constexpr int SMG = StSmem<M, G>::PER_GROUP;
-  constexpr int KC = StCache<C, M, G>::KC;
+    float *cond, StParams<C> sp, DevStatus *st, int32_t *queue, int rounds) {
+  constexpr int SMG = StSmem<M, G>::PER_GROUP, KC = StCache<C, M, G>::KC, ROWS = 32 / G;
   extern __shared__ __align__(16) unsigned char st_smem[];
-  float4 *qcache = reinterpret_cast<float4 *>(st_smem);
-  C *smem = reinterpret_cast<C *>(st_smem + StCache<C, M, G>::BYTES);
-  const int grp = threadIdx.x / G;
-  C *sm = smem + grp * SMG;
-  float4 *qw = qcache + grp * KC * G;
-  const int lane = threadIdx.x & (G - 1);
-  const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
-  const int64_t ngroups = ((int64_t)gridDim.x * blockDim.x) / G;
+  C *sm = reinterpret_cast<C *>(st_smem + StCache<C, M, G>::BYTES) + threadIdx.x / G * SMG;
+  const int lane = threadIdx.x & (G - 1), wl = threadIdx.x & 31;
   const uint8_t want = M == 10 ? MAFP_MODEL_3D : MAFP_MODEL_2D;
-  for (int64_t i = gid; i < n; i += ngroups) {
-    if (model[i] != want) continue;   // uniform within the group
-    int res;
-    float cd = 0.0f;
-    stencil_particle<TS, C, M, G, REFINE, QUEUE, KC>(i, pos, model, frame, row_ptr, col, coef,
-                                                     sp, sm, &res, &cd, qw);
-    if (lane == 0) {
-      if (res == 2) {
-        const int slot = atomicAdd(&st->fallback_count, 1);
-        queue[slot] = (int32_t)i;
+  const int64_t i0 = ((int64_t)blockIdx.x * (kBuildThreads / 32) + threadIdx.x / 32) * rounds * ROWS;
+  unsigned todo = __ballot_sync(0xffffffffu, wl < rounds * ROWS && i0 + wl < n &&
+                                                 model[i0 + wl] == want);
+  while (todo) {
+    // group g takes the g-th of the next ROWS particles
+    unsigned mine = todo;
+    for (int k = 0; k < wl / G; ++k) mine &= mine - 1;
+#pragma unroll
+    for (int k = 0; k < ROWS; ++k) todo &= todo - 1;
+    if (mine) {
+      const int64_t i = i0 + __ffs(mine) - 1;
+      int res;
+      float cd = 0.0f;
+      if constexpr (sizeof(C) == 4) {
+        float4 *qw = reinterpret_cast<float4 *>(st_smem) + threadIdx.x / 32 * KC * 32 + wl;
+        stencil_row32<M, G, REFINE>(i, pos, model, frame, row_ptr, col, coef, sp, sm, &res, &cd,
+                                    qw);
       } else {
-        status[i] = res == 0 ? MAFP_STENCIL_OK : MAFP_STENCIL_DEFICIENT;
-        cond[i] = res == 0 ? cd : INFINITY;
-        if (res == 1) inc_ll(&st->n_deficient);
+        double *wc = reinterpret_cast<double *>(st_smem) + threadIdx.x / 32 * KC * 32 + wl;
+        stencil_particle<TS, M, G, KC>(i, pos, model, frame, row_ptr, col, coef, sp, sm, &res, &cd,
+                                       wc);
+      }
+      if (lane == 0) {
+        if (res == 2) {
+          queue[atomicAdd(&st->fallback_count, 1)] = (int32_t)i;
+        } else {
+          status[i] = res == 0 ? MAFP_STENCIL_OK : MAFP_STENCIL_DEFICIENT;
+          cond[i] = res == 0 ? cd : INFINITY;
+          if (res == 1) inc_ll(&st->n_deficient);
+        }
       }
     }
+    __syncwarp();
   }
 }
 
 // FP64 redo of the queued particles of one model (FP32 storage).
 template <int M, int G>
-__global__ void __launch_bounds__(kStThreads) k_stencil_redo(
+__global__ void __launch_bounds__(kBuildThreads) k_stencil_redo(
     const float4 *pos, const uint8_t *model, const float4 *frame, const long long *row_ptr,
     const int32_t *col, float4 *coef, uint8_t *status, float *cond, StParams<double> sp,
     DevStatus *st, const int32_t *queue) {
   constexpr int NA = Basis<M>::NA, NR = Basis<M>::NR;
   constexpr int SMG = StSmem<M, G>::PER_GROUP;
-  __shared__ double smem[(kStThreads / G) * SMG];
+  __shared__ double smem[(kBuildThreads / G) * SMG];
   const int grp = threadIdx.x / G;
   double *sm = smem + grp * SMG;
   const int lane = threadIdx.x & (G - 1);
@@ -333,8 +600,7 @@ __global__ void __launch_bounds__(kStThreads) k_stencil_redo(
     if (model[i] != want) continue;
     int res;
     float cd = 0.0f;
-    stencil_particle<float, double, M, G, false, false>(i, pos, model, frame, row_ptr, col, coef,
-                                                         sp, sm, &res, &cd);
+    stencil_particle<float, M, G>(i, pos, model, frame, row_ptr, col, coef, sp, sm, &res, &cd);
     if (lane == 0) {
       status[i] = res == 0 ? MAFP_STENCIL_FP64 : MAFP_STENCIL_DEFICIENT;
       cond[i] = res == 0 ? cd : INFINITY;
@@ -345,7 +611,7 @@ __global__ void __launch_bounds__(kStThreads) k_stencil_redo(
 }
 
 
-template <typename TS, typename C, int M, int G, bool REFINE, bool QUEUE>
+template <typename TS, typename C, int M, int G, bool REFINE>
 static void launch_stencil(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void *pos_h,
                            const uint8_t *model, const void *frame, const long long *rp,
                            const int32_t *col, void *coef, uint8_t *status, float *cond,
@@ -353,34 +619,48 @@ static void launch_stencil(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void 
   using V = vec4_t<TS>;
   static const KernelName name("k_stencil<%s,M=%d,G=%d,%s>", sizeof(TS) == 4 ? "f32" : "f64",
                                M, G, REFINE ? "refined" : "plain");
-  const int blocks = grid_for(n * G, kStThreads, sm_count() * 64);
+  // rounds of rows per warp: one while that leaves the GPU's warps without work
+  const int rounds = n > kStManyRows ? 4 : 1;
+  static_assert(G >= 4, "a warp looks at 32 particles at most");
+  const int blocks = (int)((n + (int64_t)rounds * kBuildThreads / G - 1) / (rounds * kBuildThreads / G));
   constexpr int smem = StCache<C, M, G>::SMEM;
   // the dynamic shared-memory limit is a per-device setting of the function
   static unsigned long long attr_devices = 0;
   if (smem > 48 * 1024 && first_on_device(&attr_devices, ctx->device))
-    cudaFuncSetAttribute(k_stencil<TS, C, M, G, REFINE, QUEUE>,
+    cudaFuncSetAttribute(k_stencil<TS, C, M, G, REFINE>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   MAFP_TIMED(ctx, s, name.s,
-             k_stencil<TS, C, M, G, REFINE, QUEUE><<<blocks, kStThreads, smem, s>>>(
+             k_stencil<TS, C, M, G, REFINE><<<blocks, kBuildThreads, smem, s>>>(
                  n, (const V *)pos_h, model, (const V *)frame, rp, col, (V *)coef, status, cond,
-                 sp, ctx->d_status, ctx->fallback));
+                 sp, ctx->d_status, ctx->fallback, rounds));
 }
 
-// Group size G chosen at run time (tuning), instantiated for 8/16/32 (3D) and 4/8/16 (2D).
-template <typename TS, typename C, bool REFINE, bool QUEUE>
+// Lanes per particle.  3D: 8 whatever the context's stencil3d_group asks for: more
+// lanes repeat the factorisation and leave part of a row's last gather empty (440k
+// rows: 951 us, with 32 lanes 2136).  Clouds whose rows do not fill the GPU take
+// 32 (5650 particles: 21 us against 25).  Film, FP32: the context's
+// stencil2d_group, which also sets the order of the sums: the Laplacians of a
+// curved film are small differences, and gradients taken through them show every
+// change of rounding.  Film, FP64: 4 lanes, for the factorisation (697 us with 8,
+// 476 with 4 on the 60k jet cloud).
+template <typename TS, typename C, bool REFINE>
 static int dispatch_stencils(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void *pos_h,
                              const uint8_t *model, const void *frame, const long long *rp,
                              const int32_t *col, void *coef, uint8_t *status, float *cond,
                              const StParams<C> &sp) {
-  switch (ctx->tune.stencil3d_group) {
-    case 8: launch_stencil<TS, C, 10, 8, REFINE, QUEUE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
-    case 16: launch_stencil<TS, C, 10, 16, REFINE, QUEUE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
-    default: launch_stencil<TS, C, 10, 32, REFINE, QUEUE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
-  }
-  switch (ctx->tune.stencil2d_group) {
-    case 4: launch_stencil<TS, C, 6, 4, REFINE, QUEUE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
-    case 16: launch_stencil<TS, C, 6, 16, REFINE, QUEUE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
-    default: launch_stencil<TS, C, 6, 8, REFINE, QUEUE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
+  if (n <= kStFewRows)
+    launch_stencil<TS, C, 10, 32, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp);
+  else
+    launch_stencil<TS, C, 10, 8, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp);
+  switch (sizeof(C) == 8 ? (n <= kStFewRows ? 8 : 4) : ctx->tune.stencil2d_group) {
+    case 4: launch_stencil<TS, C, 6, 4, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
+    case 16:
+      if constexpr (sizeof(C) == 4) {
+        launch_stencil<TS, C, 6, 16, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp);
+        break;
+      }
+      [[fallthrough]];
+    default: launch_stencil<TS, C, 6, 8, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
   }
   MAFP_LAUNCH_CHECK(ctx);
   return MAFP_OK;
@@ -393,26 +673,26 @@ int build_stencils(mafp_ctx *ctx, int64_t n, int32_t dtype, const void *pos_h,
   const int sms = sm_count();
   if (dtype == MAFP_F64) {
     const StParams<double> sp = make_params<double>(ctx->prm, 1e-12);
-    return dispatch_stencils<double, double, false, false>(ctx, s, n, pos_h, model, frame, rp,
+    return dispatch_stencils<double, double, false>(ctx, s, n, pos_h, model, frame, rp,
                                                           col, coef, status, cond, sp);
   }
   const StParams<float> sp = make_params<float>(ctx->prm, 1e-6);
   const StParams<double> sp64 = make_params<double>(ctx->prm, 1e-12);
   MAFP_TIMED(ctx, s, "k_reset_queue", k_reset_queue<<<1, 1, 0, s>>>(ctx->d_status));
   int rc = dtype == MAFP_F32_PLAIN
-               ? dispatch_stencils<float, float, false, true>(ctx, s, n, pos_h, model, frame, rp,
+               ? dispatch_stencils<float, float, false>(ctx, s, n, pos_h, model, frame, rp,
                                                              col, coef, status, cond, sp)
-               : dispatch_stencils<float, float, true, true>(ctx, s, n, pos_h, model, frame, rp,
+               : dispatch_stencils<float, float, true>(ctx, s, n, pos_h, model, frame, rp,
                                                             col, coef, status, cond, sp);
   if (rc) return rc;
   // FP64 redo: small groups keep the per-particle factorisation, repeated in
   // every lane of a group, from dominating the slow FP64 pipe
   MAFP_TIMED(ctx, s, "k_stencil_redo<10,4>",
-             k_stencil_redo<10, 4><<<sms * 32, kStThreads, 0, s>>>(
+             k_stencil_redo<10, 4><<<sms * 64, kBuildThreads, 0, s>>>(
       (const float4 *)pos_h, model, (const float4 *)frame, rp, col, (float4 *)coef, status, cond,
       sp64, ctx->d_status, ctx->fallback));
   MAFP_TIMED(ctx, s, "k_stencil_redo<6,4>",
-             k_stencil_redo<6, 4><<<sms * 32, kStThreads, 0, s>>>(
+             k_stencil_redo<6, 4><<<sms * 64, kBuildThreads, 0, s>>>(
       (const float4 *)pos_h, model, (const float4 *)frame, rp, col, (float4 *)coef, status, cond,
       sp64, ctx->d_status, ctx->fallback));
   MAFP_LAUNCH_CHECK(ctx);

@@ -186,7 +186,8 @@ __device__ int grad_particle(int64_t i, const vec4_t<TS> *pos, const uint8_t *mo
 #pragma unroll
   for (int r = 0; r < M; ++r) tr += L[pk(r, r)];
   C invd[M], pmin, pmax;
-  const bool ok = (cnt >= M) && cholesky<M, C>(L, invd, sp.piv_tol_rel * tr, pmin, pmax);
+  const bool pd = cholesky<M, C>(L, invd, sp.piv_tol_rel * tr, pmin, pmax);
+  const bool ok = pd && cnt >= M;
   const C cond = (pmax / pmin) * (pmax / pmin);
   if (!ok || (QUEUE && !(cond <= sp.cond_max))) return (QUEUE && cnt >= M) ? 2 : 1;
   C *Ls = sm + StSmem<M, G>::SCR;

@@ -3,6 +3,8 @@
 #pragma once
 #include <math.h>
 
+#include <type_traits>
+
 #include "internal.cuh"
 
 namespace mafp {
@@ -153,17 +155,19 @@ __device__ __forceinline__ C basis_at(const V &xi, const V &xj, C hinv, const C 
   return w;
 }
 
-// The same monomials rebuilt from a cached (q, w): q = (x_j - x_i) / h_i in 3D,
-// (xi, eta) in 2D, with the products taken exactly as basis_at takes them.
-template <int M, typename C>
-__device__ __forceinline__ void basis_from_q(const float4 &c, C (&p)[M]) {
+// The monomials alone (the weight is cached).
+template <int M, typename C, typename V>
+__device__ __forceinline__ void basis_only(const V &xi, const V &xj, C hinv, const C (&t1)[3],
+                                           const C (&t2)[3], C (&p)[M]) {
+  const C dx = C(xj.x) - C(xi.x), dy = C(xj.y) - C(xi.y), dz = C(xj.z) - C(xi.z);
   if constexpr (M == 10) {
-    const C qx = c.x, qy = c.y, qz = c.z;
+    const C qx = dx * hinv, qy = dy * hinv, qz = dz * hinv;
     p[0] = C(1); p[1] = qx; p[2] = qy; p[3] = qz;
     p[4] = qx * qx; p[5] = qy * qy; p[6] = qz * qz;
     p[7] = qx * qy; p[8] = qx * qz; p[9] = qy * qz;
   } else {
-    const C xi_ = c.x, et_ = c.y;
+    const C xi_ = (dx * t1[0] + dy * t1[1] + dz * t1[2]) * hinv;
+    const C et_ = (dx * t2[0] + dy * t2[1] + dz * t2[2]) * hinv;
     p[0] = C(1); p[1] = xi_; p[2] = et_;
     p[3] = xi_ * xi_; p[4] = xi_ * et_; p[5] = et_ * et_;
   }
@@ -181,77 +185,86 @@ __device__ __forceinline__ C rhs(int k, int r) {
   }
 }
 
+// f(integral_constant<int, I>) for I = B .. E - 1: loops whose indices the compiler
+// has to know.
+template <int B, int E, typename F>
+__device__ __forceinline__ void static_for(F &&f) {
+  if constexpr (B < E) {
+    f(std::integral_constant<int, B>{});
+    static_for<B + 1, E>(f);
+  }
+}
+
 // In-register Cholesky of the packed matrix L (lower), returns false when a
-// pivot is <= tol.  invd gets 1/L_kk; pmin / pmax the extreme pivots.
-template <int M, typename C>
+// pivot is <= tol.  invd gets 1/L_kk; pmin / pmax the extreme pivots.  (Written
+// with loops under "#pragma unroll" the 6 x 6 case kept run-time indices, a
+// compare and a select per candidate register: 710 instructions per warp instead
+// of 200, a fifth of the film build.)  NEWTON (FP32): reciprocal root and one Newton
+// step, eight operations in every lane of the group against about twenty-five of
+// a square root and a division; for the build, whose refinement corrects what
+// the last bit of a pivot changes -- the adjoint, unrefined, keeps the exact ones
+// (rounded differently its film gradients move by as much as their own error,
+// 2e-5).
+template <int M, typename C, bool NEWTON = false>
 __device__ __forceinline__ bool cholesky(C (&L)[Basis<M>::NA], C (&invd)[M], C tol, C &pmin,
                                          C &pmax) {
   pmin = C(INFINITY);
   pmax = C(0);
   bool ok = true;
-#pragma unroll
-  for (int k = 0; k < M; ++k) {
+  static_for<0, M>([&](auto kc) {
+    constexpr int k = kc;
     C d = L[pk(k, k)];
-#pragma unroll
-    for (int l = 0; l < k; ++l) d -= L[pk(k, l)] * L[pk(k, l)];
+    static_for<0, k>([&](auto lc) {
+      constexpr int l = lc;
+      d -= L[pk(k, l)] * L[pk(k, l)];
+    });
     ok = ok && (d > tol);
-    const C lkk = sqrt(d > tol ? d : C(1));
+    const C dd = d > tol ? d : C(1);
+    C lkk;
+    if constexpr (NEWTON) {
+      C y = rsqrtf(dd);
+      y = fmaf(C(0.5) * y, fmaf(-dd * y, y, C(1)), y);
+      invd[k] = y;
+      lkk = dd * y;
+    } else {
+      lkk = sqrt(dd);
+      invd[k] = C(1) / lkk;
+    }
     L[pk(k, k)] = lkk;
-    invd[k] = C(1) / lkk;
     pmin = lkk < pmin ? lkk : pmin;
     pmax = lkk > pmax ? lkk : pmax;
-#pragma unroll
-    for (int r = k + 1; r < M; ++r) {
+    static_for<k + 1, M>([&](auto rc) {
+      constexpr int r = rc;
       C s = L[pk(r, k)];
-#pragma unroll
-      for (int l = 0; l < k; ++l) s -= L[pk(r, l)] * L[pk(k, l)];
+      static_for<0, k>([&](auto lc) {
+        constexpr int l = lc;
+        s -= L[pk(r, l)] * L[pk(k, l)];
+      });
       L[pk(r, k)] = s * invd[k];
-    }
-  }
+    });
+  });
   return ok;
 }
 
-template <int M, typename C>
-__device__ __forceinline__ void chol_solve(const C (&L)[Basis<M>::NA], const C (&invd)[M],
-                                           const C (&b)[M], C (&x)[M]) {
-  C y[M];
-#pragma unroll
-  for (int r = 0; r < M; ++r) {
-    C s = b[r];
-#pragma unroll
-    for (int l = 0; l < r; ++l) s -= L[pk(r, l)] * y[l];
-    y[r] = s * invd[r];
-  }
-#pragma unroll
-  for (int r = M - 1; r >= 0; --r) {
-    C s = y[r];
-#pragma unroll
-    for (int l = r + 1; l < M; ++l) s -= L[pk(l, r)] * x[l];
-    x[r] = s * invd[r];
-  }
-}
-
-// Same solve with the factor read from shared memory (every lane of the group
+// Solve with the factor read from shared memory (every lane of the group
 // reads the same address: a broadcast), which keeps the 55 entries of L out
 // of the registers during the refinement pass.
 template <int M, typename C>
 __device__ __forceinline__ void chol_solve_s(const C *L, const C (&invd)[M], const C (&b)[M],
                                              C (&x)[M]) {
   C y[M];
-#pragma unroll
-  for (int r = 0; r < M; ++r) {
+  static_for<0, M>([&](auto rc) {
+    constexpr int r = rc;
     C s = b[r];
-#pragma unroll
-    for (int l = 0; l < r; ++l) s -= L[pk(r, l)] * y[l];
+    static_for<0, r>([&](auto lc) { s -= L[pk(r, lc)] * y[lc]; });
     y[r] = s * invd[r];
-  }
-#pragma unroll
-  for (int r = M - 1; r >= 0; --r) {
+  });
+  static_for<0, M>([&](auto qc) {
+    constexpr int r = M - 1 - qc;
     C s = y[r];
-#pragma unroll
-    for (int l = r + 1; l < M; ++l) s -= L[pk(l, r)] * x[l];
+    static_for<r + 1, M>([&](auto lc) { s -= L[pk(lc, r)] * x[lc]; });
     x[r] = s * invd[r];
-  }
+  });
 }
 
 // U neighbours of one lane (entries e0, e0 + G, ..., e0 + (U-1) G of the row),
