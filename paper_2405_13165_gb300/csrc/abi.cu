@@ -165,7 +165,7 @@ int mafp_create(mafp_ctx **out, const mafp_params *params, int64_t cap_particles
       {(void **)&ctx->one_cloud, sizeof(long long) * 2},
       {(void **)&ctx->cloud_partial, sizeof(double) * (kMaxClouds + 16384) * 8},
       {(void **)&ctx->remap_i64, sizeof(int64_t) * i64_len},
-      {(void **)&ctx->remap_i32, sizeof(int32_t) * 3 * cap},
+      {(void **)&ctx->remap_i32, sizeof(int32_t) * 5 * cap},
   };
   for (auto &a : allocs) {
     cudaError_t e = cudaMalloc(a.p, a.bytes);

@@ -79,7 +79,7 @@ struct mafp_ctx {
   long long *one_cloud;      // [2] offsets of the single-cloud case
   double *cloud_partial;     // [(kMaxClouds + 16384) * 8] bounding-box partials
   int64_t *remap_i64;       // [3 * cap + 8]
-  int32_t *remap_i32;       // [2 * cap]
+  int32_t *remap_i32;       // [5 * cap]
   char err[512];
   // kernel-level CUDA-event timing (off unless mafp_profile(ctx, 1))
   int prof_on;
