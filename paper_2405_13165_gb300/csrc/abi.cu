@@ -162,7 +162,6 @@ int mafp_create(mafp_ctx **out, const mafp_params *params, int64_t cap_particles
       {(void **)&ctx->d_grids, sizeof(GridDev) * kMaxClouds},
       {(void **)&ctx->cell_base, sizeof(long long) * (kMaxClouds + 1)},
       {(void **)&ctx->cloud_id, sizeof(int32_t) * cap},
-      {(void **)&ctx->one_cloud, sizeof(long long) * 2},
       {(void **)&ctx->cloud_partial, sizeof(double) * (kMaxClouds + 16384) * 8},
       {(void **)&ctx->remap_i64, sizeof(int64_t) * i64_len},
       {(void **)&ctx->remap_i32, sizeof(int32_t) * 5 * cap},
@@ -196,7 +195,7 @@ int mafp_destroy(mafp_ctx *ctx) {
                   ctx->nbr_mask,  ctx->cell_table, ctx->overflow,
                   ctx->fallback, ctx->d_status,  ctx->d_grid,
                   ctx->remap_i64, ctx->remap_i32, ctx->d_grids,   ctx->cell_base,
-                  ctx->cloud_id,  ctx->one_cloud, ctx->cloud_partial};
+                  ctx->cloud_id,  ctx->cloud_partial};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (ctx->prof_ev) {

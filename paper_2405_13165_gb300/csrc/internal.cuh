@@ -76,7 +76,6 @@ struct mafp_ctx {
   mafp::GridDev *d_grids;    // [kMaxClouds] one grid per cloud
   long long *cell_base;      // [kMaxClouds + 1] first global cell of each cloud
   int32_t *cloud_id;         // [cap] cloud of every particle
-  long long *one_cloud;      // [2] offsets of the single-cloud case
   double *cloud_partial;     // [(kMaxClouds + 16384) * 8] bounding-box partials
   int64_t *remap_i64;       // [3 * cap + 8]
   int32_t *remap_i32;       // [5 * cap]
@@ -254,8 +253,9 @@ inline void prof_end(mafp_ctx *ctx, cudaStream_t s, const char *name) {
     prof_end(ctx, s, name);           \
   } while (0)
 
-// Device-wide exclusive scan of int32 values into int64 prefix (out[n] = total).
+// Device-wide exclusive scan of int32 values into int64 prefix (out[n] = total);
+// with `wanted` (device), nothing is done when *wanted is 0.
 int scan_i32_to_i64(mafp_ctx *ctx, const int32_t *in, long long *out, int64_t n,
-                    cudaStream_t s);
+                    cudaStream_t s, const int32_t *wanted = nullptr);
 
 }  // namespace mafp

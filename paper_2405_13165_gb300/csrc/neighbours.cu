@@ -26,9 +26,9 @@ struct CloudGrids {
   const GridDev *all;        // ok flag and total cell count
 };
 
-__global__ void k_set_one_cloud(long long *off, int64_t n) {
-  off[0] = 0;
-  off[1] = n;
+// First particle of cloud b (off == nullptr: one cloud of n particles).
+__device__ __forceinline__ long long cloud_begin(const long long *off, int b, int64_t n) {
+  return off ? off[b] : (b == 0 ? 0 : (long long)n);
 }
 
 // Block (b, part) reduces part `part` of cloud b: min / max of x, y, z, max h,
@@ -47,8 +47,8 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_bbox(const vec4_t<T> *pos
                                                             int32_t *cloud_id) {
   const int b = blockIdx.x / parts, part = blockIdx.x % parts;
   // offsets are checked in k_cloud_grid; clamping keeps every access in [0, n)
-  const long long lo = max(0LL, min(off[b], (long long)n));
-  const long long hi = max(lo, min(off[b + 1], (long long)n));
+  const long long lo = max(0LL, min(cloud_begin(off, b, n), (long long)n));
+  const long long hi = max(lo, min(cloud_begin(off, b + 1, n), (long long)n));
   const T inf = T(INFINITY);
   T v[7] = {inf, inf, inf, -inf, -inf, -inf, T(0)};
   int bad = 0;
@@ -97,30 +97,32 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_bbox(const vec4_t<T> *pos
   }
 }
 
-// One warp per cloud folds the cloud's `parts` partials (lanes over parts,
-// then shuffles) and leaves the cloud's box in its first partial slot.
-__global__ void __launch_bounds__(kBoxThreads) k_cloud_fold(double *partial, int nb, int parts) {
-  const int lane = threadIdx.x & 31;
-  const int b = blockIdx.x * (kBoxThreads / 32) + (threadIdx.x >> 5);
-  if (b >= nb) return;
-  double v[8] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY, 0.0, 0.0};
-  double *pb = partial + (long long)b * parts * 8;
-  for (int q = lane; q < parts; q += 32)
-    for (int k = 0; k < 8; ++k) {
-      const double a = pb[q * 8 + k];
-      v[k] = k < 3 ? fmin(v[k], a) : (k < 7 ? fmax(v[k], a) : v[k] + a);
-    }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) v[k] = fmin(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
-#pragma unroll
-    for (int k = 3; k < 7; ++k) v[k] = fmax(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
-    v[7] += __shfl_xor_sync(0xffffffffu, v[7], o);
+// One block folds a cloud's `parts` partials and leaves the cloud's box in its
+// first partial slot.  Thread t takes value t & 7 of partials t >> 3, + 32, ...: a
+// warp reads 256 consecutive bytes, up to eight reads in flight.  (A warp per
+// cloud with a lane per partial took 22 us for 1024 partials, one latency after
+// another.)  Every thread of a block of 256 has to call it.
+__device__ __forceinline__ void fold_cloud(double *pb, int parts) {
+  __shared__ double red[8][8];
+  const int k = threadIdx.x & 7;
+  const double none = k < 3 ? INFINITY : (k < 6 ? -INFINITY : 0.0);
+  auto join = [&](double x, double y) { return k < 3 ? fmin(x, y) : (k < 7 ? fmax(x, y) : x + y); };
+  double v = none;
+#pragma unroll 8
+  for (int q = threadIdx.x >> 3; q < parts; q += kBoxThreads / 8) v = join(v, pb[q * 8 + k]);
+  v = join(v, __shfl_xor_sync(0xffffffffu, v, 8));
+  v = join(v, __shfl_xor_sync(0xffffffffu, v, 16));
+  if ((threadIdx.x & 31) < 8) red[threadIdx.x >> 5][k] = v;
+  __syncthreads();   // (also: every partial is read before the first is overwritten)
+  if (threadIdx.x < 8) {
+    for (int w = 1; w < kBoxThreads / 32; ++w) v = join(v, red[w][k]);
+    pb[k] = v;
   }
-  __syncwarp();
-  if (lane == 0)
-    for (int k = 0; k < 8; ++k) pb[k] = v[k];
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(kBoxThreads) k_cloud_fold(double *partial, int parts) {
+  fold_cloud(partial + (long long)blockIdx.x * parts * 8, parts);
 }
 
 // Cells of cloud b at edge c (>= max h of the cloud); 0 for an empty cloud.
@@ -138,7 +140,8 @@ __device__ double cloud_cells(const double v[8], double c, int dim[3]) {
   return cells;
 }
 
-// One block: per-cloud grids from the folded boxes, the global cell numbering
+// One block: the box of a single cloud (several are folded before), per-cloud
+// grids from the folded boxes, the global cell numbering
 // (exclusive scan of the clouds' cell counts) and the all-clouds flag.  The cell
 // edge of every cloud starts strictly above its max h times edge_factor >= 1
 // (so S_i lies in the 27 cells around i's cell) and grows uniformly when the
@@ -156,16 +159,18 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_grid(double *partial,
   if (threadIdx.x == 0) {
     s_nonfinite = 0.0;
     s_scale = 1.0;
-    s_bad = (off[0] != 0 || off[nb] != n) ? 1 : 0;
+    s_bad = (cloud_begin(off, 0, n) != 0 || cloud_begin(off, nb, n) != n) ? 1 : 0;
   }
+  if (nb == 1) fold_cloud(partial, parts);
   __syncthreads();
   for (int b = threadIdx.x; b < nb; b += blockDim.x)
-    if (off[b + 1] < off[b]) s_bad = 1;
+    if (cloud_begin(off, b + 1, n) < cloud_begin(off, b, n)) s_bad = 1;
   __syncthreads();
   if (s_bad) {
     // the offsets do not split [0, n) into consecutive ranges
     if (threadIdx.x == 0) {
       all->ok = 0;
+      st->cells_identity = st->not_identity ? 0 : 1;
       set_error(st, MAFP_EINVAL, -1);
     }
     return;
@@ -178,6 +183,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_grid(double *partial,
   if (s_nonfinite > 0.0) {
     if (threadIdx.x == 0) {
       all->ok = 0;
+      st->cells_identity = st->not_identity ? 0 : 1;
       st->n_nonfinite += (long long)s_nonfinite;
       set_error(st, MAFP_ENONFINITE, (long long)s_nonfinite);
     }
@@ -240,43 +246,8 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_grid(double *partial,
     if (acc > cap_cells) set_error(st, MAFP_ECAPACITY, cap_cells);
     st->ncells = acc;
     st->cell_size = grids[0].c;
-    st->not_identity = 0;
-  }
-}
-
-template <typename T>
-__global__ void k_hash(const vec4_t<T> *pos, int64_t n, const int32_t *cloud_id, CloudGrids cg,
-                       uint32_t *keys, int32_t *vals) {
-  if (!cg.all->ok) return;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int b = cloud_id[i];
-    const GridDev &g = cg.grids[b];
-    vec4_t<T> p = ld4(pos + i);
-    double q[3] = {(double)p.x, (double)p.y, (double)p.z};
-    long long c[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      long long v = (long long)floor((q[a] - g.lo[a]) * g.inv_c);
-      v = v < 0 ? 0 : (v >= g.dim[a] ? g.dim[a] - 1 : v);
-      c[a] = v;
-    }
-    keys[i] = (uint32_t)(cg.cell_base[b] + (c[2] * g.dim[1] + c[1]) * g.dim[0] + c[0]);
-    vals[i] = (int32_t)i;
-  }
-}
-
-__global__ void k_clear_cells(const GridDev *g, int32_t *cell_start, int32_t *cell_end,
-                              int32_t *n_ucell) {
-  if (!g->ok) return;
-  const long long nc = g->ncells;
-  // cell counts, overflow items, the work tickets and the mask pool's counter
-  if (blockIdx.x == 0 && threadIdx.x == 0)
-    for (int k = 0; k < 8; ++k) n_ucell[k] = 0;
-  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < nc;
-       k += (long long)gridDim.x * blockDim.x) {
-    cell_start[k] = INT_MAX;
-    cell_end[k] = 0;
+    st->not_identity = 0;     // k_hash clears / sets them when the keys are out of order
+    st->cells_identity = 1;
   }
 }
 
@@ -285,10 +256,87 @@ constexpr int kRadixThreads = 256;
 constexpr int kRadixItems = 8;
 constexpr int kRadixTile = kRadixThreads * kRadixItems;
 
+template <typename T>
+__device__ __forceinline__ uint32_t cell_key(const vec4_t<T> &p, int b, const CloudGrids &cg) {
+  const GridDev &g = cg.grids[b];
+  const double q[3] = {(double)p.x, (double)p.y, (double)p.z};
+  uint32_t c[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const double v = floor((q[a] - g.lo[a]) * g.inv_c), top = (double)(g.dim[a] - 1);
+    c[a] = (uint32_t)(v < 0.0 ? 0.0 : (v > top ? top : v));
+  }
+  return (uint32_t)cg.cell_base[b] +
+         (c[2] * (uint32_t)g.dim[1] + c[1]) * (uint32_t)g.dim[0] + c[0];
+}
+
+// One block per radix tile: the particles' cell keys, the tile's histogram of the
+// first digit, and whether a key is below the one before it.  Clouds that are in
+// cell order already (a time loop keeps them so) show it here, and the sort's
+// passes, their scans and the gather of the positions are left out: 165 of the
+// 215 us before the lists on the 1M jet cloud.  All blocks together also clear the
+// cells and the work counters.
+template <typename T>
+__global__ void __launch_bounds__(kRadixThreads) k_hash(const vec4_t<T> *pos, int64_t n,
+                                                        const int32_t *cloud_id, CloudGrids cg,
+                                                        uint32_t *keys, int32_t *vals,
+                                                        int32_t *hist, int tiles,
+                                                        int32_t *cell_start, int32_t *cell_end,
+                                                        int32_t *n_ucell, DevStatus *st) {
+  __shared__ int32_t cnt[256];
+  __shared__ uint32_t last[kRadixItems + 1][kRadixThreads / 32];
+  if (!cg.all->ok) return;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  cnt[tid] = 0;
+  const int64_t base = (int64_t)blockIdx.x * kRadixTile;
+  uint32_t key[kRadixItems];
+#pragma unroll
+  for (int c = 0; c < kRadixItems; ++c) {
+    const int64_t i = base + c * kRadixThreads + tid;
+    key[c] = 0xffffffffu;
+    if (i < n) {
+      key[c] = cell_key<T>(ld4(pos + i), cg.nb > 1 ? cloud_id[i] : 0, cg);
+      keys[i] = key[c];
+      vals[i] = (int32_t)i;
+    }
+    if (lane == 31) last[c][w] = key[c];
+  }
+  // the key before the tile's first one
+  if (tid == 0)
+    last[kRadixItems][0] =
+        base > 0 ? cell_key<T>(ld4(pos + base - 1), cg.nb > 1 ? cloud_id[base - 1] : 0, cg) : 0u;
+  __syncthreads();
+  bool out_of_order = false;
+#pragma unroll
+  for (int c = 0; c < kRadixItems; ++c) {
+    uint32_t before = __shfl_up_sync(0xffffffffu, key[c], 1);
+    if (lane == 0)
+      before = w > 0 ? last[c][w - 1]
+                     : (c > 0 ? last[c - 1][kRadixThreads / 32 - 1] : last[kRadixItems][0]);
+    out_of_order |= key[c] < before;
+    if (base + c * kRadixThreads + tid < n) atomicAdd(&cnt[key[c] & 255u], 1);
+  }
+  if (__syncthreads_or(out_of_order) && tid == 0) {
+    st->not_identity = 1;
+    st->cells_identity = 0;
+  }
+  hist[(int64_t)tid * tiles + blockIdx.x] = cnt[tid];
+  // the cells and the work counters (cell counts, overflow cells, the tickets of the
+  // mask and fill kernels and the mask pool's counter)
+  const long long nc = cg.all->ncells;
+  if (blockIdx.x == 0 && tid < 8) n_ucell[tid] = 0;
+  for (long long k = (long long)blockIdx.x * kRadixThreads + tid; k < nc;
+       k += (long long)gridDim.x * kRadixThreads) {
+    cell_start[k] = INT_MAX;
+    cell_end[k] = 0;
+  }
+}
+
 __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const uint32_t *keys, int64_t n,
                                                               int shift, int32_t *hist,
-                                                              int tiles, const GridDev *g) {
-  if (!g->ok) return;
+                                                              int tiles, const GridDev *g,
+                                                              const DevStatus *st) {
+  if (!g->ok || !st->not_identity) return;
   __shared__ int32_t cnt[256];
   cnt[threadIdx.x] = 0;
   __syncthreads();
@@ -303,8 +351,8 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const uint32_t *ke
 
 __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
     const uint32_t *kin, const int32_t *vin, uint32_t *kout, int32_t *vout, int64_t n, int shift,
-    const long long *offs, int tiles, const GridDev *g) {
-  if (!g->ok) return;
+    const long long *offs, int tiles, const GridDev *g, const DevStatus *st) {
+  if (!g->ok || !st->not_identity) return;
   __shared__ long long base_d[256];
   __shared__ int32_t wcnt[kRadixThreads / 32][256];
   __shared__ int32_t ctot[256];
@@ -344,7 +392,6 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
   }
 }
 
-// Exclusive scan of the (digit-major) histogram; reuses the int32->int64 scan.
 // --------------------------------------------------------- cell ranges
 // Occupied cells go to the work queue in two groups, the ones holding at least
 // kBigCell particles (3D cells at the usual h / dx) ahead of the rest, so the
@@ -355,19 +402,39 @@ constexpr int kBigCell = 24;
 __device__ __forceinline__ int cell_slot(int t, int nbig, int64_t n) {
   return t < nbig ? t : (int)(n - 1 - (t - nbig));
 }
+// The sorted keys, indices and positions: what the passes left, or, of a cloud in
+// cell order, the unsorted ones.
 template <typename T>
-__global__ void k_cells(const uint32_t *skeys, const int32_t *svals, int64_t n,
-                        const vec4_t<T> *pos, vec4_t<T> *spos, int32_t *cell_start,
-                        int32_t *cell_end, int32_t *ucell, int32_t *n_ucell, DevStatus *st,
-                        int32_t *order, const GridDev *g) {
+struct Sorted {
+  const uint32_t *keys, *keys0;
+  const int32_t *vals, *vals0;
+  const vec4_t<T> *spos, *pos;
+  const DevStatus *st;
+  __device__ __forceinline__ const uint32_t *key() const { return st->not_identity ? keys : keys0; }
+  __device__ __forceinline__ const int32_t *val() const { return st->not_identity ? vals : vals0; }
+  __device__ __forceinline__ const vec4_t<T> *position() const {
+    return st->not_identity ? spos : pos;
+  }
+};
+
+template <typename T>
+__global__ void k_cells(Sorted<T> so, int64_t n, vec4_t<T> *spos, int32_t *cell_start,
+                        int32_t *cell_end, int32_t *ucell, int32_t *n_ucell, int32_t *order,
+                        const GridDev *g) {
   if (!g->ok) return;
+  const bool moved = so.st->not_identity;
+  const uint32_t *skeys = so.key();
+  const int32_t *svals = so.val();
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
        s += (int64_t)gridDim.x * blockDim.x) {
     uint32_t key = skeys[s];
-    int32_t i = svals[s];
-    st4(spos + s, ld4(pos + i));
-    if (order) order[s] = i;
-    if (i != (int32_t)s) st->not_identity = 1;
+    if (moved) {
+      const int32_t i = svals[s];
+      st4(spos + s, ld4(so.pos + i));
+      if (order) order[s] = i;
+    } else if (order) {
+      order[s] = (int32_t)s;
+    }
     if (s == 0 || skeys[s - 1] != key) {
       cell_start[key] = (int32_t)s;
       // the work queue of the mask and fill kernels, costly cells first: cells
@@ -381,10 +448,6 @@ __global__ void k_cells(const uint32_t *skeys, const int32_t *svals, int64_t n,
     }
     if (s == n - 1 || skeys[s + 1] != key) cell_end[key] = (int32_t)(s + 1);
   }
-}
-
-__global__ void k_identity_flag(DevStatus *st) {
-  st->cells_identity = st->not_identity ? 0 : 1;
 }
 
 // --------------------------------------------------------- count / fill
@@ -429,13 +492,15 @@ enum { kRecS0 = 0, kRecP = 1, kRecTotal = 2, kRecRuns = 3, kRecPool = 4, kRecRun
 template <typename T, bool FILL>
 __global__ void __launch_bounds__(kNbrThreads) k_nbr(
     const GridDev *all, const int32_t *table, const int32_t *sel, const int32_t *n_sel,
-    const vec4_t<T> *spos, const int32_t *svals, int32_t *counts, const long long *row_ptr,
-    int32_t *col, long long cap_nnz, int64_t n) {
+    Sorted<T> so, int32_t *counts, const long long *row_ptr, int32_t *col, long long cap_nnz,
+    int64_t n) {
   using V = vec4_t<T>;
   constexpr int CAP = kNbrSmemBytes / sizeof(V);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V *cand = reinterpret_cast<V *>(smem_raw);
   if (!all->ok) return;
+  const V *spos = so.position();
+  const int32_t *svals = so.val();
   if (FILL && row_ptr[n] > cap_nnz) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = kNbrThreads / 32;
   const unsigned lt = (1u << lane) - 1u;
@@ -783,8 +848,8 @@ __device__ __forceinline__ void test_window(const float2 (&X)[kWinWords / 2],
 
 template <typename T>
 __global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
-    const GridDev *all, const int32_t *table, int32_t *n_ucell, const vec4_t<T> *spos,
-    const int32_t *svals, int32_t *counts, uint32_t *mask, Split split) {
+    const GridDev *all, const int32_t *table, int32_t *n_ucell, Sorted<T> so, int32_t *counts,
+    uint32_t *mask, Split split) {
   using V = vec4_t<T>;
   // prepared particles (-2 u, -h/2) and |u|^2 - h^2/4; the words of 32 particles
   __shared__ float4 s_part[kMaskWarps][kMaskBlock];
@@ -792,6 +857,8 @@ __global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
   __shared__ __align__(16) uint32_t s_res[kMaskWarps][32][kWinWords + 4];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   if (!all->ok) return;
+  const V *spos = so.position();
+  const int32_t *svals = so.val();
   ItemWalk walk;
   walk.start(table, n_ucell + 2, n_ucell[0], n_ucell[4], split, lane);
   int rec, s0, p0, P;
@@ -891,12 +958,13 @@ __global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
 // pay for a 16-word window: 382 -> 184 us on the 1M jet cloud.  Rows come out ascending when the cloud is in cell
 // order (candidates are runs of consecutive sorted positions, ascending).
 __global__ void __launch_bounds__(kFillThreads) k_nbr_fill(
-    const GridDev *all, const int32_t *table, int32_t *n_ucell, const int32_t *svals,
-    const uint32_t *mask, Split split, const long long *row_ptr, int32_t *col, long long cap_nnz,
+    const GridDev *all, const int32_t *table, int32_t *n_ucell, const int32_t *vals,
+    const int32_t *vals0, const DevStatus *st, const uint32_t *mask, Split split, const long long *row_ptr, int32_t *col, long long cap_nnz,
     int64_t n) {
   __shared__ __align__(16) uint2 srec[kFillWarps][32][kFillRec];     // (hit word, place)
   if (!all->ok) return;
   if (row_ptr[n] > cap_nnz) return;
+  const int32_t *svals = st->not_identity ? vals : vals0;
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u, bit = 1u << lane;
   uint2(*wr)[kFillRec] = srec[threadIdx.x >> 5];
@@ -1091,23 +1159,25 @@ __global__ void k_tmap(const long long *row_ptr, const int32_t *col, int64_t n, 
 
 // ------------------------------------------------------------------ host side
 // A1: grids, cell keys, stable radix sort, cell ranges, sorted positions and
-// (optionally) the cell order.  On return the sorted keys / indices are in
-// *kin / *vin.
+// (optionally) the cell order.  On return *so says where the sorted keys, indices
+// and positions are.
 template <typename T>
 static int sort_into_cells_t(mafp_ctx *ctx, int64_t n, int nb, const long long *cloud_off,
-                             const void *pos_h, int32_t *order, uint32_t **kin_out,
-                             int32_t **vin_out, cudaStream_t s) {
+                             const void *pos_h, int32_t *order, Sorted<T> *so, cudaStream_t s) {
   using V = vec4_t<T>;
   const V *pos = reinterpret_cast<const V *>(pos_h);
   const int sms = sm_count();
-  const int parts = std::max(1, std::min(kBoxBlocks / std::max(nb, 1), kBoxPartsMax));
+  // about 1024 particles per bounding-box block
+  const int64_t want = (n / nb + 1023) / 1024;
+  const int parts = (int)std::max<int64_t>(
+      1, std::min<int64_t>(want, std::min(kBoxBlocks / std::max(nb, 1), kBoxPartsMax)));
   MAFP_TIMED(ctx, s, "k_cloud_bbox",
              k_cloud_bbox<T><<<nb * parts, kBoxThreads, 0, s>>>(pos, n, cloud_off, nb, parts,
                                                                  ctx->cloud_partial,
                                                                  ctx->cloud_id));
-  MAFP_TIMED(ctx, s, "k_cloud_fold",
-             k_cloud_fold<<<(nb + kBoxThreads / 32 - 1) / (kBoxThreads / 32), kBoxThreads, 0, s>>>(
-                 ctx->cloud_partial, nb, parts));
+  if (nb > 1 && parts > 1)
+    MAFP_TIMED(ctx, s, "k_cloud_fold",
+               k_cloud_fold<<<nb, kBoxThreads, 0, s>>>(ctx->cloud_partial, parts));
   MAFP_TIMED(ctx, s, "k_cloud_grid",
              k_cloud_grid<<<1, kBoxThreads, 0, s>>>(ctx->cloud_partial, cloud_off, n, nb, parts,
                                                     ctx->d_grids,
@@ -1115,40 +1185,41 @@ static int sort_into_cells_t(mafp_ctx *ctx, int64_t n, int nb, const long long *
                                                     ctx->cap_cells,
                                                     0.01 * (double)ctx->tune.cell_edge_pct));
   CloudGrids cg{ctx->d_grids, ctx->cell_base, nb, ctx->d_grid};
-  MAFP_TIMED(ctx, s, "k_hash",
-             k_hash<T><<<grid_for(n, 256, sms * 16), 256, 0, s>>>(pos, n, ctx->cloud_id, cg,
-                                                                  ctx->keys_a, ctx->vals_a));
-  MAFP_TIMED(ctx, s, "k_clear_cells",
-             k_clear_cells<<<sms * 8, 256, 0, s>>>(ctx->d_grid, ctx->cell_start, ctx->cell_end,
-                                                   ctx->n_ucell));
-  MAFP_LAUNCH_CHECK(ctx);
   const int tiles = (int)((n + kRadixTile - 1) / kRadixTile);
+  MAFP_TIMED(ctx, s, "k_hash",
+             k_hash<T><<<tiles, kRadixThreads, 0, s>>>(pos, n, ctx->cloud_id, cg, ctx->keys_a,
+                                                       ctx->vals_a, ctx->radix_hist, tiles,
+                                                       ctx->cell_start, ctx->cell_end,
+                                                       ctx->n_ucell, ctx->d_status));
+  MAFP_LAUNCH_CHECK(ctx);
   uint32_t *kin = ctx->keys_a, *kout = ctx->keys_b;
   int32_t *vin = ctx->vals_a, *vout = ctx->vals_b;
   long long *offs = reinterpret_cast<long long *>(ctx->remap_i64);
   for (int p = 0; p < ctx->radix_passes; ++p) {
-    MAFP_TIMED(ctx, s, "k_radix_hist",
-               k_radix_hist<<<tiles, kRadixThreads, 0, s>>>(kin, n, 8 * p, ctx->radix_hist, tiles,
-                                                  ctx->d_grid));
-    int rc = scan_i32_to_i64(ctx, ctx->radix_hist, offs, (int64_t)256 * tiles, s);
+    if (p > 0)
+      MAFP_TIMED(ctx, s, "k_radix_hist",
+                 k_radix_hist<<<tiles, kRadixThreads, 0, s>>>(kin, n, 8 * p, ctx->radix_hist,
+                                                              tiles, ctx->d_grid, ctx->d_status));
+    int rc = scan_i32_to_i64(ctx, ctx->radix_hist, offs, (int64_t)256 * tiles, s,
+                             &ctx->d_status->not_identity);
     if (rc) return rc;
     MAFP_TIMED(ctx, s, "k_radix_scatter",
-               k_radix_scatter<<<tiles, kRadixThreads, 0, s>>>(kin, vin, kout, vout, n, 8 * p, offs, tiles,
-                                                     ctx->d_grid));
+               k_radix_scatter<<<tiles, kRadixThreads, 0, s>>>(kin, vin, kout, vout, n, 8 * p,
+                                                               offs, tiles, ctx->d_grid,
+                                                               ctx->d_status));
     MAFP_LAUNCH_CHECK(ctx);
-    uint32_t *tk = kin; kin = kout; kout = tk;
-    int32_t *tv = vin; vin = vout; vout = tv;
+    // (the unsorted keys and indices stay where they are: a cloud in cell order
+    // is read from them)
+    std::swap(kin, kout);
+    std::swap(vin, vout);
   }
   V *spos = reinterpret_cast<V *>(ctx->spos);
+  *so = Sorted<T>{kin, ctx->keys_a, vin, ctx->vals_a, spos, pos, ctx->d_status};
   MAFP_TIMED(ctx, s, "k_cells<T>",
-             k_cells<T><<<grid_for(n, 256, sms * 16), 256, 0, s>>>(kin, vin, n, pos, spos, ctx->cell_start,
-                                                        ctx->cell_end, ctx->ucell, ctx->n_ucell,
-                                                        ctx->d_status, order, ctx->d_grid));
-  MAFP_TIMED(ctx, s, "k_identity_flag",
-             k_identity_flag<<<1, 1, 0, s>>>(ctx->d_status));
+             k_cells<T><<<grid_for(n, 256, sms * 16), 256, 0, s>>>(
+                 *so, n, spos, ctx->cell_start, ctx->cell_end, ctx->ucell, ctx->n_ucell, order,
+                 ctx->d_grid));
   MAFP_LAUNCH_CHECK(ctx);
-  *kin_out = kin;
-  *vin_out = vin;
   return MAFP_OK;
 }
 
@@ -1156,13 +1227,10 @@ template <typename T>
 static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long *cloud_off,
                               const void *pos_h, int64_t *row_ptr, int32_t *col,
                               int64_t cap_nnz, int64_t *nnz_dev, int32_t *order, cudaStream_t s) {
-  using V = vec4_t<T>;
   const int sms = sm_count();
-  uint32_t *kin = nullptr;
-  int32_t *vin = nullptr;
-  int rc0 = sort_into_cells_t<T>(ctx, n, nb, cloud_off, pos_h, order, &kin, &vin, s);
+  Sorted<T> so;
+  int rc0 = sort_into_cells_t<T>(ctx, n, nb, cloud_off, pos_h, order, &so, s);
   if (rc0) return rc0;
-  V *spos = reinterpret_cast<V *>(ctx->spos);
   CloudGrids cg{ctx->d_grids, ctx->cell_base, nb, ctx->d_grid};
   const int nbr_blocks = sms * 8;
   int32_t *n_overflow = ctx->n_ucell + 1;
@@ -1180,11 +1248,11 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
                  pool_words, ctx->overflow, n));
   MAFP_TIMED(ctx, s, sizeof(T) == 4 ? "k_nbr_mask<float>" : "k_nbr_mask<double>",
              k_nbr_mask<T><<<sms * 8, kMaskThreads, 0, s>>>(
-                 ctx->d_grid, ctx->cell_table, ctx->n_ucell, spos, vin, ctx->counts,
-                 ctx->nbr_mask, split));
+                 ctx->d_grid, ctx->cell_table, ctx->n_ucell, so, ctx->counts, ctx->nbr_mask,
+                 split));
   MAFP_TIMED(ctx, s, "k_nbr<T,false>(overflow cells)",
              k_nbr<T, false><<<nbr_blocks, kNbrThreads, kNbrSmemBytes, s>>>(
-                 ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, spos, vin, ctx->counts,
+                 ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, so, ctx->counts,
                  nullptr, nullptr, 0, n));
   MAFP_LAUNCH_CHECK(ctx);
   int rc = scan_i32_to_i64(ctx, ctx->counts, reinterpret_cast<long long *>(row_ptr), n, s);
@@ -1193,11 +1261,12 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
              k_check_nnz<<<1, 1, 0, s>>>(rp, n, cap_nnz, nnz_dev, ctx->d_status, ctx->d_grid));
   MAFP_TIMED(ctx, s, "k_nbr_fill",
              k_nbr_fill<<<sms * 8, kFillThreads, 0, s>>>(ctx->d_grid, ctx->cell_table,
-                                                         ctx->n_ucell, vin, ctx->nbr_mask, split,
-                                                         rp, col, cap_nnz, n));
+                                                         ctx->n_ucell, so.vals, so.vals0,
+                                                         ctx->d_status, ctx->nbr_mask, split, rp,
+                                                         col, cap_nnz, n));
   MAFP_TIMED(ctx, s, "k_nbr<T,true>(overflow cells)",
              k_nbr<T, true><<<nbr_blocks, kNbrThreads, kNbrSmemBytes, s>>>(
-                 ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, spos, vin, ctx->counts,
+                 ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, so, ctx->counts,
                  rp, col, cap_nnz, n));
   MAFP_TIMED(ctx, s, "k_rowsort",
              k_rowsort<<<grid_for(n, kSortWarps, sms * 8), kSortWarps * 32, 0, s>>>(
@@ -1210,22 +1279,21 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
 int build_neighbours(mafp_ctx *ctx, int64_t n, int32_t dtype, const void *pos_h,
                      int64_t *row_ptr, int32_t *col, int64_t cap_nnz, int64_t *nnz_dev,
                      int32_t *order, cudaStream_t s) {
-  MAFP_TIMED(ctx, s, "k_set_one_cloud", k_set_one_cloud<<<1, 1, 0, s>>>(ctx->one_cloud, n));
   if (dtype == MAFP_F64)
-    return build_neighbours_t<double>(ctx, n, 1, ctx->one_cloud, pos_h, row_ptr, col, cap_nnz,
+    return build_neighbours_t<double>(ctx, n, 1, nullptr, pos_h, row_ptr, col, cap_nnz,
                                       nnz_dev, order, s);
-  return build_neighbours_t<float>(ctx, n, 1, ctx->one_cloud, pos_h, row_ptr, col, cap_nnz,
+  return build_neighbours_t<float>(ctx, n, 1, nullptr, pos_h, row_ptr, col, cap_nnz,
                                    nnz_dev, order, s);
 }
 
 int cell_order(mafp_ctx *ctx, int64_t n, int32_t dtype, const void *pos_h, int32_t *order,
                cudaStream_t s) {
-  MAFP_TIMED(ctx, s, "k_set_one_cloud", k_set_one_cloud<<<1, 1, 0, s>>>(ctx->one_cloud, n));
-  uint32_t *kin = nullptr;
-  int32_t *vin = nullptr;
-  if (dtype == MAFP_F64)
-    return sort_into_cells_t<double>(ctx, n, 1, ctx->one_cloud, pos_h, order, &kin, &vin, s);
-  return sort_into_cells_t<float>(ctx, n, 1, ctx->one_cloud, pos_h, order, &kin, &vin, s);
+  if (dtype == MAFP_F64) {
+    Sorted<double> so;
+    return sort_into_cells_t<double>(ctx, n, 1, nullptr, pos_h, order, &so, s);
+  }
+  Sorted<float> so;
+  return sort_into_cells_t<float>(ctx, n, 1, nullptr, pos_h, order, &so, s);
 }
 
 int build_neighbours_batched(mafp_ctx *ctx, int64_t n, int32_t dtype, int32_t nclouds,

@@ -68,7 +68,9 @@ __device__ __forceinline__ void store_state(unsigned long long *p, unsigned long
 __global__ void __launch_bounds__(kScanThreads) k_scan(const int32_t *in, long long *out,
                                                        int64_t n, int ntiles,
                                                        unsigned long long *state, int *ctr,
-                                                       DevStatus *st, long long wait_limit) {
+                                                       DevStatus *st, long long wait_limit,
+                                                       const int32_t *wanted) {
+  if (wanted && !*wanted) return;   // (every block alike: no ticket is taken)
   __shared__ int s_tile, s_last, s_gave_up;
   __shared__ long long s_prefix, s_red[kScanThreads / 32];
   if (threadIdx.x == 0) s_tile = atomicAdd(ctr, 1);
@@ -182,7 +184,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const int32_t *in, long l
   }
 }
 
-int scan_i32_to_i64(mafp_ctx *ctx, const int32_t *in, long long *out, int64_t n, cudaStream_t s) {
+int scan_i32_to_i64(mafp_ctx *ctx, const int32_t *in, long long *out, int64_t n, cudaStream_t s,
+                    const int32_t *wanted) {
   if (n <= 0) {
     MAFP_CUDA_TRY(ctx, cudaMemsetAsync(out, 0, sizeof(long long), s));
     return MAFP_OK;
@@ -192,7 +195,7 @@ int scan_i32_to_i64(mafp_ctx *ctx, const int32_t *in, long long *out, int64_t n,
   MAFP_TIMED(ctx, s, "k_scan",
              k_scan<<<(unsigned)ntiles, kScanThreads, 0, s>>>(
                  in, out, n, (int)ntiles, reinterpret_cast<unsigned long long *>(ctx->scan_tmp),
-                 ctx->scan_ctr, ctx->d_status, limit));
+                 ctx->scan_ctr, ctx->d_status, limit, wanted));
   MAFP_LAUNCH_CHECK(ctx);
   return MAFP_OK;
 }
