@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_bbox(const vec4_t<T> *pos
   int bad = 0;
   for (long long i = lo + (long long)part * blockDim.x + threadIdx.x; i < hi;
        i += (long long)parts * blockDim.x) {
-    cloud_id[i] = b;
+    if (nb > 1) cloud_id[i] = b;
     const vec4_t<T> p = ld4(pos + i);
     const bool ok = isfinite(p.x) && isfinite(p.y) && isfinite(p.z) && isfinite(p.w) && p.w > T(0);
     if (!ok) {
@@ -256,26 +256,40 @@ constexpr int kRadixThreads = 256;
 constexpr int kRadixItems = 8;
 constexpr int kRadixTile = kRadixThreads * kRadixItems;
 
+// Cell of coordinate x on one axis, floor((x - lo) inv_c) in FP64 clamped to the grid.
+// FP32 decides away from the cell faces: (x - lo) inv_c with the difference, 1/c and
+// the product each rounded once is off by at most 3 x 2^-24 of itself (a fourth
+// of that is to spare below), so the floor is certain unless a face lies nearer.
+// The face at lo is none (x >= lo), nor is the grid's upper one (clamped there).
+// The FP64 pipe has 1/64 of the FP32 rate: all particles on it, the kernel took
+// 64 us on the 1M jet cloud, 21 us so (its 4.3M cells cleared beside).
+template <typename T>
+__device__ __forceinline__ uint32_t cell_on_axis(T x, double lo, double inv_c, int dim) {
+  const float d = sizeof(T) == 4 ? (float)x - (float)lo : (float)((double)x - lo);
+  const float fi = (float)inv_c, v = d * fi, f = floorf(v), err = 2.4e-7f * v + 1e-30f;
+  const float top = (float)(dim - 1);
+  if ((f > 0.0f && v - f <= err) || (f < top && f + 1.0f - v <= err) || !(v < 4194304.0f) ||
+      !(fi > 1e-30f && fi < 1e30f)) {
+    const double w = floor(((double)x - lo) * inv_c), t = (double)(dim - 1);
+    return (uint32_t)(w < 0.0 ? 0.0 : (w > t ? t : w));
+  }
+  return (uint32_t)(f > top ? top : f);
+}
+
 template <typename T>
 __device__ __forceinline__ uint32_t cell_key(const vec4_t<T> &p, int b, const CloudGrids &cg) {
   const GridDev &g = cg.grids[b];
-  const double q[3] = {(double)p.x, (double)p.y, (double)p.z};
-  uint32_t c[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const double v = floor((q[a] - g.lo[a]) * g.inv_c), top = (double)(g.dim[a] - 1);
-    c[a] = (uint32_t)(v < 0.0 ? 0.0 : (v > top ? top : v));
-  }
-  return (uint32_t)cg.cell_base[b] +
-         (c[2] * (uint32_t)g.dim[1] + c[1]) * (uint32_t)g.dim[0] + c[0];
+  const uint32_t cx = cell_on_axis<T>(p.x, g.lo[0], g.inv_c, g.dim[0]);
+  const uint32_t cy = cell_on_axis<T>(p.y, g.lo[1], g.inv_c, g.dim[1]);
+  const uint32_t cz = cell_on_axis<T>(p.z, g.lo[2], g.inv_c, g.dim[2]);
+  return (uint32_t)cg.cell_base[b] + (cz * (uint32_t)g.dim[1] + cy) * (uint32_t)g.dim[0] + cx;
 }
 
 // One block per radix tile: the particles' cell keys, the tile's histogram of the
 // first digit, and whether a key is below the one before it.  Clouds that are in
 // cell order already (a time loop keeps them so) show it here, and the sort's
-// passes, their scans and the gather of the positions are left out: 165 of the
-// 215 us before the lists on the 1M jet cloud.  All blocks together also clear the
-// cells and the work counters.
+// passes and their scans are left out (100 us on the 1M jet cloud).  All blocks
+// together also clear the cells and the work counters.
 template <typename T>
 __global__ void __launch_bounds__(kRadixThreads) k_hash(const vec4_t<T> *pos, int64_t n,
                                                         const int32_t *cloud_id, CloudGrids cg,
@@ -402,51 +416,66 @@ constexpr int kBigCell = 24;
 __device__ __forceinline__ int cell_slot(int t, int nbig, int64_t n) {
   return t < nbig ? t : (int)(n - 1 - (t - nbig));
 }
-// The sorted keys, indices and positions: what the passes left, or, of a cloud in
-// cell order, the unsorted ones.
+// Cell ranges, sorted positions, the cell order and the work queue.  A cloud in
+// cell order is read from the unsorted keys (keys0) and its identity order written
+// to svals.  The queue's slots are taken by two atomics per block of particles (one
+// per warp, all on one address at 0.75 ns each, took 26 us on the 1M jet cloud).
+constexpr int kCellThreads = 512;
 template <typename T>
-struct Sorted {
-  const uint32_t *keys, *keys0;
-  const int32_t *vals, *vals0;
-  const vec4_t<T> *spos, *pos;
-  const DevStatus *st;
-  __device__ __forceinline__ const uint32_t *key() const { return st->not_identity ? keys : keys0; }
-  __device__ __forceinline__ const int32_t *val() const { return st->not_identity ? vals : vals0; }
-  __device__ __forceinline__ const vec4_t<T> *position() const {
-    return st->not_identity ? spos : pos;
-  }
-};
-
-template <typename T>
-__global__ void k_cells(Sorted<T> so, int64_t n, vec4_t<T> *spos, int32_t *cell_start,
-                        int32_t *cell_end, int32_t *ucell, int32_t *n_ucell, int32_t *order,
-                        const GridDev *g) {
+__global__ void __launch_bounds__(kCellThreads) k_cells(
+    const uint32_t *keys, const uint32_t *keys0, int32_t *svals, int64_t n,
+    const vec4_t<T> *pos, vec4_t<T> *spos, int32_t *cell_start, int32_t *cell_end,
+    int32_t *ucell, int32_t *n_ucell, int32_t *order, const DevStatus *st, const GridDev *g) {
+  __shared__ int s_cnt[2][kCellThreads / 32 + 1];
   if (!g->ok) return;
-  const bool moved = so.st->not_identity;
-  const uint32_t *skeys = so.key();
-  const int32_t *svals = so.val();
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
-       s += (int64_t)gridDim.x * blockDim.x) {
-    uint32_t key = skeys[s];
-    if (moved) {
-      const int32_t i = svals[s];
-      st4(spos + s, ld4(so.pos + i));
+  const bool moved = st->not_identity;
+  const uint32_t *skeys = moved ? keys : keys0;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int64_t s0 = (int64_t)blockIdx.x * kCellThreads; s0 < n;
+       s0 += (int64_t)gridDim.x * kCellThreads) {
+    const int64_t s = s0 + threadIdx.x;
+    bool head = false, big = false;
+    uint32_t key = 0;
+    if (s < n) {
+      key = skeys[s];
+      const int32_t i = moved ? svals[s] : (int32_t)s;
+      if (!moved) svals[s] = i;
+      st4(spos + s, ld4(pos + i));
       if (order) order[s] = i;
-    } else if (order) {
-      order[s] = (int32_t)s;
+      head = s == 0 || skeys[s - 1] != key;
+      big = head && s + kBigCell - 1 < n && skeys[s + kBigCell - 1] == key;
+      if (head) cell_start[key] = (int32_t)s;
+      if (s == n - 1 || skeys[s + 1] != key) cell_end[key] = (int32_t)(s + 1);
     }
-    if (s == 0 || skeys[s - 1] != key) {
-      cell_start[key] = (int32_t)s;
-      // the work queue of the mask and fill kernels, costly cells first: cells
-      // of at least kBigCell particles fill the list from the front, the others
-      // from the back (slot n - 1 - u; there are at most n cells)
-      const bool big = s + kBigCell - 1 < n && skeys[s + kBigCell - 1] == key;
-      const int64_t u = big ? (int64_t)atomicAdd(n_ucell, 1)
-                            : n - 1 - (int64_t)atomicAdd(n_ucell + 4, 1);
+    // the work queue of the mask and fill kernels, costly cells first: cells
+    // of at least kBigCell particles fill the list from the front, the others
+    // from the back (slot n - 1 - u; there are at most n cells)
+    const unsigned mb = __ballot_sync(0xffffffffu, big);
+    const unsigned ml = __ballot_sync(0xffffffffu, head && !big);
+    if (lane == 0) {
+      s_cnt[0][w] = __popc(mb);
+      s_cnt[1][w] = __popc(ml);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {   // first slots of the warps' cells in either group
+      int *c = s_cnt[threadIdx.x], total = 0;
+      for (int k = 0; k < kCellThreads / 32; ++k) {
+        const int v = c[k];
+        c[k] = total;
+        total += v;
+      }
+      const int first = total ? atomicAdd(n_ucell + 4 * threadIdx.x, total) : 0;
+      for (int k = 0; k < kCellThreads / 32; ++k) c[k] += first;
+    }
+    __syncthreads();
+    if (head) {
+      const unsigned m = big ? mb : ml;
+      const int64_t u0 = s_cnt[big ? 0 : 1][w] + __popc(m & ((1u << lane) - 1u));
+      const int64_t u = big ? u0 : n - 1 - u0;
       ucell[2 * u] = (int32_t)key;
       ucell[2 * u + 1] = (int32_t)s;
     }
-    if (s == n - 1 || skeys[s + 1] != key) cell_end[key] = (int32_t)(s + 1);
+    __syncthreads();   // the counts are read before the next particles' overwrite them
   }
 }
 
@@ -492,15 +521,13 @@ enum { kRecS0 = 0, kRecP = 1, kRecTotal = 2, kRecRuns = 3, kRecPool = 4, kRecRun
 template <typename T, bool FILL>
 __global__ void __launch_bounds__(kNbrThreads) k_nbr(
     const GridDev *all, const int32_t *table, const int32_t *sel, const int32_t *n_sel,
-    Sorted<T> so, int32_t *counts, const long long *row_ptr, int32_t *col, long long cap_nnz,
-    int64_t n) {
+    const vec4_t<T> *spos, const int32_t *svals, int32_t *counts, const long long *row_ptr,
+    int32_t *col, long long cap_nnz, int64_t n) {
   using V = vec4_t<T>;
   constexpr int CAP = kNbrSmemBytes / sizeof(V);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V *cand = reinterpret_cast<V *>(smem_raw);
   if (!all->ok) return;
-  const V *spos = so.position();
-  const int32_t *svals = so.val();
   if (FILL && row_ptr[n] > cap_nnz) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = kNbrThreads / 32;
   const unsigned lt = (1u << lane) - 1u;
@@ -848,8 +875,8 @@ __device__ __forceinline__ void test_window(const float2 (&X)[kWinWords / 2],
 
 template <typename T>
 __global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
-    const GridDev *all, const int32_t *table, int32_t *n_ucell, Sorted<T> so, int32_t *counts,
-    uint32_t *mask, Split split) {
+    const GridDev *all, const int32_t *table, int32_t *n_ucell, const vec4_t<T> *spos,
+    const int32_t *svals, int32_t *counts, uint32_t *mask, Split split) {
   using V = vec4_t<T>;
   // prepared particles (-2 u, -h/2) and |u|^2 - h^2/4; the words of 32 particles
   __shared__ float4 s_part[kMaskWarps][kMaskBlock];
@@ -857,8 +884,6 @@ __global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
   __shared__ __align__(16) uint32_t s_res[kMaskWarps][32][kWinWords + 4];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   if (!all->ok) return;
-  const V *spos = so.position();
-  const int32_t *svals = so.val();
   ItemWalk walk;
   walk.start(table, n_ucell + 2, n_ucell[0], n_ucell[4], split, lane);
   int rec, s0, p0, P;
@@ -958,13 +983,12 @@ __global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
 // pay for a 16-word window: 382 -> 184 us on the 1M jet cloud.  Rows come out ascending when the cloud is in cell
 // order (candidates are runs of consecutive sorted positions, ascending).
 __global__ void __launch_bounds__(kFillThreads) k_nbr_fill(
-    const GridDev *all, const int32_t *table, int32_t *n_ucell, const int32_t *vals,
-    const int32_t *vals0, const DevStatus *st, const uint32_t *mask, Split split, const long long *row_ptr, int32_t *col, long long cap_nnz,
+    const GridDev *all, const int32_t *table, int32_t *n_ucell, const int32_t *svals,
+    const uint32_t *mask, Split split, const long long *row_ptr, int32_t *col, long long cap_nnz,
     int64_t n) {
   __shared__ __align__(16) uint2 srec[kFillWarps][32][kFillRec];     // (hit word, place)
   if (!all->ok) return;
   if (row_ptr[n] > cap_nnz) return;
-  const int32_t *svals = st->not_identity ? vals : vals0;
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u, bit = 1u << lane;
   uint2(*wr)[kFillRec] = srec[threadIdx.x >> 5];
@@ -1159,16 +1183,17 @@ __global__ void k_tmap(const long long *row_ptr, const int32_t *col, int64_t n, 
 
 // ------------------------------------------------------------------ host side
 // A1: grids, cell keys, stable radix sort, cell ranges, sorted positions and
-// (optionally) the cell order.  On return *so says where the sorted keys, indices
-// and positions are.
+// (optionally) the cell order.  On return the sorted indices are in *svals, the
+// sorted positions in the context's spos.
 template <typename T>
 static int sort_into_cells_t(mafp_ctx *ctx, int64_t n, int nb, const long long *cloud_off,
-                             const void *pos_h, int32_t *order, Sorted<T> *so, cudaStream_t s) {
+                             const void *pos_h, int32_t *order, const int32_t **svals,
+                             cudaStream_t s) {
   using V = vec4_t<T>;
   const V *pos = reinterpret_cast<const V *>(pos_h);
   const int sms = sm_count();
-  // about 1024 particles per bounding-box block
-  const int64_t want = (n / nb + 1023) / 1024;
+  // about 2048 particles per bounding-box block, two blocks per SM of one cloud
+  const int64_t want = std::min<int64_t>((n / nb + 2047) / 2048, 2 * sms);
   const int parts = (int)std::max<int64_t>(
       1, std::min<int64_t>(want, std::min(kBoxBlocks / std::max(nb, 1), kBoxPartsMax)));
   MAFP_TIMED(ctx, s, "k_cloud_bbox",
@@ -1214,12 +1239,12 @@ static int sort_into_cells_t(mafp_ctx *ctx, int64_t n, int nb, const long long *
     std::swap(vin, vout);
   }
   V *spos = reinterpret_cast<V *>(ctx->spos);
-  *so = Sorted<T>{kin, ctx->keys_a, vin, ctx->vals_a, spos, pos, ctx->d_status};
   MAFP_TIMED(ctx, s, "k_cells<T>",
-             k_cells<T><<<grid_for(n, 256, sms * 16), 256, 0, s>>>(
-                 *so, n, spos, ctx->cell_start, ctx->cell_end, ctx->ucell, ctx->n_ucell, order,
-                 ctx->d_grid));
+             k_cells<T><<<grid_for(n, kCellThreads, sms * 4), kCellThreads, 0, s>>>(
+                 kin, ctx->keys_a, vin, n, pos, spos, ctx->cell_start, ctx->cell_end, ctx->ucell,
+                 ctx->n_ucell, order, ctx->d_status, ctx->d_grid));
   MAFP_LAUNCH_CHECK(ctx);
+  *svals = vin;
   return MAFP_OK;
 }
 
@@ -1228,9 +1253,10 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
                               const void *pos_h, int64_t *row_ptr, int32_t *col,
                               int64_t cap_nnz, int64_t *nnz_dev, int32_t *order, cudaStream_t s) {
   const int sms = sm_count();
-  Sorted<T> so;
-  int rc0 = sort_into_cells_t<T>(ctx, n, nb, cloud_off, pos_h, order, &so, s);
+  const int32_t *vin = nullptr;
+  int rc0 = sort_into_cells_t<T>(ctx, n, nb, cloud_off, pos_h, order, &vin, s);
   if (rc0) return rc0;
+  const vec4_t<T> *spos = reinterpret_cast<const vec4_t<T> *>(ctx->spos);
   CloudGrids cg{ctx->d_grids, ctx->cell_base, nb, ctx->d_grid};
   const int nbr_blocks = sms * 8;
   int32_t *n_overflow = ctx->n_ucell + 1;
@@ -1248,11 +1274,11 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
                  pool_words, ctx->overflow, n));
   MAFP_TIMED(ctx, s, sizeof(T) == 4 ? "k_nbr_mask<float>" : "k_nbr_mask<double>",
              k_nbr_mask<T><<<sms * 8, kMaskThreads, 0, s>>>(
-                 ctx->d_grid, ctx->cell_table, ctx->n_ucell, so, ctx->counts, ctx->nbr_mask,
-                 split));
+                 ctx->d_grid, ctx->cell_table, ctx->n_ucell, spos, vin, ctx->counts,
+                 ctx->nbr_mask, split));
   MAFP_TIMED(ctx, s, "k_nbr<T,false>(overflow cells)",
              k_nbr<T, false><<<nbr_blocks, kNbrThreads, kNbrSmemBytes, s>>>(
-                 ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, so, ctx->counts,
+                 ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, spos, vin, ctx->counts,
                  nullptr, nullptr, 0, n));
   MAFP_LAUNCH_CHECK(ctx);
   int rc = scan_i32_to_i64(ctx, ctx->counts, reinterpret_cast<long long *>(row_ptr), n, s);
@@ -1261,12 +1287,11 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
              k_check_nnz<<<1, 1, 0, s>>>(rp, n, cap_nnz, nnz_dev, ctx->d_status, ctx->d_grid));
   MAFP_TIMED(ctx, s, "k_nbr_fill",
              k_nbr_fill<<<sms * 8, kFillThreads, 0, s>>>(ctx->d_grid, ctx->cell_table,
-                                                         ctx->n_ucell, so.vals, so.vals0,
-                                                         ctx->d_status, ctx->nbr_mask, split, rp,
-                                                         col, cap_nnz, n));
+                                                         ctx->n_ucell, vin, ctx->nbr_mask, split,
+                                                         rp, col, cap_nnz, n));
   MAFP_TIMED(ctx, s, "k_nbr<T,true>(overflow cells)",
              k_nbr<T, true><<<nbr_blocks, kNbrThreads, kNbrSmemBytes, s>>>(
-                 ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, so, ctx->counts,
+                 ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, spos, vin, ctx->counts,
                  rp, col, cap_nnz, n));
   MAFP_TIMED(ctx, s, "k_rowsort",
              k_rowsort<<<grid_for(n, kSortWarps, sms * 8), kSortWarps * 32, 0, s>>>(
@@ -1288,12 +1313,10 @@ int build_neighbours(mafp_ctx *ctx, int64_t n, int32_t dtype, const void *pos_h,
 
 int cell_order(mafp_ctx *ctx, int64_t n, int32_t dtype, const void *pos_h, int32_t *order,
                cudaStream_t s) {
-  if (dtype == MAFP_F64) {
-    Sorted<double> so;
-    return sort_into_cells_t<double>(ctx, n, 1, nullptr, pos_h, order, &so, s);
-  }
-  Sorted<float> so;
-  return sort_into_cells_t<float>(ctx, n, 1, nullptr, pos_h, order, &so, s);
+  const int32_t *vin = nullptr;
+  if (dtype == MAFP_F64)
+    return sort_into_cells_t<double>(ctx, n, 1, nullptr, pos_h, order, &vin, s);
+  return sort_into_cells_t<float>(ctx, n, 1, nullptr, pos_h, order, &vin, s);
 }
 
 int build_neighbours_batched(mafp_ctx *ctx, int64_t n, int32_t dtype, int32_t nclouds,
