@@ -335,7 +335,10 @@ __global__ void __launch_bounds__(kClsThreads) k_smooth(int64_t n, const uint8_t
       int ok = 0;
       for (long long e = row_ptr[i] + lane; e < row_ptr[i + 1]; e += G) {
         const int j = col[e];
-        if (j != i && (model[j] == target || preflag[j] == f)) ok = 1;
+        if (j != i && (model[j] == target || preflag[j] == f)) {
+          ok = 1;   // one is enough
+          break;
+        }
       }
       if (!group_any<G>(ok)) f = 0;
     }

@@ -95,8 +95,20 @@ __global__ void k_owner_mark(const uint8_t *model, const uint8_t *type, const lo
   }
 }
 
+// FP32 squared distance, its differences taken in the input's own type: off by at
+// most 5 x 2^-24 of itself.
+template <typename T>
+__device__ __forceinline__ float dist2_32(const vec4_t<T> &a, const vec4_t<T> &b) {
+  const float dx = (float)(b.x - a.x), dy = (float)(b.y - a.y), dz = (float)(b.z - a.z);
+  return fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+}
+
 // Every candidate b finds its nearest 3D wall particle j^w in S_b (FP64 squared
 // distance, ties to the lower index) and is mapped onto it when j^w is flagged.
+// FP32 finds the smallest distance, and only the particles that may be the nearest
+// (within 2e-6 of it) take part in the FP64 comparison; one alone needs none.  All
+// in FP64, the 16 FP64 operations per neighbour bound the kernel: 219 us on the
+// 1M-particle tray.
 template <typename T>
 __global__ void k_owner(StateT<T> in, const uint8_t *flag, const long long *row_ptr,
                         const int32_t *col, int32_t *owner, int32_t *keep, const int32_t *cand,
@@ -109,25 +121,52 @@ __global__ void k_owner(StateT<T> in, const uint8_t *flag, const long long *row_
     const int64_t b = cand[q];
     const long long r0 = row_ptr[b], r1 = row_ptr[b + 1];
     const vec4_t<T> xb = ld4(in.pos_h + b);
-    double best = INFINITY;
-    int jw = INT_MAX;
+    // squared distances are not negative: their bits are ordered as they are
+    unsigned least = 0xffffffffu;
+    int j1 = INT_MAX;
     for (long long e = r0 + lane; e < r1; e += 32) {
       const int j = col[e];
       if (in.model[j] != MAFP_MODEL_3D || in.type[j] != MAFP_TYPE_WALL) continue;
-      const vec4_t<T> xj = ld4(in.pos_h + j);
-      const double d2 = dist2_64(xb.x, xb.y, xb.z, xj.x, xj.y, xj.z);
-      if (d2 < best || (d2 == best && j < jw)) {
-        best = d2;
-        jw = j;
+      const unsigned d = __float_as_uint(dist2_32<T>(xb, ld4(in.pos_h + j)));
+      if (d < least) {
+        least = d;
+        j1 = j;
       }
     }
+    const unsigned low = __reduce_min_sync(0xffffffffu, least);
+    int jw = INT_MAX;
+    if (low != 0xffffffffu) {
+      const float near = fmaf(__uint_as_float(low), 2e-6f, __uint_as_float(low)) + 1e-30f;
+      int count = 0;
+      for (long long e = r0 + lane; e < r1; e += 32) {
+        const int j = col[e];
+        if (in.model[j] != MAFP_MODEL_3D || in.type[j] != MAFP_TYPE_WALL) continue;
+        count += !(dist2_32<T>(xb, ld4(in.pos_h + j)) > near);
+      }
+      if (__reduce_add_sync(0xffffffffu, count) == 1) {
+        jw = __reduce_min_sync(0xffffffffu, count ? j1 : INT_MAX);
+      } else {
+        double best = INFINITY;
+        for (long long e = r0 + lane; e < r1; e += 32) {
+          const int j = col[e];
+          if (in.model[j] != MAFP_MODEL_3D || in.type[j] != MAFP_TYPE_WALL) continue;
+          const vec4_t<T> xj = ld4(in.pos_h + j);
+          if (dist2_32<T>(xb, xj) > near) continue;
+          const double d2 = dist2_64(xb.x, xb.y, xb.z, xj.x, xj.y, xj.z);
+          if (d2 < best || (d2 == best && j < jw)) {
+            best = d2;
+            jw = j;
+          }
+        }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oj = __shfl_xor_sync(0xffffffffu, jw, o);
-      if (ob < best || (ob == best && oj < jw)) {
-        best = ob;
-        jw = oj;
+        for (int o = 16; o > 0; o >>= 1) {
+          const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+          const int oj = __shfl_xor_sync(0xffffffffu, jw, o);
+          if (ob < best || (ob == best && oj < jw)) {
+            best = ob;
+            jw = oj;
+          }
+        }
       }
     }
     const int32_t own = (jw != INT_MAX && flag[jw] == 1) ? jw : -1;
@@ -194,7 +233,11 @@ __global__ void k_survivors(int64_t n, StateT<T> in, StateT<T> out, const uint8_
   }
 }
 
-// 3D -> 2D data mapping of Sec. 5.1 for each flagged particle (one warp each).
+// 3D -> 2D data mapping of Sec. 5.1 for each flagged particle: a warp sums over the
+// sets of up to kTo2dBatch of them, one after another, and then finishes them
+// side by side, a particle per lane -- the droplet diameter's FP64 cube root, in
+// one lane of 32 for every particle, took most of 241 us on the 1M-particle tray.
+constexpr int kTo2dBatch = 8;
 template <typename T>
 __global__ void k_to2d(StateT<T> in, StateT<T> out, const int32_t *owner,
                        const long long *keep_scan, const long long *row_ptr, const int32_t *col,
@@ -205,41 +248,57 @@ __global__ void k_to2d(StateT<T> in, StateT<T> out, const int32_t *owner,
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t nf = (int64_t)*n_flagged;
-  for (int64_t q = wid; q < nf; q += nwarps) {
-    const int64_t i = flagged[q];
-    const vec4_t<T> xi = ld4(in.pos_h + i), ni = ld4(in.normal + i);
-    T s[7] = {0, 0, 0, 0, 0, 0, 0};  // vp(4), rho, eta, mass
-    T H = 0;
+  const int batch = (int)min((int64_t)kTo2dBatch, nf / nwarps + 1);
+  for (int64_t q0 = wid * batch; q0 < nf; q0 += nwarps * batch) {
+    const int nb = (int)min((int64_t)batch, nf - q0);
+    // of the particle that this lane finishes
+    T t[7] = {0, 0, 0, 0, 0, 0, 0}, H = 0;   // vp(4), rho, eta, mass
     int cnt = 0;
-    for (long long e = row_ptr[i] + lane; e < row_ptr[i + 1]; e += 32) {
-      const int b = col[e];
-      if (owner[b] != (int32_t)i) continue;
-      const vec4_t<T> v = ld4(in.vp + b), xb = ld4(in.pos_h + b);
-      s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
-      s[4] += in.rho[b];
-      s[5] += in.eta[b];
-      s[6] += in.mass[b];
-      const T dn = fabs((xb.x - xi.x) * ni.x + (xb.y - xi.y) * ni.y + (xb.z - xi.z) * ni.z);
-      H = dn > H ? dn : H;
-      ++cnt;
-    }
+    for (int k = 0; k < nb; ++k) {
+      const int64_t i = flagged[q0 + k];
+      const vec4_t<T> xi = ld4(in.pos_h + i), ni = ld4(in.normal + i);
+      T s[7] = {0, 0, 0, 0, 0, 0, 0};
+      T hk = 0;
+      int ck = 0;
+      for (long long e = row_ptr[i] + lane; e < row_ptr[i + 1]; e += 32) {
+        const int b = col[e];
+        if (owner[b] != (int32_t)i) continue;
+        const vec4_t<T> v = ld4(in.vp + b), xb = ld4(in.pos_h + b);
+        s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
+        s[4] += in.rho[b];
+        s[5] += in.eta[b];
+        s[6] += in.mass[b];
+        const T dn = fabs((xb.x - xi.x) * ni.x + (xb.y - xi.y) * ni.y + (xb.z - xi.z) * ni.z);
+        hk = dn > hk ? dn : hk;
+        ++ck;
+      }
+      ck = __reduce_add_sync(0xffffffffu, ck);
+      if (ck) {
 #pragma unroll
-    for (int k = 0; k < 7; ++k) s[k] = group_sum<32>(s[k]);
-    cnt = group_sum<32>(cnt);
+        for (int c = 0; c < 7; ++c) s[c] = group_sum<32>(s[c]);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const T oh = __shfl_xor_sync(0xffffffffu, H, o);
-      H = oh > H ? oh : H;
+        for (int o = 16; o > 0; o >>= 1) {
+          const T oh = __shfl_xor_sync(0xffffffffu, hk, o);
+          hk = oh > hk ? oh : hk;
+        }
+        if (lane == k) {
+#pragma unroll
+          for (int c = 0; c < 7; ++c) t[c] = s[c];
+          H = hk;
+          cnt = ck;
+        }
+      }
     }
-    if (lane == 0) {
+    if (lane < nb) {
+      const int64_t i = flagged[q0 + lane];
       const long long o = keep_scan[i];
       const vec4_t<T> v = ld4(in.vp + i);
       const T k = T(1) + T(cnt);
-      st4(out.vp + o, mk4<T>((v.x + s[0]) / k, (v.y + s[1]) / k, (v.z + s[2]) / k, (v.w + s[3]) / k));
-      const T rho = (in.rho[i] + s[4]) / k;
-      const T m = in.mass[i] + s[6];
+      st4(out.vp + o, mk4<T>((v.x + t[0]) / k, (v.y + t[1]) / k, (v.z + t[2]) / k, (v.w + t[3]) / k));
+      const T rho = (in.rho[i] + t[4]) / k;
+      const T m = in.mass[i] + t[6];
       out.rho[o] = rho;
-      out.eta[o] = (in.eta[i] + s[5]) / k;
+      out.eta[o] = (in.eta[i] + t[5]) / k;
       out.mass[o] = m;
       out.diam[o] = droplet_diameter<T>((double)m, (double)rho);
       out.hfilm[o] = H;
