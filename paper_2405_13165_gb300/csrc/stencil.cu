@@ -49,8 +49,8 @@ template <int M> constexpr int kGatherU = M == 10 ? 4 : 2;
 // four rows, 57 % of them FP32; the FMA pipe is busy ~60 % of the time (a packed
 // FMA with three different operands takes 3 cycles of it, measured) at 14 warps
 // per SM, the registers' limit.  Film rows: L1 wavefronts (56 % busy) and issue
-// (53 %).  1M jet cloud, 3D 890 -> 794 us, film 300 -> 252 us; with the launch
-// shapes of a new context (32 and 8 lanes before) 2136 -> 951 us for 440k 3D rows.
+// (53 %).  1M jet cloud, 3D 890 -> 759 us, film 300 -> 257 us; with the launch
+// shapes of a new context (32 and 8 lanes before) 2136 -> 909 us for 440k 3D rows.
 __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -273,6 +273,19 @@ __device__ __forceinline__ void stencil_row32(int64_t i, const float4 *pos, cons
   };
   // sums p.lambda of the packed right-hand sides (p_0 = 1)
   auto dots = [&](const float2 (&p)[M], float2 &s01, float2 &s2x) {
+    if constexpr (M == 10) {
+      // nested: the coefficient pass needs no products then, and three short
+      // chains replace one of nine (951 -> 909 us)
+      auto poly = [&](const float2 (&l)[M]) {
+        const float2 a = fma2(p[1], l[4], fma2(p[2], l[7], fma2(p[3], l[8], l[1])));
+        const float2 b = fma2(p[2], l[5], fma2(p[3], l[9], l[2]));
+        const float2 c = fma2(p[3], l[6], l[3]);
+        return fma2(p[1], a, fma2(p[2], b, fma2(p[3], c, l[0])));
+      };
+      s01 = poly(l01);
+      s2x = poly(l2x);
+      return;
+    }
     s01 = l01[0];
     s2x = l2x[0];
 #pragma unroll
@@ -354,10 +367,10 @@ __device__ __forceinline__ void stencil_row32(int64_t i, const float4 *pos, cons
       float4 out;
       if constexpr (M == 10) {
         if constexpr (REFINE) {
-          float sl = lo[0];
-#pragma unroll
-          for (int r = 1; r < M; ++r) sl = fmaf(p[r].x, lo[r], sl);
-          s2x.y += sl;
+          const float x = p[1].x, y = p[2].x, z = p[3].x;
+          const float a = fmaf(x, lo[4], fmaf(y, lo[7], fmaf(z, lo[8], lo[1])));
+          const float b = fmaf(y, lo[5], fmaf(z, lo[9], lo[2]));
+          s2x.y += fmaf(x, a, fmaf(y, b, fmaf(z, fmaf(z, lo[6], lo[3]), lo[0])));
         }
         const float2 g = fma2(dup2(wg), s01, zero), gl = fma2(make_float2(wg, wl), s2x, zero);
         out = make_float4(g.x, g.y, gl.x, gl.y);
