@@ -456,7 +456,7 @@ __device__ void stencil_particle(int64_t i, const vec4_t<TS> *pos, const uint8_t
 #pragma unroll
   for (int r = 0; r < M; ++r) tr += L[pk(r, r)];
   C invd[M], pmin, pmax;
-  const bool pd = cholesky<M, C>(L, invd, sp.piv_tol_rel * tr, pmin, pmax);
+  const bool pd = cholesky<M, C, true>(L, invd, sp.piv_tol_rel * tr, pmin, pmax);
   const bool ok = pd && cnt >= M;
   const C cond = (pmax / pmin) * (pmax / pmin);
   C *Ls = sm + StSmem<M, G>::SCR;
@@ -655,7 +655,7 @@ static void launch_stencil(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void 
 // stencil2d_group, which also sets the order of the sums: the Laplacians of a
 // curved film are small differences, and gradients taken through them show every
 // change of rounding.  Film, FP64: 4 lanes, for the factorisation (697 us with 8,
-// 476 with 4 on the 60k jet cloud).
+// 461 with 4 on the 60k jet cloud).
 template <typename TS, typename C, bool REFINE>
 static int dispatch_stencils(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void *pos_h,
                              const uint8_t *model, const void *frame, const long long *rp,

@@ -199,8 +199,8 @@ __device__ __forceinline__ void static_for(F &&f) {
 // pivot is <= tol.  invd gets 1/L_kk; pmin / pmax the extreme pivots.  (Written
 // with loops under "#pragma unroll" the 6 x 6 case kept run-time indices, a
 // compare and a select per candidate register: 710 instructions per warp instead
-// of 200, a fifth of the film build.)  NEWTON (FP32): reciprocal root and one Newton
-// step, eight operations in every lane of the group against about twenty-five of
+// of 200, a fifth of the film build.)  NEWTON: reciprocal root (in FP32 with one Newton
+// step), eight operations in every lane of the group against about twenty-five of
 // a square root and a division; for the build, whose refinement corrects what
 // the last bit of a pivot changes -- the adjoint, unrefined, keeps the exact ones
 // (rounded differently its film gradients move by as much as their own error,
@@ -222,8 +222,13 @@ __device__ __forceinline__ bool cholesky(C (&L)[Basis<M>::NA], C (&invd)[M], C t
     const C dd = d > tol ? d : C(1);
     C lkk;
     if constexpr (NEWTON) {
-      C y = rsqrtf(dd);
-      y = fmaf(C(0.5) * y, fmaf(-dd * y, y, C(1)), y);
+      C y;
+      if constexpr (sizeof(C) == 4) {
+        y = rsqrtf(dd);
+        y = fmaf(C(0.5) * y, fmaf(-dd * y, y, C(1)), y);
+      } else {
+        y = rsqrt(dd);
+      }
       invd[k] = y;
       lkk = dd * y;
     } else {
