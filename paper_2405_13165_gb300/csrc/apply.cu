@@ -18,6 +18,7 @@ __global__ void __launch_bounds__(kApThreads) k_apply(int64_t n, const long long
                                                       const int32_t *col,
                                                       const vec4_t<T> *coef,
                                                       const vec4_t<T> *fields, T *out) {
+  pdl_sync();
   using V = vec4_t<T>;
   const int lane = threadIdx.x & (G - 1);
   const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
@@ -80,6 +81,7 @@ __global__ void __launch_bounds__(kApThreads) k_apply_T(int64_t n, const long lo
                                                         const vec4_t<T> *coef,
                                                         const vec4_t<T> *gout,
                                                         vec4_t<T> *gfields) {
+  pdl_sync();
   using V = vec4_t<T>;
   const int lane = threadIdx.x & (G - 1);
   const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
@@ -139,6 +141,7 @@ __global__ void __launch_bounds__(kApThreads) k_apply_T_scatter(int64_t n,
                                                                 const vec4_t<T> *coef,
                                                                 const vec4_t<T> *gout,
                                                                 vec4_t<T> *gfields) {
+  pdl_sync();
   using V = vec4_t<T>;
   const int lane = threadIdx.x & (G - 1);
   const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
@@ -194,11 +197,11 @@ static void launch_apply(mafp_ctx *ctx, cudaStream_t s, int64_t n, const long lo
   const V *c = (const V *)coef, *f = (const V *)fields;
   T *o = (T *)out;
   if (G == 4) {
-    MAFP_TIMED(ctx, s, "k_apply<G=4>", k_apply<T, 4, U><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, f, o));
+    MAFP_TIMED(ctx, s, "k_apply<G=4>", launch(k_apply<T, 4, U>, blocks, kApThreads, 0, s, n, rp, col, c, f, o));
   } else if (G == 16) {
-    MAFP_TIMED(ctx, s, "k_apply<G=16>", k_apply<T, 16, U><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, f, o));
+    MAFP_TIMED(ctx, s, "k_apply<G=16>", launch(k_apply<T, 16, U>, blocks, kApThreads, 0, s, n, rp, col, c, f, o));
   } else {
-    MAFP_TIMED(ctx, s, "k_apply<G=8>", k_apply<T, 8, U><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, f, o));
+    MAFP_TIMED(ctx, s, "k_apply<G=8>", launch(k_apply<T, 8, U>, blocks, kApThreads, 0, s, n, rp, col, c, f, o));
   }
 }
 
@@ -214,20 +217,20 @@ static int launch_apply_T(mafp_ctx *ctx, cudaStream_t s, int64_t n, const long l
   if (!tloc) {
     MAFP_CUDA_TRY(ctx, cudaMemsetAsync(gfields, 0, (size_t)n * sizeof(V), s));
     if (G == 4) {
-      MAFP_TIMED(ctx, s, "k_apply_T_scatter<G=4>", k_apply_T_scatter<T, 4><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, g, o));
+      MAFP_TIMED(ctx, s, "k_apply_T_scatter<G=4>", launch(k_apply_T_scatter<T, 4>, blocks, kApThreads, 0, s, n, rp, col, c, g, o));
     } else if (G == 16) {
-      MAFP_TIMED(ctx, s, "k_apply_T_scatter<G=16>", k_apply_T_scatter<T, 16><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, g, o));
+      MAFP_TIMED(ctx, s, "k_apply_T_scatter<G=16>", launch(k_apply_T_scatter<T, 16>, blocks, kApThreads, 0, s, n, rp, col, c, g, o));
     } else {
-      MAFP_TIMED(ctx, s, "k_apply_T_scatter<G=8>", k_apply_T_scatter<T, 8><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, g, o));
+      MAFP_TIMED(ctx, s, "k_apply_T_scatter<G=8>", launch(k_apply_T_scatter<T, 8>, blocks, kApThreads, 0, s, n, rp, col, c, g, o));
     }
     return MAFP_OK;
   }
   if (G == 4) {
-    MAFP_TIMED(ctx, s, "k_apply_T<G=4>", k_apply_T<T, 4><<<blocks, kApThreads, 0, s>>>(n, rp, col, tloc, c, g, o));
+    MAFP_TIMED(ctx, s, "k_apply_T<G=4>", launch(k_apply_T<T, 4>, blocks, kApThreads, 0, s, n, rp, col, tloc, c, g, o));
   } else if (G == 16) {
-    MAFP_TIMED(ctx, s, "k_apply_T<G=16>", k_apply_T<T, 16><<<blocks, kApThreads, 0, s>>>(n, rp, col, tloc, c, g, o));
+    MAFP_TIMED(ctx, s, "k_apply_T<G=16>", launch(k_apply_T<T, 16>, blocks, kApThreads, 0, s, n, rp, col, tloc, c, g, o));
   } else {
-    MAFP_TIMED(ctx, s, "k_apply_T<G=8>", k_apply_T<T, 8><<<blocks, kApThreads, 0, s>>>(n, rp, col, tloc, c, g, o));
+    MAFP_TIMED(ctx, s, "k_apply_T<G=8>", launch(k_apply_T<T, 8>, blocks, kApThreads, 0, s, n, rp, col, tloc, c, g, o));
   }
   return MAFP_OK;
 }

@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(kClsThreads, sizeof(T) == 4 ? 8 : 1) k_classif
     const vec4_t<T> *normal, const T *vol, const T *h3d, const uint8_t *user,
     const long long *row_ptr, const int32_t *col, uint8_t *preflag, vec4_t<T> *eig,
     vec4_t<T> *frame, T *hfilm, uint8_t *near, mafp_params prm, ClsConst kc, DevStatus *st) {
+  pdl_sync();
   using V = vec4_t<T>;
   const int lane = threadIdx.x & (G - 1);
   const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
@@ -324,6 +325,7 @@ __global__ void __launch_bounds__(kClsThreads) k_smooth(int64_t n, const uint8_t
                                                         const uint8_t *last,
                                                         const long long *row_ptr,
                                                         const int32_t *col, uint8_t *flag) {
+  pdl_sync();
   const int lane = threadIdx.x & (G - 1);
   const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
   const int64_t ngroups = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -366,20 +368,20 @@ static int classify_pca_g(mafp_ctx *ctx, int64_t n, int32_t dtype, const void *p
   const long long *rp = reinterpret_cast<const long long *>(row_ptr);
   if (dtype == MAFP_F64) {
     MAFP_TIMED(ctx, s, n64.s,
-               k_classify<double, G><<<blocks, kClsThreads, 0, s>>>(
+               launch(k_classify<double, G>, blocks, kClsThreads, 0, s, 
                    n, (const double4_16a *)pos_h, model, type, (const double4_16a *)normal,
                    (const double *)vol, (const double *)h3d, user, rp, col, preflag,
                    (double4_16a *)eig, (double4_16a *)frame, (double *)hfilm, near, ctx->prm,
                    kc, ctx->d_status));
   } else {
     MAFP_TIMED(ctx, s, n32.s,
-               k_classify<float, G><<<blocks, kClsThreads, 0, s>>>(
+               launch(k_classify<float, G>, blocks, kClsThreads, 0, s, 
                    n, (const float4 *)pos_h, model, type, (const float4 *)normal,
                    (const float *)vol, (const float *)h3d, user, rp, col, preflag, (float4 *)eig,
                    (float4 *)frame, (float *)hfilm, near, ctx->prm, kc, ctx->d_status));
   }
   MAFP_TIMED(ctx, s, nsm.s,
-             k_smooth<G><<<blocks, kClsThreads, 0, s>>>(n, model, preflag, last, rp, col, flag));
+             launch(k_smooth<G>, blocks, kClsThreads, 0, s, n, model, preflag, last, rp, col, flag));
   MAFP_LAUNCH_CHECK(ctx);
   return MAFP_OK;
 }

@@ -12,6 +12,7 @@ namespace mafp {
 
 __global__ void k_ghost_sources(int64_t n, const uint8_t *model, const long long *row_ptr,
                                 const int32_t *col, uint8_t *src) {
+  pdl_sync();
   const int lane = threadIdx.x & 31;
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -26,6 +27,7 @@ __global__ void k_ghost_sources(int64_t n, const uint8_t *model, const long long
 }
 
 __global__ void k_u8_to_i32(int64_t n, const uint8_t *a, uint8_t want, int32_t *out) {
+  pdl_sync();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     out[i] = a[i] == want ? 1 : 0;
@@ -35,6 +37,7 @@ __global__ void k_u8_to_i32(int64_t n, const uint8_t *a, uint8_t want, int32_t *
 // rows: writes the count, flags a capacity overflow (nothing is then copied).
 __global__ void k_select_total(const long long *off, int64_t n, int64_t base, long long cap,
                                int64_t *n_dev, DevStatus *st) {
+  pdl_sync();
   const long long total = base + off[n];
   if (n_dev) *n_dev = total;
   st->remap_scratch[1] = total > cap ? 1 : 0;
@@ -44,6 +47,7 @@ __global__ void k_select_total(const long long *off, int64_t n, int64_t base, lo
 template <typename T>
 __global__ void k_ghost_seed(int64_t n, StateT<T> in, const uint8_t *src, const long long *off,
                              StateT<T> g, uint8_t *gflag, int32_t *gsrc, const DevStatus *st) {
+  pdl_sync();
   if (st->remap_scratch[1] != 0) return;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -60,6 +64,7 @@ __global__ void k_ghost_seed(int64_t n, StateT<T> in, const uint8_t *src, const 
 template <typename T>
 __global__ void k_ghost_append(int64_t ng, StateT<T> gf, const long long *off, StateT<T> all,
                                int64_t base, const DevStatus *st) {
+  pdl_sync();
   if (st->remap_scratch[1] != 0) return;
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < ng;
        g += (int64_t)gridDim.x * blockDim.x) {
@@ -72,7 +77,7 @@ int ghost_sources(mafp_ctx *ctx, int64_t n, const uint8_t *model, const int64_t 
                   const int32_t *col, uint8_t *src, cudaStream_t s) {
   const int sms = sm_count();
   MAFP_TIMED(ctx, s, "k_ghost_sources",
-             k_ghost_sources<<<grid_for(n * 32, 256, sms * 32), 256, 0, s>>>(
+             launch(k_ghost_sources, grid_for(n * 32, 256, sms * 32), 256, 0, s, 
                  n, model, reinterpret_cast<const long long *>(row_ptr), col, src));
   MAFP_LAUNCH_CHECK(ctx);
   return MAFP_OK;
@@ -86,13 +91,13 @@ static int ghost_seed_t(mafp_ctx *ctx, int64_t n, const mafp_state *in_, const u
   long long *off = reinterpret_cast<long long *>(ctx->remap_i64);
   const int sms = sm_count();
   MAFP_TIMED(ctx, s, "k_u8_to_i32",
-             k_u8_to_i32<<<grid_for(n, 256, sms * 16), 256, 0, s>>>(n, src, 1, ctx->counts));
+             launch(k_u8_to_i32, grid_for(n, 256, sms * 16), 256, 0, s, n, src, 1, ctx->counts));
   int rc = scan_i32_to_i64(ctx, ctx->counts, off, n, s);
   if (rc) return rc;
   MAFP_TIMED(ctx, s, "k_select_total",
-             k_select_total<<<1, 1, 0, s>>>(off, n, 0, cap_ghost, n_ghost_dev, ctx->d_status));
+             launch(k_select_total, 1, 1, 0, s, off, n, 0, cap_ghost, n_ghost_dev, ctx->d_status));
   MAFP_TIMED(ctx, s, "k_ghost_seed<T>",
-             k_ghost_seed<T><<<grid_for(n, 256, sms * 16), 256, 0, s>>>(n, in, src, off, g, gflag,
+             launch(k_ghost_seed<T>, grid_for(n, 256, sms * 16), 256, 0, s, n, in, src, off, g, gflag,
                                                                       gsrc, ctx->d_status));
   MAFP_LAUNCH_CHECK(ctx);
   return MAFP_OK;
@@ -106,15 +111,15 @@ static int ghost_append_t(mafp_ctx *ctx, int64_t n_regular, int64_t n_ghost,
   long long *off = reinterpret_cast<long long *>(ctx->remap_i64);
   const int sms = sm_count();
   MAFP_TIMED(ctx, s, "k_u8_to_i32",
-             k_u8_to_i32<<<grid_for(n_ghost, 256, sms * 16), 256, 0, s>>>(n_ghost, gf.last, 1,
+             launch(k_u8_to_i32, grid_for(n_ghost, 256, sms * 16), 256, 0, s, n_ghost, gf.last, 1,
                                                                          ctx->counts));
   int rc = scan_i32_to_i64(ctx, ctx->counts, off, n_ghost, s);
   if (rc) return rc;
   MAFP_TIMED(ctx, s, "k_select_total",
-             k_select_total<<<1, 1, 0, s>>>(off, n_ghost, n_regular, cap_all, n_all_dev,
+             launch(k_select_total, 1, 1, 0, s, off, n_ghost, n_regular, cap_all, n_all_dev,
                                             ctx->d_status));
   MAFP_TIMED(ctx, s, "k_ghost_append<T>",
-             k_ghost_append<T><<<grid_for(n_ghost, 256, sms * 16), 256, 0, s>>>(
+             launch(k_ghost_append<T>, grid_for(n_ghost, 256, sms * 16), 256, 0, s, 
                  n_ghost, gf, off, all, n_regular, ctx->d_status));
   MAFP_LAUNCH_CHECK(ctx);
   return MAFP_OK;

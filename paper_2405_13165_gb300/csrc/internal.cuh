@@ -193,7 +193,32 @@ __device__ __forceinline__ void inc_ll(long long *p, long long v = 1) {
 
 template <typename T> __device__ __forceinline__ bool finite_(T x) { return isfinite(x); }
 
-// Launch helpers
+// Launch helpers.  Every kernel is launched with programmatic stream serialization
+// and begins with pdl_sync(): its blocks may be set up as soon as all blocks of the
+// kernel before it have started, and wait there until that kernel is done and its
+// writes are visible.  Nothing is read or written before the wait, so the order of
+// the calls is that of plain launches, without the gap between them.
+__device__ __forceinline__ void pdl_sync() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... K, typename... A>
+inline void launch(void (*kernel)(K...), int grid, int block, size_t smem, cudaStream_t s,
+                   A &&...args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)block);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, static_cast<K>(args)...);
+}
+
 inline int grid_for(int64_t work, int per_block, int max_blocks = 1 << 20) {
   int64_t b = (work + per_block - 1) / per_block;
   if (b < 1) b = 1;

@@ -45,6 +45,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_bbox(const vec4_t<T> *pos
                                                             const long long *off, int nb,
                                                             int parts, double *partial,
                                                             int32_t *cloud_id) {
+  pdl_sync();
   const int b = blockIdx.x / parts, part = blockIdx.x % parts;
   // offsets are checked in k_cloud_grid; clamping keeps every access in [0, n)
   const long long lo = max(0LL, min(cloud_begin(off, b, n), (long long)n));
@@ -122,6 +123,7 @@ __device__ __forceinline__ void fold_cloud(double *pb, int parts) {
 }
 
 __global__ void __launch_bounds__(kBoxThreads) k_cloud_fold(double *partial, int parts) {
+  pdl_sync();
   fold_cloud(partial + (long long)blockIdx.x * parts * 8, parts);
 }
 
@@ -152,6 +154,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_grid(double *partial,
                                                             long long *cell_base, GridDev *all,
                                                             DevStatus *st, long long cap_cells,
                                                             double edge_factor) {
+  pdl_sync();
   __shared__ double s_nonfinite, s_cells;
   __shared__ double s_scale;
   __shared__ int s_bad;
@@ -297,6 +300,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_hash(const vec4_t<T> *pos, in
                                                         int32_t *hist, int tiles,
                                                         int32_t *cell_start, int32_t *cell_end,
                                                         int32_t *n_ucell, DevStatus *st) {
+  pdl_sync();
   __shared__ int32_t cnt[256];
   __shared__ uint32_t last[kRadixItems + 1][kRadixThreads / 32];
   if (!cg.all->ok) return;
@@ -350,6 +354,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const uint32_t *ke
                                                               int shift, int32_t *hist,
                                                               int tiles, const GridDev *g,
                                                               const DevStatus *st) {
+  pdl_sync();
   if (!g->ok || !st->not_identity) return;
   __shared__ int32_t cnt[256];
   cnt[threadIdx.x] = 0;
@@ -366,6 +371,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const uint32_t *ke
 __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
     const uint32_t *kin, const int32_t *vin, uint32_t *kout, int32_t *vout, int64_t n, int shift,
     const long long *offs, int tiles, const GridDev *g, const DevStatus *st) {
+  pdl_sync();
   if (!g->ok || !st->not_identity) return;
   __shared__ long long base_d[256];
   __shared__ int32_t wcnt[kRadixThreads / 32][256];
@@ -426,6 +432,7 @@ __global__ void __launch_bounds__(kCellThreads) k_cells(
     const uint32_t *keys, const uint32_t *keys0, int32_t *svals, int64_t n,
     const vec4_t<T> *pos, vec4_t<T> *spos, int32_t *cell_start, int32_t *cell_end,
     int32_t *ucell, int32_t *n_ucell, int32_t *order, const DevStatus *st, const GridDev *g) {
+  pdl_sync();
   __shared__ int s_cnt[2][kCellThreads / 32 + 1];
   if (!g->ok) return;
   const bool moved = st->not_identity;
@@ -523,6 +530,7 @@ __global__ void __launch_bounds__(kNbrThreads) k_nbr(
     const GridDev *all, const int32_t *table, const int32_t *sel, const int32_t *n_sel,
     const vec4_t<T> *spos, const int32_t *svals, int32_t *counts, const long long *row_ptr,
     int32_t *col, long long cap_nnz, int64_t n) {
+  pdl_sync();
   using V = vec4_t<T>;
   constexpr int CAP = kNbrSmemBytes / sizeof(V);
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -573,6 +581,7 @@ __global__ void __launch_bounds__(kNbrThreads) k_nbr(
 
 __global__ void k_check_nnz(const long long *row_ptr, int64_t n, long long cap_nnz,
                             int64_t *nnz_dev, DevStatus *st, const GridDev *g) {
+  pdl_sync();
   if (!g->ok) return;
   long long nnz = row_ptr[n];
   st->nnz = nnz;
@@ -647,6 +656,7 @@ __global__ void __launch_bounds__(128) k_cell_table(
     CloudGrids cg, const int32_t *ucell, int32_t *n_ucell, const int32_t *cell_start,
     const int32_t *cell_end, int32_t *table, long long pool_words, int32_t *overflow,
     int64_t n) {
+  pdl_sync();
   if (!cg.all->ok) return;
   const int lane = threadIdx.x & 31;
   const int nbig = n_ucell[0], nu = nbig + n_ucell[4];
@@ -877,6 +887,7 @@ template <typename T>
 __global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
     const GridDev *all, const int32_t *table, int32_t *n_ucell, const vec4_t<T> *spos,
     const int32_t *svals, int32_t *counts, uint32_t *mask, Split split) {
+  pdl_sync();
   using V = vec4_t<T>;
   // prepared particles (-2 u, -h/2) and |u|^2 - h^2/4; the words of 32 particles
   __shared__ float4 s_part[kMaskWarps][kMaskBlock];
@@ -986,6 +997,7 @@ __global__ void __launch_bounds__(kFillThreads) k_nbr_fill(
     const GridDev *all, const int32_t *table, int32_t *n_ucell, const int32_t *svals,
     const uint32_t *mask, Split split, const long long *row_ptr, int32_t *col, long long cap_nnz,
     int64_t n) {
+  pdl_sync();
   __shared__ __align__(16) uint2 srec[kFillWarps][32][kFillRec];     // (hit word, place)
   if (!all->ok) return;
   if (row_ptr[n] > cap_nnz) return;
@@ -1109,6 +1121,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_rowsort(const long long *ro
                                                              int32_t *col, int64_t n,
                                                              long long cap_nnz,
                                                              DevStatus *st, const GridDev *g) {
+  pdl_sync();
   if (!g->ok || !st->not_identity) return;
   if (row_ptr[n] > cap_nnz) return;
   __shared__ int32_t buf[kSortWarps][kSortBuf];
@@ -1159,6 +1172,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_rowsort(const long long *ro
 // tloc[e] = position of i inside row j for the entry e = (i, j).
 __global__ void k_tmap(const long long *row_ptr, const int32_t *col, int64_t n, uint16_t *tloc,
                        DevStatus *st) {
+  pdl_sync();
   const int lane = threadIdx.x & 31;
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1197,14 +1211,14 @@ static int sort_into_cells_t(mafp_ctx *ctx, int64_t n, int nb, const long long *
   const int parts = (int)std::max<int64_t>(
       1, std::min<int64_t>(want, std::min(kBoxBlocks / std::max(nb, 1), kBoxPartsMax)));
   MAFP_TIMED(ctx, s, "k_cloud_bbox",
-             k_cloud_bbox<T><<<nb * parts, kBoxThreads, 0, s>>>(pos, n, cloud_off, nb, parts,
+             launch(k_cloud_bbox<T>, nb * parts, kBoxThreads, 0, s, pos, n, cloud_off, nb, parts,
                                                                  ctx->cloud_partial,
                                                                  ctx->cloud_id));
   if (nb > 1 && parts > 1)
     MAFP_TIMED(ctx, s, "k_cloud_fold",
-               k_cloud_fold<<<nb, kBoxThreads, 0, s>>>(ctx->cloud_partial, parts));
+               launch(k_cloud_fold, nb, kBoxThreads, 0, s, ctx->cloud_partial, parts));
   MAFP_TIMED(ctx, s, "k_cloud_grid",
-             k_cloud_grid<<<1, kBoxThreads, 0, s>>>(ctx->cloud_partial, cloud_off, n, nb, parts,
+             launch(k_cloud_grid, 1, kBoxThreads, 0, s, ctx->cloud_partial, cloud_off, n, nb, parts,
                                                     ctx->d_grids,
                                                     ctx->cell_base, ctx->d_grid, ctx->d_status,
                                                     ctx->cap_cells,
@@ -1212,7 +1226,7 @@ static int sort_into_cells_t(mafp_ctx *ctx, int64_t n, int nb, const long long *
   CloudGrids cg{ctx->d_grids, ctx->cell_base, nb, ctx->d_grid};
   const int tiles = (int)((n + kRadixTile - 1) / kRadixTile);
   MAFP_TIMED(ctx, s, "k_hash",
-             k_hash<T><<<tiles, kRadixThreads, 0, s>>>(pos, n, ctx->cloud_id, cg, ctx->keys_a,
+             launch(k_hash<T>, tiles, kRadixThreads, 0, s, pos, n, ctx->cloud_id, cg, ctx->keys_a,
                                                        ctx->vals_a, ctx->radix_hist, tiles,
                                                        ctx->cell_start, ctx->cell_end,
                                                        ctx->n_ucell, ctx->d_status));
@@ -1223,13 +1237,13 @@ static int sort_into_cells_t(mafp_ctx *ctx, int64_t n, int nb, const long long *
   for (int p = 0; p < ctx->radix_passes; ++p) {
     if (p > 0)
       MAFP_TIMED(ctx, s, "k_radix_hist",
-                 k_radix_hist<<<tiles, kRadixThreads, 0, s>>>(kin, n, 8 * p, ctx->radix_hist,
+                 launch(k_radix_hist, tiles, kRadixThreads, 0, s, kin, n, 8 * p, ctx->radix_hist,
                                                               tiles, ctx->d_grid, ctx->d_status));
     int rc = scan_i32_to_i64(ctx, ctx->radix_hist, offs, (int64_t)256 * tiles, s,
                              &ctx->d_status->not_identity);
     if (rc) return rc;
     MAFP_TIMED(ctx, s, "k_radix_scatter",
-               k_radix_scatter<<<tiles, kRadixThreads, 0, s>>>(kin, vin, kout, vout, n, 8 * p,
+               launch(k_radix_scatter, tiles, kRadixThreads, 0, s, kin, vin, kout, vout, n, 8 * p,
                                                                offs, tiles, ctx->d_grid,
                                                                ctx->d_status));
     MAFP_LAUNCH_CHECK(ctx);
@@ -1240,7 +1254,7 @@ static int sort_into_cells_t(mafp_ctx *ctx, int64_t n, int nb, const long long *
   }
   V *spos = reinterpret_cast<V *>(ctx->spos);
   MAFP_TIMED(ctx, s, "k_cells<T>",
-             k_cells<T><<<grid_for(n, kCellThreads, sms * 4), kCellThreads, 0, s>>>(
+             launch(k_cells<T>, grid_for(n, kCellThreads, sms * 4), kCellThreads, 0, s, 
                  kin, ctx->keys_a, vin, n, pos, spos, ctx->cell_start, ctx->cell_end, ctx->ucell,
                  ctx->n_ucell, order, ctx->d_status, ctx->d_grid));
   MAFP_LAUNCH_CHECK(ctx);
@@ -1269,32 +1283,32 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
   const Split split = n <= kSplitAll ? Split{3, 1} : n <= kSplitMore ? Split{2, 0} : Split{1, 0};
   const long long *rp = reinterpret_cast<const long long *>(row_ptr);
   MAFP_TIMED(ctx, s, "k_cell_table",
-             k_cell_table<<<grid_for(n, 128, sms * 16), 128, 0, s>>>(
+             launch(k_cell_table, grid_for(n, 128, sms * 16), 128, 0, s, 
                  cg, ctx->ucell, ctx->n_ucell, ctx->cell_start, ctx->cell_end, ctx->cell_table,
                  pool_words, ctx->overflow, n));
   MAFP_TIMED(ctx, s, sizeof(T) == 4 ? "k_nbr_mask<float>" : "k_nbr_mask<double>",
-             k_nbr_mask<T><<<sms * 8, kMaskThreads, 0, s>>>(
+             launch(k_nbr_mask<T>, sms * 8, kMaskThreads, 0, s, 
                  ctx->d_grid, ctx->cell_table, ctx->n_ucell, spos, vin, ctx->counts,
                  ctx->nbr_mask, split));
   MAFP_TIMED(ctx, s, "k_nbr<T,false>(overflow cells)",
-             k_nbr<T, false><<<nbr_blocks, kNbrThreads, kNbrSmemBytes, s>>>(
+             launch(k_nbr<T, false>, nbr_blocks, kNbrThreads, kNbrSmemBytes, s, 
                  ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, spos, vin, ctx->counts,
                  nullptr, nullptr, 0, n));
   MAFP_LAUNCH_CHECK(ctx);
   int rc = scan_i32_to_i64(ctx, ctx->counts, reinterpret_cast<long long *>(row_ptr), n, s);
   if (rc) return rc;
   MAFP_TIMED(ctx, s, "k_check_nnz",
-             k_check_nnz<<<1, 1, 0, s>>>(rp, n, cap_nnz, nnz_dev, ctx->d_status, ctx->d_grid));
+             launch(k_check_nnz, 1, 1, 0, s, rp, n, cap_nnz, nnz_dev, ctx->d_status, ctx->d_grid));
   MAFP_TIMED(ctx, s, "k_nbr_fill",
-             k_nbr_fill<<<sms * 8, kFillThreads, 0, s>>>(ctx->d_grid, ctx->cell_table,
+             launch(k_nbr_fill, sms * 8, kFillThreads, 0, s, ctx->d_grid, ctx->cell_table,
                                                          ctx->n_ucell, vin, ctx->nbr_mask, split,
                                                          rp, col, cap_nnz, n));
   MAFP_TIMED(ctx, s, "k_nbr<T,true>(overflow cells)",
-             k_nbr<T, true><<<nbr_blocks, kNbrThreads, kNbrSmemBytes, s>>>(
+             launch(k_nbr<T, true>, nbr_blocks, kNbrThreads, kNbrSmemBytes, s, 
                  ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, spos, vin, ctx->counts,
                  rp, col, cap_nnz, n));
   MAFP_TIMED(ctx, s, "k_rowsort",
-             k_rowsort<<<grid_for(n, kSortWarps, sms * 8), kSortWarps * 32, 0, s>>>(
+             launch(k_rowsort, grid_for(n, kSortWarps, sms * 8), kSortWarps * 32, 0, s, 
       reinterpret_cast<const long long *>(row_ptr), col, n, cap_nnz, ctx->d_status,
       ctx->d_grid));
   MAFP_LAUNCH_CHECK(ctx);
@@ -1345,7 +1359,7 @@ void init_kernel_attributes() {
 int transpose_map(mafp_ctx *ctx, int64_t n, const int64_t *row_ptr, const int32_t *col,
                   uint16_t *tloc, cudaStream_t s) {
   MAFP_TIMED(ctx, s, "k_tmap",
-             k_tmap<<<grid_for(n * 32, 256, sm_count() * 16), 256, 0, s>>>(
+             launch(k_tmap, grid_for(n * 32, 256, sm_count() * 16), 256, 0, s, 
       reinterpret_cast<const long long *>(row_ptr), col, n, tloc, ctx->d_status));
   MAFP_LAUNCH_CHECK(ctx);
   return MAFP_OK;

@@ -16,6 +16,7 @@ __global__ void k_film_momentum(int64_t n, const uint8_t *model, vec4_t<T> *vp, 
                                 const T *eta, const T *hfilm, const vec4_t<T> *normal,
                                 const vec4_t<T> *out, double gx, double gy, double gz,
                                 double dt) {
+  pdl_sync();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     if (model[i] != MAFP_MODEL_2D) continue;
@@ -49,6 +50,7 @@ template <typename T>
 __global__ void k_plane_flux(int64_t n, const vec4_t<T> *p0, const vec4_t<T> *p1, const T *mass,
                              const T *rho, double cx, double cy, double cz, double mx, double my,
                              double mz, double *out) {
+  pdl_sync();
   double s = 0.0, cnt = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -81,6 +83,7 @@ __global__ void k_plane_flux(int64_t n, const vec4_t<T> *p0, const vec4_t<T> *p1
 template <typename T>
 __global__ void k_normal_stress(int64_t n, const uint8_t *select, const vec4_t<T> *out4,
                                 const T *eta, const vec4_t<T> *normal, double *res) {
+  pdl_sync();
   double s = 0.0, cnt = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -112,13 +115,13 @@ int film_momentum(mafp_ctx *ctx, int64_t n, int32_t dtype, const uint8_t *model,
   const int blocks = grid_for(n, kPostThreads, sm_count() * 16);
   if (dtype == MAFP_F64) {
     MAFP_TIMED(ctx, s, "k_film_momentum<double>",
-               k_film_momentum<double><<<blocks, kPostThreads, 0, s>>>(
+               launch(k_film_momentum<double>, blocks, kPostThreads, 0, s, 
                    n, model, (double4_16a *)vp, (const double *)rho, (const double *)eta,
                    (const double *)hfilm, (const double4_16a *)normal, (const double4_16a *)out,
                    g[0], g[1], g[2], dt));
   } else {
     MAFP_TIMED(ctx, s, "k_film_momentum<float>",
-               k_film_momentum<float><<<blocks, kPostThreads, 0, s>>>(
+               launch(k_film_momentum<float>, blocks, kPostThreads, 0, s, 
                    n, model, (float4 *)vp, (const float *)rho, (const float *)eta,
                    (const float *)hfilm, (const float4 *)normal, (const float4 *)out, g[0], g[1],
                    g[2], dt));
@@ -133,12 +136,12 @@ int plane_flux(mafp_ctx *ctx, int64_t n, int32_t dtype, const void *p0, const vo
   const int blocks = grid_for(n, kPostThreads, sm_count() * 8);
   if (dtype == MAFP_F64) {
     MAFP_TIMED(ctx, s, "k_plane_flux<double>",
-               k_plane_flux<double><<<blocks, kPostThreads, 0, s>>>(
+               launch(k_plane_flux<double>, blocks, kPostThreads, 0, s, 
                    n, (const double4_16a *)p0, (const double4_16a *)p1, (const double *)mass,
                    (const double *)rho, c[0], c[1], c[2], m[0], m[1], m[2], out));
   } else {
     MAFP_TIMED(ctx, s, "k_plane_flux<float>",
-               k_plane_flux<float><<<blocks, kPostThreads, 0, s>>>(
+               launch(k_plane_flux<float>, blocks, kPostThreads, 0, s, 
                    n, (const float4 *)p0, (const float4 *)p1, (const float *)mass,
                    (const float *)rho, c[0], c[1], c[2], m[0], m[1], m[2], out));
   }
@@ -152,12 +155,12 @@ int normal_stress(mafp_ctx *ctx, int64_t n, int32_t dtype, const uint8_t *select
   const int blocks = grid_for(n, kPostThreads, sm_count() * 8);
   if (dtype == MAFP_F64) {
     MAFP_TIMED(ctx, s, "k_normal_stress<double>",
-               k_normal_stress<double><<<blocks, kPostThreads, 0, s>>>(
+               launch(k_normal_stress<double>, blocks, kPostThreads, 0, s, 
                    n, select, (const double4_16a *)out, (const double *)eta,
                    (const double4_16a *)normal, res));
   } else {
     MAFP_TIMED(ctx, s, "k_normal_stress<float>",
-               k_normal_stress<float><<<blocks, kPostThreads, 0, s>>>(
+               launch(k_normal_stress<float>, blocks, kPostThreads, 0, s, 
                    n, select, (const float4 *)out, (const float *)eta, (const float4 *)normal,
                    res));
   }

@@ -49,6 +49,7 @@ template <typename T>
 __global__ void k_owner_seed(int64_t n, StateT<T> in, const uint8_t *flag, int32_t *owner,
                              int32_t *keep, int32_t *gam, double c_psi, int32_t *flagged,
                              unsigned long long *n_flagged) {
+  pdl_sync();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t b0 = (int64_t)blockIdx.x * blockDim.x; b0 < n; b0 += stride) {
     const int64_t b = b0 + threadIdx.x;
@@ -74,6 +75,7 @@ __global__ void k_owner_mark(const uint8_t *model, const uint8_t *type, const lo
                              const int32_t *col, int32_t *owner, const int32_t *flagged,
                              const unsigned long long *n_flagged, int32_t *cand,
                              unsigned long long *n_cand) {
+  pdl_sync();
   const int lane = threadIdx.x & 31;
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -113,6 +115,7 @@ template <typename T>
 __global__ void k_owner(StateT<T> in, const uint8_t *flag, const long long *row_ptr,
                         const int32_t *col, int32_t *owner, int32_t *keep, const int32_t *cand,
                         const unsigned long long *n_cand) {
+  pdl_sync();
   const int lane = threadIdx.x & 31;
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -179,6 +182,7 @@ __global__ void k_owner(StateT<T> in, const uint8_t *flag, const long long *row_
 
 __global__ void k_remap_count(const long long *keep_scan, const long long *gam_scan, int64_t n,
                               long long cap_out, int64_t *n_out_dev, DevStatus *st) {
+  pdl_sync();
   const long long n_out = keep_scan[n] + gam_scan[n];
   st->n_out = n_out;
   if (n_out_dev) *n_out_dev = n_out;
@@ -196,6 +200,7 @@ template <typename T>
 __global__ void k_survivors(int64_t n, StateT<T> in, StateT<T> out, const uint8_t *flag,
                             const int32_t *owner, const long long *keep_scan,
                             const int32_t *gam, int32_t *old2new, const DevStatus *st) {
+  pdl_sync();
   const bool skip = st->remap_scratch[0] != 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -243,6 +248,7 @@ __global__ void k_to2d(StateT<T> in, StateT<T> out, const int32_t *owner,
                        const long long *keep_scan, const long long *row_ptr, const int32_t *col,
                        const DevStatus *st, const int32_t *flagged,
                        const unsigned long long *n_flagged) {
+  pdl_sync();
   if (st->remap_scratch[0] != 0) return;
   const int lane = threadIdx.x & 31;
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -314,6 +320,7 @@ template <typename T>
 __global__ void k_append(int64_t n, StateT<T> in, StateT<T> out, const int32_t *gam,
                          const long long *keep_scan, const long long *gam_scan,
                          const DevStatus *st) {
+  pdl_sync();
   if (st->remap_scratch[0] != 0) return;
   const long long n_keep = keep_scan[n];
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -361,13 +368,13 @@ static int remap_t(mafp_ctx *ctx, int64_t n, const mafp_state *in_, const uint8_
   unsigned long long *counts = reinterpret_cast<unsigned long long *>(ctx->d_status->remap_scratch + 1);
   MAFP_CUDA_TRY(ctx, cudaMemsetAsync(counts, 0, 2 * sizeof(*counts), s));
   MAFP_TIMED(ctx, s, "k_owner_seed<T>",
-             k_owner_seed<T><<<grid_for(n, 256, sms * 16), 256, 0, s>>>(
+             launch(k_owner_seed<T>, grid_for(n, 256, sms * 16), 256, 0, s, 
                  n, in, flag, owner, keep, gam, ctx->prm.c_psi, flagged, counts));
   MAFP_TIMED(ctx, s, "k_owner_mark",
-             k_owner_mark<<<grid_for(n * 32, 256, sms * 8), 256, 0, s>>>(
+             launch(k_owner_mark, grid_for(n * 32, 256, sms * 8), 256, 0, s, 
                  in.model, in.type, rp, col, owner, flagged, counts, cand, counts + 1));
   MAFP_TIMED(ctx, s, "k_owner<T>",
-             k_owner<T><<<grid_for(n * 32, 256, sms * 8), 256, 0, s>>>(in, flag, rp, col, owner,
+             launch(k_owner<T>, grid_for(n * 32, 256, sms * 8), 256, 0, s, in, flag, rp, col, owner,
                                                                        keep, cand, counts + 1));
   MAFP_LAUNCH_CHECK(ctx);
   int rc = scan_i32_to_i64(ctx, keep, keep_scan, n, s);
@@ -375,15 +382,15 @@ static int remap_t(mafp_ctx *ctx, int64_t n, const mafp_state *in_, const uint8_
   rc = scan_i32_to_i64(ctx, gam, gam_scan, n, s);
   if (rc) return rc;
   MAFP_TIMED(ctx, s, "k_remap_count",
-             k_remap_count<<<1, 1, 0, s>>>(keep_scan, gam_scan, n, cap_out, n_out_dev, ctx->d_status));
+             launch(k_remap_count, 1, 1, 0, s, keep_scan, gam_scan, n, cap_out, n_out_dev, ctx->d_status));
   MAFP_TIMED(ctx, s, "k_survivors<T>",
-             k_survivors<T><<<grid_for(n, 256, sms * 16), 256, 0, s>>>(n, in, out, flag, owner, keep_scan,
+             launch(k_survivors<T>, grid_for(n, 256, sms * 16), 256, 0, s, n, in, out, flag, owner, keep_scan,
                                                              gam, old2new, ctx->d_status));
   MAFP_TIMED(ctx, s, "k_to2d<T>",
-             k_to2d<T><<<grid_for(n * 32, 256, sms * 8), 256, 0, s>>>(
+             launch(k_to2d<T>, grid_for(n * 32, 256, sms * 8), 256, 0, s, 
                  in, out, owner, keep_scan, rp, col, ctx->d_status, flagged, counts));
   MAFP_TIMED(ctx, s, "k_append<T>",
-             k_append<T><<<grid_for(n, 256, sms * 16), 256, 0, s>>>(n, in, out, gam, keep_scan, gam_scan,
+             launch(k_append<T>, grid_for(n, 256, sms * 16), 256, 0, s, n, in, out, gam, keep_scan, gam_scan,
                                                           ctx->d_status));
   MAFP_LAUNCH_CHECK(ctx);
   return MAFP_OK;

@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const int32_t *in, long l
                                                        unsigned long long *state, int *ctr,
                                                        DevStatus *st, long long wait_limit,
                                                        const int32_t *wanted) {
+  pdl_sync();
   if (wanted && !*wanted) return;   // (every block alike: no ticket is taken)
   __shared__ int s_tile, s_last, s_gave_up;
   __shared__ long long s_prefix, s_red[kScanThreads / 32];
@@ -193,7 +194,7 @@ int scan_i32_to_i64(mafp_ctx *ctx, const int32_t *in, long long *out, int64_t n,
   const int64_t ntiles = (n + kScanTile - 1) / kScanTile;
   const long long limit = ctx->prm.wait_limit > 0 ? (long long)ctx->prm.wait_limit : 0;
   MAFP_TIMED(ctx, s, "k_scan",
-             k_scan<<<(unsigned)ntiles, kScanThreads, 0, s>>>(
+             launch(k_scan, (unsigned)ntiles, kScanThreads, 0, s, 
                  in, out, n, (int)ntiles, reinterpret_cast<unsigned long long *>(ctx->scan_tmp),
                  ctx->scan_ctr, ctx->d_status, limit, wanted));
   MAFP_LAUNCH_CHECK(ctx);

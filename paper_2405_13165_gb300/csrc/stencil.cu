@@ -20,7 +20,7 @@ constexpr int64_t kStFewRows = 16384, kStManyRows = 65536;
 // rows are done (1M jet cloud, 3D rows: 847 us against 925 with four warps).
 constexpr int kBuildThreads = 64;
 
-__global__ void k_reset_queue(DevStatus *st) { st->fallback_count = 0; }
+__global__ void k_reset_queue(DevStatus *st) { pdl_sync(); st->fallback_count = 0; }
 
 // Per-lane cache for the passes after the moments.  FP32: (q, w) of two entries
 // together, (q1a, q1b, q2a, q2b) and (q3a, q3b, wa, wb), KC entries per lane (176
@@ -551,6 +551,7 @@ __global__ void __launch_bounds__(kBuildThreads, sizeof(C) == 4 ? (M == 10 ? 7 :
     int64_t n, const vec4_t<TS> *pos, const uint8_t *model, const vec4_t<TS> *frame,
     const long long *row_ptr, const int32_t *col, vec4_t<TS> *coef, uint8_t *status,
     float *cond, StParams<C> sp, DevStatus *st, int32_t *queue, int rounds) {
+  pdl_sync();
   constexpr int SMG = StSmem<M, G>::PER_GROUP, KC = StCache<C, M, G>::KC, ROWS = 32 / G;
   extern __shared__ __align__(16) unsigned char st_smem[];
   C *sm = reinterpret_cast<C *>(st_smem + StCache<C, M, G>::BYTES) + threadIdx.x / G * SMG;
@@ -598,6 +599,7 @@ __global__ void __launch_bounds__(kBuildThreads) k_stencil_redo(
     const float4 *pos, const uint8_t *model, const float4 *frame, const long long *row_ptr,
     const int32_t *col, float4 *coef, uint8_t *status, float *cond, StParams<double> sp,
     DevStatus *st, const int32_t *queue) {
+  pdl_sync();
   constexpr int NA = Basis<M>::NA, NR = Basis<M>::NR;
   constexpr int SMG = StSmem<M, G>::PER_GROUP;
   __shared__ double smem[(kBuildThreads / G) * SMG];
@@ -643,7 +645,7 @@ static void launch_stencil(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void 
     cudaFuncSetAttribute(k_stencil<TS, C, M, G, REFINE>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   MAFP_TIMED(ctx, s, name.s,
-             k_stencil<TS, C, M, G, REFINE><<<blocks, kBuildThreads, smem, s>>>(
+             launch(k_stencil<TS, C, M, G, REFINE>, blocks, kBuildThreads, smem, s, 
                  n, (const V *)pos_h, model, (const V *)frame, rp, col, (V *)coef, status, cond,
                  sp, ctx->d_status, ctx->fallback, rounds));
 }
@@ -691,7 +693,7 @@ int build_stencils(mafp_ctx *ctx, int64_t n, int32_t dtype, const void *pos_h,
   }
   const StParams<float> sp = make_params<float>(ctx->prm, 1e-6);
   const StParams<double> sp64 = make_params<double>(ctx->prm, 1e-12);
-  MAFP_TIMED(ctx, s, "k_reset_queue", k_reset_queue<<<1, 1, 0, s>>>(ctx->d_status));
+  MAFP_TIMED(ctx, s, "k_reset_queue", launch(k_reset_queue, 1, 1, 0, s, ctx->d_status));
   int rc = dtype == MAFP_F32_PLAIN
                ? dispatch_stencils<float, float, false>(ctx, s, n, pos_h, model, frame, rp,
                                                              col, coef, status, cond, sp)
@@ -701,11 +703,11 @@ int build_stencils(mafp_ctx *ctx, int64_t n, int32_t dtype, const void *pos_h,
   // FP64 redo: small groups keep the per-particle factorisation, repeated in
   // every lane of a group, from dominating the slow FP64 pipe
   MAFP_TIMED(ctx, s, "k_stencil_redo<10,4>",
-             k_stencil_redo<10, 4><<<sms * 64, kBuildThreads, 0, s>>>(
+             launch(k_stencil_redo<10, 4>, sms * 64, kBuildThreads, 0, s, 
       (const float4 *)pos_h, model, (const float4 *)frame, rp, col, (float4 *)coef, status, cond,
       sp64, ctx->d_status, ctx->fallback));
   MAFP_TIMED(ctx, s, "k_stencil_redo<6,4>",
-             k_stencil_redo<6, 4><<<sms * 64, kBuildThreads, 0, s>>>(
+             launch(k_stencil_redo<6, 4>, sms * 64, kBuildThreads, 0, s, 
       (const float4 *)pos_h, model, (const float4 *)frame, rp, col, (float4 *)coef, status, cond,
       sp64, ctx->d_status, ctx->fallback));
   MAFP_LAUNCH_CHECK(ctx);

@@ -362,6 +362,7 @@ __global__ void __launch_bounds__(kStThreads, sizeof(C) == 4 ? (M == 10 ? 3 : 4)
     int64_t n, const vec4_t<TS> *pos, const uint8_t *model, const vec4_t<TS> *frame,
     const long long *row_ptr, const int32_t *col, const vec4_t<TS> *fields,
     const vec4_t<TS> *gout, TS *gpos, StParams<C> sp, DevStatus *st, int32_t *queue) {
+  pdl_sync();
   constexpr int SMG = StSmem<M, G>::PER_GROUP;
   // 3D rows stream their neighbours through a shared-memory ring (measured on
   // the 1M jet cloud: 1.41 -> 1.34 ms with 2 entries in flight; 1.50 / 1.34 /
@@ -390,6 +391,7 @@ __global__ void __launch_bounds__(kStThreads) k_stencil_grad_redo(
     const float4 *pos, const uint8_t *model, const float4 *frame, const long long *row_ptr,
     const int32_t *col, const float4 *fields, const float4 *gout, float *gpos,
     StParams<double> sp, const DevStatus *st, const int32_t *queue) {
+  pdl_sync();
   constexpr int SMG = StSmem<M, G>::PER_GROUP;
   __shared__ double smem[(kStThreads / G) * SMG];
   double *sm = smem + (threadIdx.x / G) * SMG;
@@ -405,7 +407,7 @@ __global__ void __launch_bounds__(kStThreads) k_stencil_grad_redo(
   }
 }
 
-__global__ void k_reset_grad_queue(DevStatus *st) { st->fallback_count = 0; }
+__global__ void k_reset_grad_queue(DevStatus *st) { pdl_sync(); st->fallback_count = 0; }
 
 template <typename TS, typename C, int M, int G, bool QUEUE>
 static void launch_grad_g(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void *pos_h,
@@ -416,8 +418,8 @@ static void launch_grad_g(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void *
   static const KernelName name("k_stencil_grad<%s,M=%d,G=%d>", sizeof(TS) == 4 ? "f32" : "f64",
                                M, G);
   MAFP_TIMED(ctx, s, name.s,
-             (k_stencil_grad<TS, C, M, G, QUEUE><<<grid_for(n * G, kStThreads, sm_count() * 64),
-                                                   kStThreads, 0, s>>>(
+             (launch(k_stencil_grad<TS, C, M, G, QUEUE>, grid_for(n * G, kStThreads, sm_count() * 64),
+                                                   kStThreads, 0, s, 
                  n, (const V *)pos_h, model, (const V *)frame, rp, col, (const V *)fields,
                  (const V *)gout, (TS *)gpos, sp, ctx->d_status, ctx->fallback)));
 }
@@ -468,18 +470,18 @@ int build_stencils_backward(mafp_ctx *ctx, int64_t n, int32_t dtype, const void 
     MAFP_LAUNCH_CHECK(ctx);
     return MAFP_OK;
   }
-  MAFP_TIMED(ctx, s, "k_reset_grad_queue", k_reset_grad_queue<<<1, 1, 0, s>>>(ctx->d_status));
+  MAFP_TIMED(ctx, s, "k_reset_grad_queue", launch(k_reset_grad_queue, 1, 1, 0, s, ctx->d_status));
   launch_grad<float, float, true>(ctx, s, n, pos_h, model, frame, rp, col, fields, gout, gpos,
                                   make_params<float>(ctx->prm, 1e-6));
   const StParams<double> sp64 = make_params<double>(ctx->prm, 1e-12);
   const int sms = sm_count();
   MAFP_TIMED(ctx, s, "k_stencil_grad_redo<10>",
-             (k_stencil_grad_redo<10, 8><<<sms * 16, kStThreads, 0, s>>>(
+             (launch(k_stencil_grad_redo<10, 8>, sms * 16, kStThreads, 0, s, 
                  (const float4 *)pos_h, model, (const float4 *)frame, rp, col,
                  (const float4 *)fields, (const float4 *)gout, (float *)gpos, sp64,
                  ctx->d_status, ctx->fallback)));
   MAFP_TIMED(ctx, s, "k_stencil_grad_redo<6>",
-             (k_stencil_grad_redo<6, 8><<<sms * 4, kStThreads, 0, s>>>(
+             (launch(k_stencil_grad_redo<6, 8>, sms * 4, kStThreads, 0, s, 
                  (const float4 *)pos_h, model, (const float4 *)frame, rp, col,
                  (const float4 *)fields, (const float4 *)gout, (float *)gpos, sp64,
                  ctx->d_status, ctx->fallback)));
