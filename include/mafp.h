@@ -120,7 +120,7 @@ void mafp_default_params(mafp_params *p);
 /* Create a context for clouds of up to cap_particles particles whose
  * neighbour grid has up to cap_cells cells (the cell edge grows beyond max h
  * when the bounding box would need more).  Allocates all device scratch
- * (about 60 bytes per particle + 8 bytes per cell) on the current device.
+ * (about 460 bytes per particle + 8 bytes per cell) on the current device.
  * params may be NULL (defaults).  Returns MAFP_OK and *out, or MAFP_EINVAL /
  * MAFP_ECUDA. */
 int mafp_create(mafp_ctx **out, const mafp_params *params, int64_t cap_particles,

@@ -412,6 +412,83 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
   }
 }
 
+// The whole sort of a small cloud in one block: the passes that its number of cells
+// needs, each a histogram, a scan of it and a stable scatter in chunks of 1024.
+// (Eight launches less; a launch costs the host ~3 us, which bounds the step of a
+// cloud of a few thousand particles.)  The result is in keys_b / vals_b.
+constexpr int64_t kSmallSort = 8192;
+__global__ void __launch_bounds__(1024) k_sort_small(uint32_t *keys_a, int32_t *vals_a,
+                                                     uint32_t *keys_b, int32_t *vals_b, int n,
+                                                     const GridDev *g, const DevStatus *st) {
+  pdl_sync();
+  if (!g->ok || !st->not_identity) return;
+  __shared__ int32_t base[256], wcnt[32][256];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  const unsigned long long top = (unsigned long long)(g->ncells - 1);
+  uint32_t *kin = keys_a, *kout = keys_b;
+  int32_t *vin = vals_a, *vout = vals_b;
+  for (int shift = 0; shift == 0 || (shift < 32 && (top >> shift) != 0); shift += 8) {
+    if (tid < 256) base[tid] = 0;
+    __syncthreads();
+    for (int k = tid; k < n; k += 1024) atomicAdd(&base[(kin[k] >> shift) & 255u], 1);
+    __syncthreads();
+    if (w == 0) {   // exclusive scan, eight digits per lane
+      int c[8], sum = 0;
+      for (int k = 0; k < 8; ++k) {
+        c[k] = base[8 * lane + k];
+        sum += c[k];
+      }
+      int inc = sum;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += u;
+      }
+      int run = inc - sum;
+      for (int k = 0; k < 8; ++k) {
+        base[8 * lane + k] = run;
+        run += c[k];
+      }
+    }
+    for (int k0 = 0; k0 < n; k0 += 1024) {
+      for (int k = tid; k < 32 * 256; k += 1024) (&wcnt[0][0])[k] = 0;
+      __syncthreads();
+      const int k = k0 + tid;
+      const bool valid = k < n;
+      const uint32_t key = valid ? kin[k] : 0u;
+      const int32_t val = valid ? vin[k] : 0;
+      const int d = valid ? (int)((key >> shift) & 255u) : 256;
+      const unsigned peers = __match_any_sync(0xffffffffu, d);
+      const int rank = __popc(peers & lt);
+      if (valid && rank == 0) wcnt[w][d] = __popc(peers);
+      __syncthreads();
+      int total = 0;
+      if (tid < 256)
+        for (int ww = 0; ww < 32; ++ww) {
+          const int t = wcnt[ww][tid];
+          wcnt[ww][tid] = total;
+          total += t;
+        }
+      __syncthreads();
+      if (valid) {
+        const int p = base[d] + wcnt[w][d] + rank;
+        kout[p] = key;
+        vout[p] = val;
+      }
+      __syncthreads();
+      if (tid < 256) base[tid] += total;
+    }
+    __syncthreads();   // (the block's own writes are read in the next pass)
+    uint32_t *tk = kin; kin = kout; kout = tk;
+    int32_t *tv = vin; vin = vout; vout = tv;
+  }
+  if (kin != keys_b)
+    for (int k = tid; k < n; k += 1024) {
+      keys_b[k] = kin[k];
+      vals_b[k] = vin[k];
+    }
+}
+
 // --------------------------------------------------------- cell ranges
 // Occupied cells go to the work queue in two groups, the ones holding at least
 // kBigCell particles (3D cells at the usual h / dx) ahead of the rest, so the
@@ -577,16 +654,6 @@ __global__ void __launch_bounds__(kNbrThreads) k_nbr(
     }
     __syncthreads();
   }
-}
-
-__global__ void k_check_nnz(const long long *row_ptr, int64_t n, long long cap_nnz,
-                            int64_t *nnz_dev, DevStatus *st, const GridDev *g) {
-  pdl_sync();
-  if (!g->ok) return;
-  long long nnz = row_ptr[n];
-  st->nnz = nnz;
-  if (nnz_dev) *nnz_dev = nnz;
-  if (nnz > cap_nnz) set_error(st, MAFP_ECAPACITY, nnz);
 }
 
 // ------------------------------------------------ warp-per-cell mask path
@@ -996,11 +1063,17 @@ __global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
 __global__ void __launch_bounds__(kFillThreads) k_nbr_fill(
     const GridDev *all, const int32_t *table, int32_t *n_ucell, const int32_t *svals,
     const uint32_t *mask, Split split, const long long *row_ptr, int32_t *col, long long cap_nnz,
-    int64_t n) {
+    int64_t n, int64_t *nnz_dev, DevStatus *st) {
   pdl_sync();
   __shared__ __align__(16) uint2 srec[kFillWarps][32][kFillRec];     // (hit word, place)
   if (!all->ok) return;
-  if (row_ptr[n] > cap_nnz) return;
+  const long long nnz = row_ptr[n];
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st->nnz = nnz;
+    if (nnz_dev) *nnz_dev = nnz;
+    if (nnz > cap_nnz) set_error(st, MAFP_ECAPACITY, nnz);
+  }
+  if (nnz > cap_nnz) return;
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u, bit = 1u << lane;
   uint2(*wr)[kFillRec] = srec[threadIdx.x >> 5];
@@ -1234,7 +1307,14 @@ static int sort_into_cells_t(mafp_ctx *ctx, int64_t n, int nb, const long long *
   uint32_t *kin = ctx->keys_a, *kout = ctx->keys_b;
   int32_t *vin = ctx->vals_a, *vout = ctx->vals_b;
   long long *offs = reinterpret_cast<long long *>(ctx->remap_i64);
-  for (int p = 0; p < ctx->radix_passes; ++p) {
+  if (n <= kSmallSort) {
+    MAFP_TIMED(ctx, s, "k_sort_small",
+               launch(k_sort_small, 1, 1024, 0, s, kin, vin, kout, vout, (int)n, ctx->d_grid,
+                      ctx->d_status));
+    std::swap(kin, kout);
+    std::swap(vin, vout);
+  }
+  for (int p = 0; n > kSmallSort && p < ctx->radix_passes; ++p) {
     if (p > 0)
       MAFP_TIMED(ctx, s, "k_radix_hist",
                  launch(k_radix_hist, tiles, kRadixThreads, 0, s, kin, n, 8 * p, ctx->radix_hist,
@@ -1297,12 +1377,13 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
   MAFP_LAUNCH_CHECK(ctx);
   int rc = scan_i32_to_i64(ctx, ctx->counts, reinterpret_cast<long long *>(row_ptr), n, s);
   if (rc) return rc;
-  MAFP_TIMED(ctx, s, "k_check_nnz",
-             launch(k_check_nnz, 1, 1, 0, s, rp, n, cap_nnz, nnz_dev, ctx->d_status, ctx->d_grid));
+  // (launched plainly: set up beside the scan's last blocks, the persistent blocks
+  // share the SMs out unevenly, 683 against 663 us for the 200k-particle search)
   MAFP_TIMED(ctx, s, "k_nbr_fill",
-             launch(k_nbr_fill, sms * 8, kFillThreads, 0, s, ctx->d_grid, ctx->cell_table,
+             k_nbr_fill<<<sms * 8, kFillThreads, 0, s>>>(ctx->d_grid, ctx->cell_table,
                                                          ctx->n_ucell, vin, ctx->nbr_mask, split,
-                                                         rp, col, cap_nnz, n));
+                                                         rp, col, cap_nnz, n, nnz_dev,
+                                                         ctx->d_status));
   MAFP_TIMED(ctx, s, "k_nbr<T,true>(overflow cells)",
              launch(k_nbr<T, true>, nbr_blocks, kNbrThreads, kNbrSmemBytes, s, 
                  ctx->d_grid, ctx->cell_table, ctx->overflow, n_overflow, spos, vin, ctx->counts,

@@ -593,18 +593,14 @@ __global__ void __launch_bounds__(kBuildThreads, sizeof(C) == 4 ? (M == 10 ? 7 :
   }
 }
 
-// FP64 redo of the queued particles of one model (FP32 storage).
+// FP64 redo of the queued particles (FP32 storage), 3D and film by turns.
 template <int M, int G>
-__global__ void __launch_bounds__(kBuildThreads) k_stencil_redo(
-    const float4 *pos, const uint8_t *model, const float4 *frame, const long long *row_ptr,
-    const int32_t *col, float4 *coef, uint8_t *status, float *cond, StParams<double> sp,
-    DevStatus *st, const int32_t *queue) {
-  pdl_sync();
-  constexpr int NA = Basis<M>::NA, NR = Basis<M>::NR;
-  constexpr int SMG = StSmem<M, G>::PER_GROUP;
-  __shared__ double smem[(kBuildThreads / G) * SMG];
-  const int grp = threadIdx.x / G;
-  double *sm = smem + grp * SMG;
+__device__ __forceinline__ void stencil_redo(const float4 *pos, const uint8_t *model,
+                                             const float4 *frame, const long long *row_ptr,
+                                             const int32_t *col, float4 *coef, uint8_t *status,
+                                             float *cond, const StParams<double> &sp,
+                                             DevStatus *st, const int32_t *queue, double *smem) {
+  double *sm = smem + threadIdx.x / G * StSmem<M, G>::PER_GROUP;
   const int lane = threadIdx.x & (G - 1);
   const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
   const int64_t ngroups = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -623,6 +619,19 @@ __global__ void __launch_bounds__(kBuildThreads) k_stencil_redo(
       else inc_ll(&st->n_fp64_stencil);
     }
   }
+}
+
+constexpr int kRedoG = 4;   // small groups: the factorisation is repeated in every lane
+__global__ void __launch_bounds__(kBuildThreads) k_stencil_redo(
+    const float4 *pos, const uint8_t *model, const float4 *frame, const long long *row_ptr,
+    const int32_t *col, float4 *coef, uint8_t *status, float *cond, StParams<double> sp,
+    DevStatus *st, const int32_t *queue) {
+  pdl_sync();
+  static_assert(StSmem<6, kRedoG>::PER_GROUP <= StSmem<10, kRedoG>::PER_GROUP, "film fits");
+  __shared__ double smem[(kBuildThreads / kRedoG) * StSmem<10, kRedoG>::PER_GROUP];
+  stencil_redo<10, kRedoG>(pos, model, frame, row_ptr, col, coef, status, cond, sp, st, queue, smem);
+  __syncthreads();   // the scratch is laid out anew
+  stencil_redo<6, kRedoG>(pos, model, frame, row_ptr, col, coef, status, cond, sp, st, queue, smem);
 }
 
 
@@ -700,16 +709,10 @@ int build_stencils(mafp_ctx *ctx, int64_t n, int32_t dtype, const void *pos_h,
                : dispatch_stencils<float, float, true>(ctx, s, n, pos_h, model, frame, rp,
                                                             col, coef, status, cond, sp);
   if (rc) return rc;
-  // FP64 redo: small groups keep the per-particle factorisation, repeated in
-  // every lane of a group, from dominating the slow FP64 pipe
-  MAFP_TIMED(ctx, s, "k_stencil_redo<10,4>",
-             launch(k_stencil_redo<10, 4>, sms * 64, kBuildThreads, 0, s, 
-      (const float4 *)pos_h, model, (const float4 *)frame, rp, col, (float4 *)coef, status, cond,
-      sp64, ctx->d_status, ctx->fallback));
-  MAFP_TIMED(ctx, s, "k_stencil_redo<6,4>",
-             launch(k_stencil_redo<6, 4>, sms * 64, kBuildThreads, 0, s, 
-      (const float4 *)pos_h, model, (const float4 *)frame, rp, col, (float4 *)coef, status, cond,
-      sp64, ctx->d_status, ctx->fallback));
+  MAFP_TIMED(ctx, s, "k_stencil_redo",
+             launch(k_stencil_redo, sms * 8, kBuildThreads, 0, s, (const float4 *)pos_h, model,
+                    (const float4 *)frame, rp, col, (float4 *)coef, status, cond, sp64,
+                    ctx->d_status, ctx->fallback));
   MAFP_LAUNCH_CHECK(ctx);
   return MAFP_OK;
 }
