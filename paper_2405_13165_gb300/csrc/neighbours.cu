@@ -288,8 +288,9 @@ __device__ __forceinline__ uint32_t cell_key(const vec4_t<T> &p, int b, const Cl
   return (uint32_t)cg.cell_base[b] + (cz * (uint32_t)g.dim[1] + cy) * (uint32_t)g.dim[0] + cx;
 }
 
-// One block per radix tile: the particles' cell keys, the tile's histogram of the
-// first digit, and whether a key is below the one before it.  Clouds that are in
+// One block per radix tile (blocks beyond the tiles only help to clear the cells, of
+// which a small sparse cloud has many more): the particles' cell keys, the tile's
+// histogram of the first digit, and whether a key is below the one before it.  Clouds that are in
 // cell order already (a time loop keeps them so) show it here, and the sort's
 // passes and their scans are left out (100 us on the 1M jet cloud).  All blocks
 // together also clear the cells and the work counters.
@@ -307,6 +308,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_hash(const vec4_t<T> *pos, in
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   cnt[tid] = 0;
   const int64_t base = (int64_t)blockIdx.x * kRadixTile;
+  const bool tile = blockIdx.x < tiles;
   uint32_t key[kRadixItems];
 #pragma unroll
   for (int c = 0; c < kRadixItems; ++c) {
@@ -322,7 +324,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_hash(const vec4_t<T> *pos, in
   // the key before the tile's first one
   if (tid == 0)
     last[kRadixItems][0] =
-        base > 0 ? cell_key<T>(ld4(pos + base - 1), cg.nb > 1 ? cloud_id[base - 1] : 0, cg) : 0u;
+        base > 0 && tile ? cell_key<T>(ld4(pos + base - 1), cg.nb > 1 ? cloud_id[base - 1] : 0, cg) : 0u;
   __syncthreads();
   bool out_of_order = false;
 #pragma unroll
@@ -338,7 +340,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_hash(const vec4_t<T> *pos, in
     st->not_identity = 1;
     st->cells_identity = 0;
   }
-  hist[(int64_t)tid * tiles + blockIdx.x] = cnt[tid];
+  if (tile) hist[(int64_t)tid * tiles + blockIdx.x] = cnt[tid];
   // the cells and the work counters (cell counts, overflow cells, the tickets of the
   // mask and fill kernels and the mask pool's counter)
   const long long nc = cg.all->ncells;
@@ -1299,7 +1301,7 @@ static int sort_into_cells_t(mafp_ctx *ctx, int64_t n, int nb, const long long *
   CloudGrids cg{ctx->d_grids, ctx->cell_base, nb, ctx->d_grid};
   const int tiles = (int)((n + kRadixTile - 1) / kRadixTile);
   MAFP_TIMED(ctx, s, "k_hash",
-             launch(k_hash<T>, tiles, kRadixThreads, 0, s, pos, n, ctx->cloud_id, cg, ctx->keys_a,
+             launch(k_hash<T>, std::max(tiles, 2 * sms), kRadixThreads, 0, s, pos, n, ctx->cloud_id, cg, ctx->keys_a,
                                                        ctx->vals_a, ctx->radix_hist, tiles,
                                                        ctx->cell_start, ctx->cell_end,
                                                        ctx->n_ucell, ctx->d_status));
