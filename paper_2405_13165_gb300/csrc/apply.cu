@@ -196,12 +196,15 @@ static void launch_apply(mafp_ctx *ctx, cudaStream_t s, int64_t n, const long lo
   constexpr int U = sizeof(T) == 4 ? 8 : 1;
   const V *c = (const V *)coef, *f = (const V *)fields;
   T *o = (T *)out;
+  // Launched plainly: set up early, its blocks join an SM that still runs the kernel
+  // before it, and keep that kernel's division into shared memory and L1.  Behind a trial FP64
+  // redo with 5 resident blocks per SM (small L1) the 1M jet step took 2616 us, 1948 so.
   if (G == 4) {
-    MAFP_TIMED(ctx, s, "k_apply<G=4>", launch(k_apply<T, 4, U>, blocks, kApThreads, 0, s, n, rp, col, c, f, o));
+    MAFP_TIMED(ctx, s, "k_apply<G=4>", (k_apply<T, 4, U><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, f, o)));
   } else if (G == 16) {
-    MAFP_TIMED(ctx, s, "k_apply<G=16>", launch(k_apply<T, 16, U>, blocks, kApThreads, 0, s, n, rp, col, c, f, o));
+    MAFP_TIMED(ctx, s, "k_apply<G=16>", (k_apply<T, 16, U><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, f, o)));
   } else {
-    MAFP_TIMED(ctx, s, "k_apply<G=8>", launch(k_apply<T, 8, U>, blocks, kApThreads, 0, s, n, rp, col, c, f, o));
+    MAFP_TIMED(ctx, s, "k_apply<G=8>", (k_apply<T, 8, U><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, f, o)));
   }
 }
 

@@ -193,11 +193,11 @@ __device__ __forceinline__ void inc_ll(long long *p, long long v = 1) {
 
 template <typename T> __device__ __forceinline__ bool finite_(T x) { return isfinite(x); }
 
-// Launch helpers.  Every kernel is launched with programmatic stream serialization
-// and begins with pdl_sync(): its blocks may be set up as soon as all blocks of the
-// kernel before it have started, and wait there until that kernel is done and its
-// writes are visible.  Nothing is read or written before the wait, so the order of
-// the calls is that of plain launches, without the gap between them.
+// Launch helpers.  Kernels are launched with programmatic stream serialization
+// (k_nbr_fill and k_apply plainly) and begin with pdl_sync(): their blocks may be set
+// up as soon as all blocks of the kernel before have started, and wait there until that
+// kernel is done and its writes are visible.  Nothing is read or written before the
+// wait, so the order of the calls is that of plain launches, without the gap between.
 __device__ __forceinline__ void pdl_sync() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
