@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(kApThreads) k_apply(int64_t n, const long long
                                                       const int32_t *col,
                                                       const vec4_t<T> *coef,
                                                       const vec4_t<T> *fields, T *out) {
-  pdl_sync();
+  pdl_wait();
   using V = vec4_t<T>;
   const int lane = threadIdx.x & (G - 1);
   const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kApThreads) k_apply_T(int64_t n, const long lo
                                                         const vec4_t<T> *coef,
                                                         const vec4_t<T> *gout,
                                                         vec4_t<T> *gfields) {
-  pdl_sync();
+  pdl_wait();
   using V = vec4_t<T>;
   const int lane = threadIdx.x & (G - 1);
   const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kApThreads) k_apply_T(int64_t n, const long lo
     for (int k = 0; k < (G < 4 ? 4 : G); ++k) acc[k] = T(0);
     V csum = mk4<T>(0, 0, 0, 0);
     for (long long e = b + lane; e < e1; e += G) {
-      const int i = __ldg(col + e);
+      const int i = col[e];
       const long long ei = row_ptr[i] + tloc[e];
       const V c = ld4(coef + ei);
       const V cs = ld4(coef + e);
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kApThreads) k_apply_T_scatter(int64_t n,
                                                                 const vec4_t<T> *coef,
                                                                 const vec4_t<T> *gout,
                                                                 vec4_t<T> *gfields) {
-  pdl_sync();
+  pdl_wait();
   using V = vec4_t<T>;
   const int lane = threadIdx.x & (G - 1);
   const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kApThreads) k_apply_T_scatter(int64_t n,
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const bool in = e + u * G < e1;
-        j[u] = in ? __ldg(col + e + u * G) : -1;
+        j[u] = in ? col[e + u * G] : -1;
         c[u] = in ? ld4(coef + e + u * G) : mk4<T>(0, 0, 0, 0);
       }
 #pragma unroll

@@ -47,7 +47,7 @@ __global__ void k_select_total(const long long *off, int64_t n, int64_t base, lo
 template <typename T>
 __global__ void k_ghost_seed(int64_t n, StateT<T> in, const uint8_t *src, const long long *off,
                              StateT<T> g, uint8_t *gflag, int32_t *gsrc, const DevStatus *st) {
-  pdl_sync();
+  pdl_wait();
   if (st->remap_scratch[1] != 0) return;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -64,7 +64,7 @@ __global__ void k_ghost_seed(int64_t n, StateT<T> in, const uint8_t *src, const 
 template <typename T>
 __global__ void k_ghost_append(int64_t ng, StateT<T> gf, const long long *off, StateT<T> all,
                                int64_t base, const DevStatus *st) {
-  pdl_sync();
+  pdl_wait();
   if (st->remap_scratch[1] != 0) return;
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < ng;
        g += (int64_t)gridDim.x * blockDim.x) {

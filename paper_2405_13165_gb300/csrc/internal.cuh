@@ -194,12 +194,20 @@ __device__ __forceinline__ void inc_ll(long long *p, long long v = 1) {
 template <typename T> __device__ __forceinline__ bool finite_(T x) { return isfinite(x); }
 
 // Launch helpers.  Kernels are launched with programmatic stream serialization
-// (k_nbr_fill and k_apply plainly) and begin with pdl_sync(): their blocks may be set
-// up as soon as all blocks of the kernel before have started, and wait there until that
-// kernel is done and its writes are visible.  Nothing is read or written before the
-// wait, so the order of the calls is that of plain launches, without the gap between.
-__device__ __forceinline__ void pdl_sync() {
+// (k_nbr_fill and k_apply plainly) and begin with pdl_sync() or pdl_wait(): their blocks
+// are set up before the kernel ahead of them is done, and wait there until it is and its
+// writes are visible.  Nothing is read or written before the wait, so the order of the
+// calls is that of plain launches, without the gap between.
+//   pdl_sync() lets the next kernel's blocks be set up as soon as all of this kernel's
+// have started.  Not for a kernel that writes 4-vectors or other real arrays: ld4 and
+// __ldg take the non-coherent path, for data that nobody writes while the reading kernel
+// is resident, and the next kernel (of this call or of any other) may read them so.
+//   pdl_wait() leaves the set-up to the end of this kernel's last block.
+__device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_sync() {
+  pdl_wait();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 

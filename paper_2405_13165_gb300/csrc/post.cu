@@ -16,7 +16,7 @@ __global__ void k_film_momentum(int64_t n, const uint8_t *model, vec4_t<T> *vp, 
                                 const T *eta, const T *hfilm, const vec4_t<T> *normal,
                                 const vec4_t<T> *out, double gx, double gy, double gz,
                                 double dt) {
-  pdl_sync();
+  pdl_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     if (model[i] != MAFP_MODEL_2D) continue;

@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(kBuildThreads, sizeof(C) == 4 ? (M == 10 ? 7 :
     int64_t n, const vec4_t<TS> *pos, const uint8_t *model, const vec4_t<TS> *frame,
     const long long *row_ptr, const int32_t *col, vec4_t<TS> *coef, uint8_t *status,
     float *cond, StParams<C> sp, DevStatus *st, int32_t *queue, int rounds) {
-  pdl_sync();
+  pdl_wait();
   constexpr int SMG = StSmem<M, G>::PER_GROUP, KC = StCache<C, M, G>::KC, ROWS = 32 / G;
   extern __shared__ __align__(16) unsigned char st_smem[];
   C *sm = reinterpret_cast<C *>(st_smem + StCache<C, M, G>::BYTES) + threadIdx.x / G * SMG;
@@ -626,7 +626,7 @@ __global__ void __launch_bounds__(kBuildThreads) k_stencil_redo(
     const float4 *pos, const uint8_t *model, const float4 *frame, const long long *row_ptr,
     const int32_t *col, float4 *coef, uint8_t *status, float *cond, StParams<double> sp,
     DevStatus *st, const int32_t *queue) {
-  pdl_sync();
+  pdl_wait();
   static_assert(StSmem<6, kRedoG>::PER_GROUP <= StSmem<10, kRedoG>::PER_GROUP, "film fits");
   __shared__ double smem[(kBuildThreads / kRedoG) * StSmem<10, kRedoG>::PER_GROUP];
   stencil_redo<10, kRedoG>(pos, model, frame, row_ptr, col, coef, status, cond, sp, st, queue, smem);

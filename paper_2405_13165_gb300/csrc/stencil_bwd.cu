@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(kStThreads, sizeof(C) == 4 ? (M == 10 ? 3 : 4)
     int64_t n, const vec4_t<TS> *pos, const uint8_t *model, const vec4_t<TS> *frame,
     const long long *row_ptr, const int32_t *col, const vec4_t<TS> *fields,
     const vec4_t<TS> *gout, TS *gpos, StParams<C> sp, DevStatus *st, int32_t *queue) {
-  pdl_sync();
+  pdl_wait();
   constexpr int SMG = StSmem<M, G>::PER_GROUP;
   // 3D rows stream their neighbours through a shared-memory ring (measured on
   // the 1M jet cloud: 1.41 -> 1.34 ms with 2 entries in flight; 1.50 / 1.34 /
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(kStThreads) k_stencil_grad_redo(
     const float4 *pos, const uint8_t *model, const float4 *frame, const long long *row_ptr,
     const int32_t *col, const float4 *fields, const float4 *gout, float *gpos,
     StParams<double> sp, const DevStatus *st, const int32_t *queue) {
-  pdl_sync();
+  pdl_wait();
   constexpr int SMG = StSmem<M, G>::PER_GROUP;
   __shared__ double smem[(kStThreads / G) * SMG];
   double *sm = smem + (threadIdx.x / G) * SMG;
