@@ -202,7 +202,12 @@ template <typename T> __device__ __forceinline__ bool finite_(T x) { return isfi
 // have started.  Not for a kernel that writes 4-vectors or other real arrays: ld4 and
 // __ldg take the non-coherent path, for data that nobody writes while the reading kernel
 // is resident, and the next kernel (of this call or of any other) may read them so.
-//   pdl_wait() leaves the set-up to the end of this kernel's last block.
+//   pdl_wait() leaves the set-up to the end of this kernel's last block.  Also where the
+// next kernel has few blocks with work, or is bound by the FP64 pipe: set up beside a
+// kernel that still runs, its blocks pile up on the SMs that have room (the search of
+// 50000 particles in 64 cells, whose cells the warp-per-particle kernels take, in FP64
+// 509 ms behind early triggers, 190 ms so; the FP64 redo of 1630 rows 302 and 176 us; the
+// 5650-particle step, 142 us, does not change).
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

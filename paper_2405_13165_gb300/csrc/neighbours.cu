@@ -609,7 +609,7 @@ __global__ void __launch_bounds__(kNbrThreads) k_nbr(
     const GridDev *all, const int32_t *table, const int32_t *sel, const int32_t *n_sel,
     const vec4_t<T> *spos, const int32_t *svals, int32_t *counts, const long long *row_ptr,
     int32_t *col, long long cap_nnz, int64_t n) {
-  pdl_sync();
+  pdl_wait();
   using V = vec4_t<T>;
   constexpr int CAP = kNbrSmemBytes / sizeof(V);
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -956,7 +956,7 @@ template <typename T>
 __global__ void __launch_bounds__(kMaskThreads) k_nbr_mask(
     const GridDev *all, const int32_t *table, int32_t *n_ucell, const vec4_t<T> *spos,
     const int32_t *svals, int32_t *counts, uint32_t *mask, Split split) {
-  pdl_sync();
+  pdl_wait();
   using V = vec4_t<T>;
   // prepared particles (-2 u, -h/2) and |u|^2 - h^2/4; the words of 32 particles
   __shared__ float4 s_part[kMaskWarps][kMaskBlock];
@@ -1066,7 +1066,7 @@ __global__ void __launch_bounds__(kFillThreads) k_nbr_fill(
     const GridDev *all, const int32_t *table, int32_t *n_ucell, const int32_t *svals,
     const uint32_t *mask, Split split, const long long *row_ptr, int32_t *col, long long cap_nnz,
     int64_t n, int64_t *nnz_dev, DevStatus *st) {
-  pdl_sync();
+  pdl_wait();
   __shared__ __align__(16) uint2 srec[kFillWarps][32][kFillRec];     // (hit word, place)
   if (!all->ok) return;
   const long long nnz = row_ptr[n];
