@@ -76,8 +76,9 @@ struct mafp_ctx {
   mafp::GridDev *d_grids;    // [kMaxClouds] one grid per cloud
   long long *cell_base;      // [kMaxClouds + 1] first global cell of each cloud
   int32_t *cloud_id;         // [cap] cloud of every particle
-  double *cloud_partial;     // [(kMaxClouds + 16384) * 8] bounding-box partials
-  int64_t *remap_i64;       // [3 * cap + 8]
+  double *cloud_partial;     // [(kMaxClouds + 16384) * 8] bounding-box partials, then
+                             // [kMaxClouds * 8] the clouds' boxes
+  int64_t *remap_i64;       // [2 * cap + 8] (radix offsets, remap scans)
   int32_t *remap_i32;       // [5 * cap]
   char err[512];
   // kernel-level CUDA-event timing (off unless mafp_profile(ctx, 1))

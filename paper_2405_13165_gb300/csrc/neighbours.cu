@@ -12,8 +12,7 @@ namespace mafp {
 
 // ---------------------------------------------------------------- grid set-up
 constexpr int kBoxThreads = 256;
-constexpr int kBoxBlocks = 16384;   // bounding-box blocks over all clouds
-constexpr int kBoxPartsMax = 1024;  // blocks of one cloud
+constexpr int kBoxBlocks = 16384;   // bounding-box blocks over all clouds, beside one per cloud
 
 // ------------------------------------------------ several clouds, one grid each
 // Cloud b owns particles [off[b], off[b+1]) and cells [cell_base[b], cell_base[b+1])
@@ -31,7 +30,15 @@ __device__ __forceinline__ long long cloud_begin(const long long *off, int b, in
   return off ? off[b] : (b == 0 ? 0 : (long long)n);
 }
 
-// Block (b, part) reduces part `part` of cloud b: min / max of x, y, z, max h,
+// First bounding-box block of cloud b: a block per cloud and one more per `chunk`
+// particles, so that clouds of any sizes get blocks by their own size (by the mean size, a
+// cloud of 10^6 particles beside 1000 of 100 had one block, and its search took 2247 us
+// for 560).
+__device__ __forceinline__ int box_first(const long long *off, int b, int64_t n, int64_t chunk) {
+  return b + (int)(max(0LL, min(cloud_begin(off, b, n), (long long)n)) / chunk);
+}
+
+// Block box_first(b) + part reduces part `part` of cloud b: min / max of x, y, z, max h,
 // count of non-finite entries; also records each particle's cloud.  Min and
 // max are exact in the input's own type, so they are taken in it and widened
 // once per block.
@@ -43,13 +50,24 @@ __device__ __forceinline__ T hi_of(T a, T b) { return b > a ? b : a; }
 template <typename T>
 __global__ void __launch_bounds__(kBoxThreads) k_cloud_bbox(const vec4_t<T> *pos, int64_t n,
                                                             const long long *off, int nb,
-                                                            int parts, double *partial,
+                                                            int64_t chunk, double *partial,
                                                             int32_t *cloud_id) {
   pdl_sync();
-  const int b = blockIdx.x / parts, part = blockIdx.x % parts;
-  // offsets are checked in k_cloud_grid; clamping keeps every access in [0, n)
+  int b = 0;   // the last cloud that begins at or before this block, 32 looked at together
+  for (int b1 = nb; b1 - b > 1;) {
+    const int step = (b1 - b + 31) >> 5, q = b + step * (int)(threadIdx.x & 31);
+    const unsigned m = __ballot_sync(
+        0xffffffffu, q == b || (q < b1 && box_first(off, q, n, chunk) <= (int)blockIdx.x));
+    b += step * (31 - __clz(m));
+    b1 = min(b1, b + step);
+  }
+  const int part = (int)blockIdx.x - box_first(off, b, n, chunk);
+  const int parts = box_first(off, b + 1, n, chunk) - box_first(off, b, n, chunk);
+  // offsets are checked in k_cloud_grid; clamping keeps every access in [0, n), and a
+  // block that offsets out of order leave without a part reads nothing
   const long long lo = max(0LL, min(cloud_begin(off, b, n), (long long)n));
-  const long long hi = max(lo, min(cloud_begin(off, b + 1, n), (long long)n));
+  const long long hi =
+      part < 0 || part >= parts ? lo : max(lo, min(cloud_begin(off, b + 1, n), (long long)n));
   const T inf = T(INFINITY);
   T v[7] = {inf, inf, inf, -inf, -inf, -inf, T(0)};
   int bad = 0;
@@ -98,12 +116,11 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_bbox(const vec4_t<T> *pos
   }
 }
 
-// One block folds a cloud's `parts` partials and leaves the cloud's box in its
-// first partial slot.  Thread t takes value t & 7 of partials t >> 3, + 32, ...: a
-// warp reads 256 consecutive bytes, up to eight reads in flight.  (A warp per
-// cloud with a lane per partial took 22 us for 1024 partials, one latency after
-// another.)  Every thread of a block of 256 has to call it.
-__device__ __forceinline__ void fold_cloud(double *pb, int parts) {
+// One block folds a cloud's `parts` partials into its box.  Thread t takes value t & 7
+// of partials t >> 3, + 32, ...: a warp reads 256 consecutive bytes, up to eight reads
+// in flight.  (A warp per cloud with a lane per partial took 22 us for 1024 partials, one
+// latency after another.)  Every thread of a block of 256 has to call it.
+__device__ __forceinline__ void fold_cloud(const double *pb, int parts, double *box) {
   __shared__ double red[8][8];
   const int k = threadIdx.x & 7;
   const double none = k < 3 ? INFINITY : (k < 6 ? -INFINITY : 0.0);
@@ -114,17 +131,27 @@ __device__ __forceinline__ void fold_cloud(double *pb, int parts) {
   v = join(v, __shfl_xor_sync(0xffffffffu, v, 8));
   v = join(v, __shfl_xor_sync(0xffffffffu, v, 16));
   if ((threadIdx.x & 31) < 8) red[threadIdx.x >> 5][k] = v;
-  __syncthreads();   // (also: every partial is read before the first is overwritten)
+  __syncthreads();
   if (threadIdx.x < 8) {
     for (int w = 1; w < kBoxThreads / 32; ++w) v = join(v, red[w][k]);
-    pb[k] = v;
+    box[k] = v;
   }
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(kBoxThreads) k_cloud_fold(double *partial, int parts) {
+__global__ void __launch_bounds__(kBoxThreads) k_cloud_fold(const double *partial, double *box,
+                                                            const long long *off, int64_t n,
+                                                            int64_t chunk) {
   pdl_sync();
-  fold_cloud(partial + (long long)blockIdx.x * parts * 8, parts);
+  const int b = blockIdx.x, first = box_first(off, b, n, chunk);
+  const int parts = box_first(off, b + 1, n, chunk) - first;
+  partial += (long long)first * 8;
+  box += (long long)b * 8;
+  if (parts == 1) {
+    if (threadIdx.x < 8) box[threadIdx.x] = partial[threadIdx.x];
+    return;
+  }
+  fold_cloud(partial, parts, box);
 }
 
 // Cells of cloud b at edge c (>= max h of the cloud); 0 for an empty cloud.
@@ -148,9 +175,10 @@ __device__ double cloud_cells(const double v[8], double c, int dim[3]) {
 // edge of every cloud starts strictly above its max h times edge_factor >= 1
 // (so S_i lies in the 27 cells around i's cell) and grows uniformly when the
 // total exceeds cap_cells.
-__global__ void __launch_bounds__(kBoxThreads) k_cloud_grid(double *partial,
+__global__ void __launch_bounds__(kBoxThreads) k_cloud_grid(const double *partial, double *box,
                                                             const long long *off, int64_t n,
-                                                            int nb, int parts, GridDev *grids,
+                                                            int nb, int64_t chunk,
+                                                            GridDev *grids,
                                                             long long *cell_base, GridDev *all,
                                                             DevStatus *st, long long cap_cells,
                                                             double edge_factor) {
@@ -164,7 +192,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_grid(double *partial,
     s_scale = 1.0;
     s_bad = (cloud_begin(off, 0, n) != 0 || cloud_begin(off, nb, n) != n) ? 1 : 0;
   }
-  if (nb == 1) fold_cloud(partial, parts);
+  if (nb == 1) fold_cloud(partial, box_first(off, 1, n, chunk), box);
   __syncthreads();
   for (int b = threadIdx.x; b < nb; b += blockDim.x)
     if (cloud_begin(off, b + 1, n) < cloud_begin(off, b, n)) s_bad = 1;
@@ -179,7 +207,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_grid(double *partial,
     return;
   }
   for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-    const double bad = partial[(long long)b * parts * 8 + 7];
+    const double bad = box[(long long)b * 8 + 7];
     if (bad > 0.0) atomicAdd(&s_nonfinite, bad);
   }
   __syncthreads();
@@ -197,7 +225,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_grid(double *partial,
     __syncthreads();
     for (int b = threadIdx.x; b < nb; b += blockDim.x) {
       double v[8];
-      for (int k = 0; k < 8; ++k) v[k] = partial[(long long)b * parts * 8 + k];
+      for (int k = 0; k < 8; ++k) v[k] = box[(long long)b * 8 + k];
       int dim[3];
       const double c = v[6] * (1.0 + 1e-6) * edge_factor * s_scale;
       const double cells = cloud_cells(v, c, dim);
@@ -218,9 +246,9 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_grid(double *partial,
     if (threadIdx.x == 0) s_scale *= cbrt(s_cells / (double)cap_cells) * 1.0001;
     __syncthreads();
   }
-  // exclusive scan of the cell counts: thread t takes a contiguous chunk
-  const int chunk = (nb + kBoxThreads - 1) / kBoxThreads;
-  const int b0 = threadIdx.x * chunk, b1 = min(nb, b0 + chunk);
+  // exclusive scan of the cell counts: thread t takes a contiguous span
+  const int span = (nb + kBoxThreads - 1) / kBoxThreads;
+  const int b0 = threadIdx.x * span, b1 = min(nb, b0 + span);
   long long part_sum = 0;
   for (int b = b0; b < b1; ++b) part_sum += grids[b].ncells;
   s_sum[threadIdx.x] = part_sum;
@@ -241,7 +269,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_cloud_grid(double *partial,
   }
   if (threadIdx.x == 0) {
     long long acc = s_sum[kBoxThreads - 1];
-    for (int b = (kBoxThreads - 1) * chunk; b < nb; ++b) acc += grids[b].ncells;
+    for (int b = (kBoxThreads - 1) * span; b < nb; ++b) acc += grids[b].ncells;
     cell_base[nb] = acc;
     all->ok = acc <= cap_cells ? 1 : 0;
     all->ncells = acc;
@@ -1289,23 +1317,20 @@ static int sort_into_cells_t(mafp_ctx *ctx, int64_t n, int nb, const long long *
   using V = vec4_t<T>;
   const V *pos = reinterpret_cast<const V *>(pos_h);
   const int sms = sm_count();
-  // about 2048 particles per bounding-box block, two blocks per SM of one cloud
-  const int64_t want = std::min<int64_t>((n / nb + 2047) / 2048, 2 * sms);
-  const int parts = (int)std::max<int64_t>(
-      1, std::min<int64_t>(want, std::min(kBoxBlocks / std::max(nb, 1), kBoxPartsMax)));
+  // particles per bounding-box block: 2048, and at most two blocks per SM of one cloud
+  const int64_t chunk = std::max<int64_t>(2048, nb > 1 ? n / kBoxBlocks + 1 : n / (2 * sms) + 1);
+  double *box = ctx->cloud_partial + (int64_t)(kMaxClouds + kBoxBlocks) * 8;
   MAFP_TIMED(ctx, s, "k_cloud_bbox",
-             launch(k_cloud_bbox<T>, nb * parts, kBoxThreads, 0, s, pos, n, cloud_off, nb, parts,
-                                                                 ctx->cloud_partial,
-                                                                 ctx->cloud_id));
-  if (nb > 1 && parts > 1)
+             launch(k_cloud_bbox<T>, (int)(nb + n / chunk), kBoxThreads, 0, s, pos, n, cloud_off, nb,
+                    chunk, ctx->cloud_partial, ctx->cloud_id));
+  if (nb > 1)
     MAFP_TIMED(ctx, s, "k_cloud_fold",
-               launch(k_cloud_fold, nb, kBoxThreads, 0, s, ctx->cloud_partial, parts));
+               launch(k_cloud_fold, nb, kBoxThreads, 0, s, ctx->cloud_partial, box, cloud_off, n,
+                      chunk));
   MAFP_TIMED(ctx, s, "k_cloud_grid",
-             launch(k_cloud_grid, 1, kBoxThreads, 0, s, ctx->cloud_partial, cloud_off, n, nb, parts,
-                                                    ctx->d_grids,
-                                                    ctx->cell_base, ctx->d_grid, ctx->d_status,
-                                                    ctx->cap_cells,
-                                                    0.01 * (double)ctx->tune.cell_edge_pct));
+             launch(k_cloud_grid, 1, kBoxThreads, 0, s, ctx->cloud_partial, box, cloud_off, n, nb,
+                    chunk, ctx->d_grids, ctx->cell_base, ctx->d_grid, ctx->d_status,
+                    ctx->cap_cells, 0.01 * (double)ctx->tune.cell_edge_pct));
   CloudGrids cg{ctx->d_grids, ctx->cell_base, nb, ctx->d_grid};
   const int tiles = (int)((n + kRadixTile - 1) / kRadixTile);
   MAFP_TIMED(ctx, s, "k_hash",
