@@ -13,8 +13,24 @@
 namespace mafp {
 
 // Clouds of at most kStFewRows particles take the wide groups (too few rows for
-// the GPU's warps otherwise); of more than kStManyRows, four rounds per warp.
-constexpr int64_t kStFewRows = 16384, kStManyRows = 65536;
+// the GPU's warps otherwise).
+constexpr int64_t kStFewRows = 16384;
+
+// Rounds of rows per warp.  More share a warp's start and its last, partly filled round,
+// but leave the GPU idle where few warps hold rows of the model: a column of 3D rows in a
+// wide film keeps its rows in few warps.  Whole builds with 1 / 2 / 4 rounds, us --
+//   3D: jet on a film, 66k particles 85 / 102 / 129, 131k 152 / 159 / 180, 262k 296 / 291 /
+//   305, 1M 1234 / 1152 / 1146; cube 131k 270 / 267 / 288, 262k 528 / 512 / 534, 517k 1029 /
+//   1002 / 1016;
+//   film: 30k 40 / 41 / 41, 66k 64 / 59 / 63, 131k 108 / 98 / 96, 262k 198 / 178 / 172.
+// FP64 (its pipe is full with few warps, and uneven warps are its time): jet 66k 1081 /
+// 1265 / 1692, cube 134k 5774 / 5919 / 6347, film 131k 1116 / 1146 / 1149.
+template <typename C, int M>
+static int rounds_of(int64_t n) {
+  if (sizeof(C) == 8) return 1;
+  if (M == 10) return n > 196608 ? 2 : 1;
+  return n > 131072 ? 4 : (n > 65536 ? 2 : 1);
+}
 
 // Two warps per block: a block's slot is free again as soon as its two warps'
 // rows are done (1M jet cloud, 3D rows: 847 us against 925 with four warps).
@@ -643,8 +659,7 @@ static void launch_stencil(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void 
   using V = vec4_t<TS>;
   static const KernelName name("k_stencil<%s,M=%d,G=%d,%s>", sizeof(TS) == 4 ? "f32" : "f64",
                                M, G, REFINE ? "refined" : "plain");
-  // rounds of rows per warp: one while that leaves the GPU's warps without work
-  const int rounds = n > kStManyRows ? 4 : 1;
+  const int rounds = rounds_of<C, M>(n);
   static_assert(G >= 4, "a warp looks at 32 particles at most");
   const int blocks = (int)((n + (int64_t)rounds * kBuildThreads / G - 1) / (rounds * kBuildThreads / G));
   constexpr int smem = StCache<C, M, G>::SMEM;
