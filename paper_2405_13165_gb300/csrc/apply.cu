@@ -13,8 +13,12 @@ constexpr int kApThreads = 256;
 // Sec. 2.3), so this is Eq. GFDM_Definition; differencing first removes the
 // u_i * sum_j c_ij term that FP32 rounding of the coefficients leaves behind.
 // A group of G lanes per row; lanes stride over the row with U loads in flight.
+// Threads per block.  FP64 keeps few blocks resident (80 registers), and the rows of
+// one model lie side by side: blocks of half the rows share out more evenly (jet on a
+// film, FP64, 15k particles 72 -> 61 us, 30k 101 -> 81 us; cube 197k unchanged).
+template <typename T> constexpr int kApplyThreads = sizeof(T) == 4 ? 256 : 128;
 template <typename T, int G, int U>
-__global__ void __launch_bounds__(kApThreads) k_apply(int64_t n, const long long *row_ptr,
+__global__ void __launch_bounds__(kApplyThreads<T>) k_apply(int64_t n, const long long *row_ptr,
                                                       const int32_t *col,
                                                       const vec4_t<T> *coef,
                                                       const vec4_t<T> *fields, T *out) {
@@ -30,7 +34,10 @@ __global__ void __launch_bounds__(kApThreads) k_apply(int64_t n, const long long
 #pragma unroll
     for (int k = 0; k < 16; ++k) acc[k] = T(0);
     // U entries per lane in flight; past the row end the slot reads particle
-    // i itself with a zero coefficient (an exact zero contribution)
+    // i itself with a zero coefficient (an exact zero contribution).  FP64 is bound by
+    // its pipe, which such a slot would occupy like others: a warp without a second
+    // entry leaves it out (film 200k, 4 / 8 / 16 lanes: 297 / 361 / 498 us with it, 317 /
+    // 342 / 429 with one entry in flight, 284 / 313 / 407 so)
     for (long long e = b + lane; e < e1; e += U * G) {
       int j[U];
       V c[U], f[U];
@@ -42,6 +49,7 @@ __global__ void __launch_bounds__(kApThreads) k_apply(int64_t n, const long long
       for (int u = 0; u < U; ++u) f[u] = ld4(fields + j[u]);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
+        if (sizeof(T) == 8 && u > 0 && e + u * G >= e1) break;
         const T fv[4] = {f[u].x - fi.x, f[u].y - fi.y, f[u].z - fi.z, f[u].w - fi.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -190,21 +198,19 @@ static void launch_apply(mafp_ctx *ctx, cudaStream_t s, int64_t n, const long lo
                          const int32_t *col, const void *coef, const void *fields, void *out) {
   using V = vec4_t<T>;
   const int G = ctx->tune.apply_group;
-  const int blocks = grid_for(n * G, kApThreads, sm_count() * 64);
-  // entries in flight per lane; FP64 is bound by its pipe, which slots past the row's
-  // end occupy like others (60k jet cloud: two in flight 174 us, one 153 us)
-  constexpr int U = sizeof(T) == 4 ? 8 : 1;
+  const int blocks = grid_for(n * G, kApplyThreads<T>, sm_count() * 64);
+  constexpr int U = sizeof(T) == 4 ? 8 : 2;
   const V *c = (const V *)coef, *f = (const V *)fields;
   T *o = (T *)out;
   // Launched plainly: set up early, its blocks join an SM that still runs the kernel
   // before it, and keep that kernel's division into shared memory and L1.  Behind a trial FP64
   // redo with 5 resident blocks per SM (small L1) the 1M jet step took 2616 us, 1948 so.
   if (G == 4) {
-    MAFP_TIMED(ctx, s, "k_apply<G=4>", (k_apply<T, 4, U><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, f, o)));
+    MAFP_TIMED(ctx, s, "k_apply<G=4>", (k_apply<T, 4, U><<<blocks, kApplyThreads<T>, 0, s>>>(n, rp, col, c, f, o)));
   } else if (G == 16) {
-    MAFP_TIMED(ctx, s, "k_apply<G=16>", (k_apply<T, 16, U><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, f, o)));
+    MAFP_TIMED(ctx, s, "k_apply<G=16>", (k_apply<T, 16, U><<<blocks, kApplyThreads<T>, 0, s>>>(n, rp, col, c, f, o)));
   } else {
-    MAFP_TIMED(ctx, s, "k_apply<G=8>", (k_apply<T, 8, U><<<blocks, kApThreads, 0, s>>>(n, rp, col, c, f, o)));
+    MAFP_TIMED(ctx, s, "k_apply<G=8>", (k_apply<T, 8, U><<<blocks, kApplyThreads<T>, 0, s>>>(n, rp, col, c, f, o)));
   }
 }
 
