@@ -1,7 +1,6 @@
 """Autotuner of the launch shapes: the neighbour search's cell tile (cell edge
 in percent of max h) and the lanes per particle / per row of classify_pca,
-build_stencils (film rows; the library chooses 3D rows' by size), apply_ops and
-the stencil adjoint.
+build_stencils, apply_ops and the stencil adjoint.
 
 For a cloud already on the device it times every supported group size of a
 stage with CUDA events (a few repetitions, best taken), keeps the fastest,
@@ -19,8 +18,8 @@ import torch
 from . import mafp as M
 
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "tuning.json")
-CHOICES = {"stencil2d_group": (4, 8, 16), "apply_group": (4, 8, 16),
-           "grad3d_group": (2, 4, 8, 16, 32),
+CHOICES = {"stencil3d_group": (8, 16, 32), "stencil2d_group": (4, 8, 16),
+           "apply_group": (4, 8, 16), "grad3d_group": (2, 4, 8, 16, 32),
            "grad2d_group": (1, 2, 4, 8, 16), "cell_edge_pct": (100, 115, 130),
            "classify_group": (1, 2, 4, 8, 16)}
 
@@ -78,12 +77,13 @@ def tune(ctx: M.Context, pipe, d, use_cache: bool = True, verbose: bool = False)
     timings["classify_group"] = res
     ctx.set_tuning(**best)
     pipe.classify(d)
-    res = {}
-    for g in CHOICES["stencil2d_group"]:
-        ctx.set_tuning(**{**best, "stencil2d_group": g})
-        res[g] = _time(lambda: pipe.stencils(d))
-    best["stencil2d_group"] = min(res, key=res.get)
-    timings["stencil2d_group"] = res
+    for knob in ("stencil3d_group", "stencil2d_group"):
+        res = {}
+        for g in CHOICES[knob]:
+            ctx.set_tuning(**{**best, knob: g})
+            res[g] = _time(lambda: pipe.stencils(d))
+        best[knob] = min(res, key=res.get)
+        timings[knob] = res
     ctx.set_tuning(**best)
     pipe.stencils(d)
     res = {}

@@ -1,7 +1,7 @@
 // stencil.cu -- GFDM stencils of Eq. GFDM_Definition (Sec. 2.3), order 2.
 //
-// One group of G lanes per particle (8 for 3D rows of ~180 entries, 4 for film
-// rows of ~40).  Lanes stride over the row, accumulate the distinct moments of
+// One group of G lanes per particle (8 or more for 3D rows of ~180 entries, 4 or
+// more for film rows of ~40).  Lanes stride over the row, accumulate the distinct moments of
 // A = sum_j w_j p_j p_j^T, reduce them with a reduce-scatter of shuffles, factor
 // A (Cholesky) and solve for the four right-hand sides, one per lane.
 // FP32 path: one refinement step with the residual b - sum_j c_j p_j of the
@@ -674,31 +674,33 @@ static void launch_stencil(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void 
                  sp, ctx->d_status, ctx->fallback, rounds));
 }
 
-// Lanes per particle.  3D: 8 whatever the context's stencil3d_group asks for: more
-// lanes repeat the factorisation and leave part of a row's last gather empty (440k
-// rows: 951 us, with 32 lanes 2136).  Clouds whose rows do not fill the GPU take
-// 32 (5650 particles: 21 us against 25).  Film, FP32: the context's
-// stencil2d_group, which also sets the order of the sums: the Laplacians of a
-// curved film are small differences, and gradients taken through them show every
-// change of rounding.  Film, FP64: 4 lanes, for the factorisation (697 us with 8,
-// 461 with 4 on the 60k jet cloud).
+// Lanes per particle: the context's stencil3d_group and stencil2d_group, whose default
+// values 32 (3D) and 8 (film, FP64) leave the choice to the size.  More lanes repeat the
+// factorisation and leave part of a row's last gather empty, fewer leave the GPU idle
+// where rows are few.  3D, FP32, 8 / 16 / 32 lanes: cube 4852 particles 40 / 32 / 36 us,
+// 10k 45 / 45 / 50, 20k 59 / 60 / 76, 80k 164 / 193 / 275; FP64, jet on a film, 10k 255 /
+// 208 / 202 us, 16k 374 / 331 / 337, 40k 677 / 650 / 737; cube 5k 292 / 332 / 334, 20k
+// 924 / 996 / 1310.  By default 32 up to kStFewRows (jets in FP64 want them there, cubes
+// from 8k on would take 8), 8 beyond.  Film, FP32: 8, which also sets the order of the
+// sums: the Laplacians of a curved film are small differences, and gradients taken
+// through them show every change of rounding.  Film, FP64, 4 / 8 / 16 lanes: 16k 181 / 202 /
+// 287 us, 80k 709 / 869 / 1290.
 template <typename TS, typename C, bool REFINE>
 static int dispatch_stencils(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void *pos_h,
                              const uint8_t *model, const void *frame, const long long *rp,
                              const int32_t *col, void *coef, uint8_t *status, float *cond,
                              const StParams<C> &sp) {
-  if (n <= kStFewRows)
-    launch_stencil<TS, C, 10, 32, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp);
-  else
-    launch_stencil<TS, C, 10, 8, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp);
-  switch (sizeof(C) == 8 ? (n <= kStFewRows ? 8 : 4) : ctx->tune.stencil2d_group) {
+  int g3 = ctx->tune.stencil3d_group, g2 = ctx->tune.stencil2d_group;
+  if (g3 == 32 && n > kStFewRows) g3 = 8;
+  if (sizeof(C) == 8 && g2 == 8 && n > kStFewRows) g2 = 4;
+  switch (g3) {
+    case 8: launch_stencil<TS, C, 10, 8, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
+    case 16: launch_stencil<TS, C, 10, 16, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
+    default: launch_stencil<TS, C, 10, 32, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
+  }
+  switch (g2) {
     case 4: launch_stencil<TS, C, 6, 4, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
-    case 16:
-      if constexpr (sizeof(C) == 4) {
-        launch_stencil<TS, C, 6, 16, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp);
-        break;
-      }
-      [[fallthrough]];
+    case 16: launch_stencil<TS, C, 6, 16, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
     default: launch_stencil<TS, C, 6, 8, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
   }
   MAFP_LAUNCH_CHECK(ctx);
