@@ -264,15 +264,6 @@ struct KernelName {
   }
 };
 
-// One bit per device (devices 0..63): set once a per-device, per-function
-// setting (such as a dynamic shared-memory limit) has been applied there.
-// Returns true when the caller still has to apply it on `dev`.
-inline bool first_on_device(unsigned long long *mask, int dev) {
-  if (dev < 0 || dev >= 64) return true;
-  const unsigned long long bit = 1ull << dev;
-  return (__atomic_fetch_or(mask, bit, __ATOMIC_ACQ_REL) & bit) == 0;
-}
-
 constexpr int kProfCap = 4096;
 
 // Bracket one kernel launch with CUDA events on its stream when profiling is on.

@@ -663,11 +663,7 @@ static void launch_stencil(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void 
   static_assert(G >= 4, "a warp looks at 32 particles at most");
   const int blocks = (int)((n + (int64_t)rounds * kBuildThreads / G - 1) / (rounds * kBuildThreads / G));
   constexpr int smem = StCache<C, M, G>::SMEM;
-  // the dynamic shared-memory limit is a per-device setting of the function
-  static unsigned long long attr_devices = 0;
-  if (smem > 48 * 1024 && first_on_device(&attr_devices, ctx->device))
-    cudaFuncSetAttribute(k_stencil<TS, C, M, G, REFINE>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  static_assert(smem <= 48 * 1024, "more has to be asked for, per device and function");
   MAFP_TIMED(ctx, s, name.s,
              launch(k_stencil<TS, C, M, G, REFINE>, blocks, kBuildThreads, smem, s, 
                  n, (const V *)pos_h, model, (const V *)frame, rp, col, (V *)coef, status, cond,
