@@ -17,19 +17,21 @@ namespace mafp {
 constexpr int64_t kStFewRows = 16384;
 
 // Rounds of rows per warp.  More share a warp's start and its last, partly filled round,
-// but leave the GPU idle where few warps hold rows of the model: a column of 3D rows in a
-// wide film keeps its rows in few warps.  Whole builds with 1 / 2 / 4 rounds, us --
-//   3D: jet on a film, 66k particles 85 / 102 / 129, 131k 152 / 159 / 180, 262k 296 / 291 /
-//   305, 1M 1234 / 1152 / 1146; cube 131k 270 / 267 / 288, 262k 528 / 512 / 534, 517k 1029 /
-//   1002 / 1016;
-//   film: 30k 40 / 41 / 41, 66k 64 / 59 / 63, 131k 108 / 98 / 96, 262k 198 / 178 / 172.
+// and leave fewer warps that find no row of the model; but where the rows lie in few warps
+// (a column of 3D rows in a wide film) the others are idle.  Whole builds, us, with 1 / 2 /
+// 4 rounds --
+//   3D (film rounds as below): jet on a film, 70k particles 82 / 93 / 116, 141k 147 / 155 /
+//   167, 180k 185 / 185 / 197, 1M 1234 / 1152 / 1146; cube 70k 144 / 146 / 171, 142k 274 /
+//   283 / 304, 178k 338 / 344 / 360, 517k 1029 / 1002 / 1016; a film alone, whose 3D pass
+//   finds nothing, 160k 111 / 106 / 102;
+//   film: 70k 57 / 56 / 61, 131k 96 / 94 / 95, 230k 150 / 145 / 146, 1M 704 / 619 / 583.
 // FP64 (its pipe is full with few warps, and uneven warps are its time): jet 66k 1081 /
 // 1265 / 1692, cube 134k 5774 / 5919 / 6347, film 131k 1116 / 1146 / 1149.
 template <typename C, int M>
 static int rounds_of(int64_t n) {
   if (sizeof(C) == 8) return 1;
-  if (M == 10) return n > 196608 ? 2 : 1;
-  return n > 131072 ? 4 : (n > 65536 ? 2 : 1);
+  if (M == 10) return n > 163840 ? 2 : 1;
+  return n > 262144 ? 4 : (n > 65536 ? 2 : 1);
 }
 
 // Two warps per block: a block's slot is free again as soon as its two warps'

@@ -37,9 +37,9 @@ def _build_us(cloud, dtype):
 
 @pytest.mark.parametrize("dtype", [M.F32_REFINED, M.F64])
 @pytest.mark.parametrize("shape", ["jet", "cube"])
-@pytest.mark.parametrize("n", [16384, 65536, 131072, 196608])
+@pytest.mark.parametrize("n", [16384, 65536, 163840, 262144])
 def test_build_time_has_no_step(n, shape, dtype):
-    if dtype == M.F64 and n > 131072:
+    if dtype == M.F64 and n > 65536:
         pytest.skip("FP64 has no switch there")
     if shape == "jet":
         c = C.cell_sorted(C.jet_on_plate(None, n + n // 20))
