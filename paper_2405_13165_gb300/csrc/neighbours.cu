@@ -731,7 +731,11 @@ __global__ void __launch_bounds__(kNbrThreads) k_nbr(
 // The bits go to a pool, P rows of nwords (rounded up to 4) per cell (pool_words
 // in all, kMaskWords per particle of the context's capacity on average): film
 // cells need 4 words per particle, cells of an irregular cloud 60, and only what
-// exceeds the pool takes the warp-per-particle kernels.
+// exceeds the pool takes the warp-per-particle kernels.  So does a cell that alone would
+// take more than a 64th of the pool (or 1 MB, if that is more): a few such cells (a
+// clump, a dense patch) would use it up, and the cells left over would crowd the heavy
+// ones in those kernels (80k film particles with 120k in a dense patch, FP64: 584 to 752
+// ms, as the cells came, 573 where only the patch's cells take them).
 constexpr int kMaskThreads = 128;
 constexpr int kMaskWarps = kMaskThreads / 32;
 constexpr int kWinWords = 8;
@@ -739,6 +743,10 @@ constexpr int kMaskBlock = 64;   // particles prepared at a time
 constexpr float kBand = 1.6e-5f;
 // Words of a particle's row in the mask pool.
 __host__ __device__ constexpr int row_words(int total) { return ((total + 127) >> 7) << 2; }
+
+__host__ __device__ constexpr long long cell_limit(long long pool_words) {
+  return pool_words / 64 > (1 << 18) ? pool_words / 64 : (1 << 18);
+}
 
 constexpr int kFillThreads = 128;
 constexpr int kFillWarps = kFillThreads / 32;
@@ -825,7 +833,8 @@ __global__ void __launch_bounds__(128) k_cell_table(
       rec[kRecP] = P;
       rec[kRecTotal] = total;
       rec[kRecRuns] = nr | ((max(-120, min(120, e)) + 128) << 8);
-      if (abs(e) <= 120) need = (long long)row_words(total) * P;
+      need = (long long)row_words(total) * P;
+      if (abs(e) > 120 || need > cell_limit(pool_words)) need = 0;
     }
     // the warp's share of the pool, by one atomic
     long long inc = need;
@@ -839,7 +848,7 @@ __global__ void __launch_bounds__(128) k_cell_table(
     base = __shfl_sync(0xffffffffu, base, 31) + inc - need;
     if (!in) continue;
     if (need == 0 || base + need > pool_words) {
-      // an edge out of range, or the pool is used up
+      // an edge out of range, a cell beyond its share, or the pool is used up
       base = -1;
       overflow[atomicAdd(n_ucell + 1, 1)] = t;
     }
