@@ -33,6 +33,7 @@ int remap_switched(mafp_ctx *, int64_t, int32_t, const mafp_state *, const uint8
                    const int64_t *, const int32_t *, const mafp_state *, int64_t, int32_t *,
                    int64_t *, cudaStream_t);
 void init_kernel_attributes();
+void init_apply_attributes();
 int ghost_sources(mafp_ctx *, int64_t, const uint8_t *, const int64_t *, const int32_t *,
                   uint8_t *, cudaStream_t);
 int film_momentum(mafp_ctx *, int64_t, int32_t, const uint8_t *, void *, const void *,
@@ -182,6 +183,7 @@ int mafp_create(mafp_ctx **out, const mafp_params *params, int64_t cap_particles
     return MAFP_ECUDA;
   }
   init_kernel_attributes();
+  init_apply_attributes();
   *out = ctx;
   return MAFP_OK;
 }

@@ -193,18 +193,20 @@ __global__ void __launch_bounds__(kApThreads) k_apply_T_scatter(int64_t n,
   }
 }
 
+// Entries in flight per lane.
+template <typename T> constexpr int kApplyU = sizeof(T) == 4 ? 8 : 2;
+
 template <typename T>
 static void launch_apply(mafp_ctx *ctx, cudaStream_t s, int64_t n, const long long *rp,
                          const int32_t *col, const void *coef, const void *fields, void *out) {
   using V = vec4_t<T>;
   const int G = ctx->tune.apply_group;
   const int blocks = grid_for(n * G, kApplyThreads<T>, sm_count() * 64);
-  constexpr int U = sizeof(T) == 4 ? 8 : 2;
+  constexpr int U = kApplyU<T>;
   const V *c = (const V *)coef, *f = (const V *)fields;
   T *o = (T *)out;
-  // Launched plainly: set up early, its blocks join an SM that still runs the kernel
-  // before it, and keep that kernel's division into shared memory and L1.  Behind a trial FP64
-  // redo with 5 resident blocks per SM (small L1) the 1M jet step took 2616 us, 1948 so.
+  // (launched plainly: nothing is gained by setting its blocks up early, 1950 us for the
+  // 1M jet step and 1945 us so)
   if (G == 4) {
     MAFP_TIMED(ctx, s, "k_apply<G=4>", (k_apply<T, 4, U><<<blocks, kApplyThreads<T>, 0, s>>>(n, rp, col, c, f, o)));
   } else if (G == 16) {
@@ -212,6 +214,27 @@ static void launch_apply(mafp_ctx *ctx, cudaStream_t s, int64_t n, const long lo
   } else {
     MAFP_TIMED(ctx, s, "k_apply<G=8>", (k_apply<T, 8, U><<<blocks, kApplyThreads<T>, 0, s>>>(n, rp, col, c, f, o)));
   }
+}
+
+// k_apply wants all of the L1 for its gathers.  Without a preference its blocks take the
+// division into shared memory and L1 that an SM has, and keep it while another kernel's
+// blocks are on that SM: beside the tail of a remap on a second stream, behind a build
+// whose blocks leave little L1, the 1M jet's build and application took 1.67 ms, 1.53 or
+// 1.41 by the build's launch shape, 1.40 ms so whichever it is (the whole step with both
+// adjoints 4.33, 4.25 and 4.14 ms, 4.09 so; with 1.5M particles 6.55 -> 6.30 ms).
+// Per device, like every attribute of a function.
+template <typename T, int G>
+static void prefer_l1() {
+  cudaFuncSetAttribute(k_apply<T, G, kApplyU<T>>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                       cudaSharedmemCarveoutMaxL1);
+}
+void init_apply_attributes() {
+  prefer_l1<float, 4>();
+  prefer_l1<float, 8>();
+  prefer_l1<float, 16>();
+  prefer_l1<double, 4>();
+  prefer_l1<double, 8>();
+  prefer_l1<double, 16>();
 }
 
 template <typename T>
