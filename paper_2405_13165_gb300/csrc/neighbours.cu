@@ -1,8 +1,10 @@
 // neighbours.cu -- fixed-radius neighbour search of Eq. Nbd (Sec. 2.2) on a
-// cell list: bounding box -> cell keys -> stable LSD radix sort -> cell ranges
-// -> count (one block per occupied cell, candidate tiles staged in shared
-// memory) -> exclusive scan -> fill -> (row sort when the input order is not
-// the cell order) ; plus the transpose map used by the apply adjoint.
+// cell list: bounding boxes -> cell keys -> stable LSD radix sort (left out for a
+// cloud in cell order) -> cell ranges and work queue -> a record per occupied cell
+// -> hit bits of its candidates (a warp per cell or part of one) -> exclusive scan
+// -> fill from the bits -> (row sort when the input order is not the cell order) ;
+// cells that the bits' pool cannot hold are counted and filled a warp per particle.
+// Plus the transpose map used by the apply adjoint.
 #include <algorithm>
 #include <climits>
 
@@ -445,7 +447,9 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
 // The whole sort of a small cloud in one block: the passes that its number of cells
 // needs, each a histogram, a scan of it and a stable scatter in chunks of 1024.
 // (Eight launches less; a launch costs the host ~3 us, which bounds the step of a
-// cloud of a few thousand particles.)  The result is in keys_b / vals_b.
+// cloud of a few thousand particles.)  Cell order of an unordered 3D cloud: 4096 particles
+// 41 us, 8192 61 us; by passes over the whole GPU 8193 take 68 us, 16384 70 us.  The
+// result is in keys_b / vals_b.
 constexpr int64_t kSmallSort = 8192;
 __global__ void __launch_bounds__(1024) k_sort_small(uint32_t *keys_a, int32_t *vals_a,
                                                      uint32_t *keys_b, int32_t *vals_b, int n,
@@ -1403,7 +1407,10 @@ static int build_neighbours_t(mafp_ctx *ctx, int64_t n, int nb, const long long 
   // fill at 5650 particles 71 + 134 us unsplit, 24 + 23 us in these parts); in
   // larger ones only the costly cells are split, so that no warp ends late
   // (200k random particles, mask + fill: 535 us unsplit, 438 in halves, 366 in
-  // quarters; the 1M jet cloud 423, 398 and 462 us).
+  // quarters; the 1M jet cloud 423, 398 and 462 us).  The lines follow such uneven
+  // clouds; in even ones the parts cost a little just below them (whole search, on
+  // either side of 131072: 3D in cell order 228 and 201 us, FP64 471 and 324, film 121
+  // and 113; of 524288: 506 and 441, 992 and 667, 188 and 188).
   const Split split = n <= kSplitAll ? Split{3, 1} : n <= kSplitMore ? Split{2, 0} : Split{1, 0};
   const long long *rp = reinterpret_cast<const long long *>(row_ptr);
   MAFP_TIMED(ctx, s, "k_cell_table",

@@ -63,12 +63,13 @@ template <int M> constexpr int kGatherU = M == 10 ? 4 : 2;
 // right-hand sides (the coefficients of one entry side by side: lambda_k stays
 // in registers once); the moment pass packs the weights and coordinates of two
 // entries.
-// What bounds it (3D, ncu on 300k particles): ~6000 instructions per round of
-// four rows, 57 % of them FP32; the FMA pipe is busy ~60 % of the time (a packed
-// FMA with three different operands takes 3 cycles of it, measured) at 14 warps
-// per SM, the registers' limit.  Film rows: L1 wavefronts (56 % busy) and issue
-// (53 %).  1M jet cloud, 3D 890 -> 759 us, film 300 -> 257 us; with the launch
-// shapes of a new context (32 and 8 lanes before) 2136 -> 909 us for 440k 3D rows.
+// What bounds it (ncu, jet cloud of 303k particles): 3D, ~6000 instructions per round
+// of four rows; the FMA pipe is 51 % busy (a packed FMA with three different operands
+// takes 3 cycles of it, measured) and 56 % of the cycles issue, at 13.9 warps per SM of the
+// 16 that registers (128) and shared memory (26 KB a block) both allow; an instruction
+// waits 1.25 cycles on fixed latencies and 1.14 on its gathers.  Film (4 lanes): issue 58 %,
+// FMA pipe 43 %, 16.7 warps of 20 (96 registers).  1M jet cloud, 3D 890 -> 746 us, film
+// 300 -> 256 us; with the launch shapes of a new context 2136 -> 889 us for 440k 3D rows.
 __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -293,7 +294,7 @@ __device__ __forceinline__ void stencil_row32(int64_t i, const float4 *pos, cons
   auto dots = [&](const float2 (&p)[M], float2 &s01, float2 &s2x) {
     if constexpr (M == 10) {
       // nested: the coefficient pass needs no products then, and three short
-      // chains replace one of nine (951 -> 909 us)
+      // chains replace one of nine (951 -> 909 us for 440k rows)
       auto poly = [&](const float2 (&l)[M]) {
         const float2 a = fma2(p[1], l[4], fma2(p[2], l[7], fma2(p[3], l[8], l[1])));
         const float2 b = fma2(p[2], l[5], fma2(p[3], l[9], l[2]));

@@ -199,13 +199,18 @@ __device__ __forceinline__ void static_for(F &&f) {
 // pivot is <= tol.  invd gets 1/L_kk; pmin / pmax the extreme pivots.  (Written
 // with loops under "#pragma unroll" the 6 x 6 case kept run-time indices, a
 // compare and a select per candidate register: 710 instructions per warp instead
-// of 200, a fifth of the film build.)  NEWTON: reciprocal root (in FP32 with one Newton
-// step), eight operations in every lane of the group against about twenty-five of
-// a square root and a division; for the build, whose refinement corrects what
-// the last bit of a pivot changes -- the adjoint, unrefined, keeps the exact ones
-// (rounded differently its film gradients move by as much as their own error,
-// 2e-5).
-template <int M, typename C, bool NEWTON = false>
+// of 200, a fifth of the film build.)
+// RECIP: reciprocal roots, eight operations in every lane of the group against about
+// twenty-five of a square root and a division.  FP32, 3D: rsqrtf with one Newton step; the
+// build's refinement corrects what the last bit of a pivot changes.  (The adjoint and the
+// film build, whose gradients move by as much as their own error, 2e-5, with it, keep the
+// exact ones.)  FP64 has no refinement and takes rsqrt as it is: the factor, its
+// reciprocal and the solves all use the one rounded root, and the coefficients come out
+// no less accurate -- against 80-bit arithmetic, 3D and film rows of condition 4e2 to
+// 8e11, error over the row's largest coefficient: mean 1.8e-15 to 4.1e-15, largest 3.2e-14
+// (square root and division: 2.0e-15 to 4.8e-15, 4.8e-14; a Newton step on top: 1.9e-15 to
+// 4.8e-15, 4.7e-14).
+template <int M, typename C, bool RECIP = false>
 __device__ __forceinline__ bool cholesky(C (&L)[Basis<M>::NA], C (&invd)[M], C tol, C &pmin,
                                          C &pmax) {
   pmin = C(INFINITY);
@@ -221,7 +226,7 @@ __device__ __forceinline__ bool cholesky(C (&L)[Basis<M>::NA], C (&invd)[M], C t
     ok = ok && (d > tol);
     const C dd = d > tol ? d : C(1);
     C lkk;
-    if constexpr (NEWTON) {
+    if constexpr (RECIP) {
       C y;
       if constexpr (sizeof(C) == 4) {
         y = rsqrtf(dd);
