@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kClsThreads, sizeof(T) == 4 ? 8 : 1) k_classif
     const vec4_t<T> *normal, const T *vol, const T *h3d, const uint8_t *user,
     const long long *row_ptr, const int32_t *col, uint8_t *preflag, vec4_t<T> *eig,
     vec4_t<T> *frame, T *hfilm, uint8_t *near, mafp_params prm, ClsConst kc, DevStatus *st) {
-  pdl_wait();
+  pdl_sync();
   using V = vec4_t<T>;
   const int lane = threadIdx.x & (G - 1);
   const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;

@@ -203,6 +203,11 @@ template <typename T> __device__ __forceinline__ bool finite_(T x) { return isfi
 // have started.  Not for a kernel that writes 4-vectors or other real arrays: ld4 and
 // __ldg take the non-coherent path, for data that nobody writes while the reading kernel
 // is resident, and the next kernel (of this call or of any other) may read them so.
+// Four do nevertheless, because the one kernel that follows them reads nothing of theirs
+// by that path: k_classify (k_smooth), k_survivors (k_to2d), k_to2d (k_append, which like
+// k_to2d reads the state that comes in) and k_cells (k_cell_table; its sorted positions
+// are read by the kernels after that one).  Small transitions show it: 20000-particle jet
+// 84.1 us waiting, 82.5 us so.
 //   pdl_wait() leaves the set-up to the end of this kernel's last block.  Also where the
 // next kernel has few blocks with work, or is bound by the FP64 pipe: set up beside a
 // kernel that still runs, its blocks pile up on the SMs that have room (the search of

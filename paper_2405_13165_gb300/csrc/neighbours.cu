@@ -543,7 +543,7 @@ __global__ void __launch_bounds__(kCellThreads) k_cells(
     const uint32_t *keys, const uint32_t *keys0, int32_t *svals, int64_t n,
     const vec4_t<T> *pos, vec4_t<T> *spos, int32_t *cell_start, int32_t *cell_end,
     int32_t *ucell, int32_t *n_ucell, int32_t *order, const DevStatus *st, const GridDev *g) {
-  pdl_wait();
+  pdl_sync();
   __shared__ int s_cnt[2][kCellThreads / 32 + 1];
   if (!g->ok) return;
   const bool moved = st->not_identity;

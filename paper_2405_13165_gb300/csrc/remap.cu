@@ -200,7 +200,7 @@ template <typename T>
 __global__ void k_survivors(int64_t n, StateT<T> in, StateT<T> out, const uint8_t *flag,
                             const int32_t *owner, const long long *keep_scan,
                             const int32_t *gam, int32_t *old2new, const DevStatus *st) {
-  pdl_wait();
+  pdl_sync();
   const bool skip = st->remap_scratch[0] != 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -248,7 +248,7 @@ __global__ void k_to2d(StateT<T> in, StateT<T> out, const int32_t *owner,
                        const long long *keep_scan, const long long *row_ptr, const int32_t *col,
                        const DevStatus *st, const int32_t *flagged,
                        const unsigned long long *n_flagged) {
-  pdl_wait();
+  pdl_sync();
   if (st->remap_scratch[0] != 0) return;
   const int lane = threadIdx.x & 31;
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;

@@ -49,11 +49,33 @@ def test_every_kernel_waits_first():
         assert re.match(r"\{\s*pdl_(sync|wait)\(\);", body), (path, name)
 
 
+# writers that do, with the kernel that always follows and what that one may read by ld4
+FOLLOWED = {"k_classify": ("k_smooth", None), "k_survivors": ("k_to2d", r"in\."),
+            "k_to2d": ("k_append", r"in\."), "k_cells": ("k_cell_table", None)}
+
+
+def test_followers_read_nothing_of_theirs_non_coherently():
+    bodies = {name: body for _, name, _, body in _kernels()}
+    for follower, allowed in FOLLOWED.values():
+        assert "__ldg" not in bodies[follower]
+        for arg in re.findall(r"\bld4\(\s*([^,]*?)\)", bodies[follower]):
+            assert allowed and re.match(allowed, arg), (follower, arg)
+    # the launches are in that order: nothing is launched between the two
+    for first, (follower, _) in FOLLOWED.items():
+        if first == "k_cells":    # the last kernel of the sort; the search goes on with the other
+            continue
+        src = "".join(open(p).read() for p in sorted(glob.glob(os.path.join(CSRC, "*.cu"))))
+        tail = src[[m.end() for m in re.finditer(r"\blaunch\(\s*" + first + r"\b", src)][-1]:]
+        assert re.search(r"\blaunch\(\s*(k_\w+)", tail).group(1) == follower, first
+
+
 def test_writers_of_real_arrays_do_not_trigger_early():
     seen = set()
     for path, name, params, body in _kernels():
         if _writes_real(params):
             seen.add(name)
+            if name in FOLLOWED:
+                continue
             assert "pdl_sync()" not in body and "launch_dependents" not in body, (path, name)
     # the parameters are recognised: the operators, the states and the step's frames
     assert {"k_stencil", "k_stencil_redo", "k_stencil_grad", "k_apply", "k_apply_T_scatter",
