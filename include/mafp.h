@@ -83,11 +83,12 @@ typedef struct {
  * particle or row.  Every value gives the same results up to rounding order;
  * the autotuner picks the fastest for a cloud's population mix. */
 typedef struct {
-  int32_t stencil3d_group; /* lanes per 3D particle in mafp_build_stencils: 8 or 16; 32 (the
-                              default) leaves the choice to the library, which takes 32 for
-                              clouds of at most 16384 particles and 8 beyond */
-  int32_t stencil2d_group; /* lanes per 2D particle in mafp_build_stencils: 4, 8 or 16; in FP64
-                              8 (the default) stands for 4 beyond 16384 particles */
+  int32_t stencil3d_group; /* lanes per 3D particle in mafp_build_stencils for clouds of more than
+                              16384 particles: 8 or 16; 32 (the default) leaves the choice to
+                              the library (8).  Smaller clouds take 32 */
+  int32_t stencil2d_group; /* lanes per 2D particle in mafp_build_stencils: 4, 8 or 16.  In FP64
+                              for clouds of more than 16384 particles, where 8 (the default)
+                              stands for 4; smaller ones take 8 */
   int32_t apply_group;     /* lanes per row in mafp_apply_ops / _backward: 4, 8 or 16 */
   int32_t grad3d_group;    /* lanes per 3D particle in mafp_build_stencils_backward: 2, 4,
                               8, 16 or 32 (the FP64 adjoint takes at least 8) */

@@ -673,25 +673,28 @@ static void launch_stencil(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void 
                  sp, ctx->d_status, ctx->fallback, rounds));
 }
 
-// Lanes per particle: the context's stencil3d_group and stencil2d_group, whose default
-// values 32 (3D) and 8 (film, FP64) leave the choice to the size.  More lanes repeat the
-// factorisation and leave part of a row's last gather empty, fewer leave the GPU idle
-// where rows are few.  3D, FP32, 8 / 16 / 32 lanes: cube 4852 particles 40 / 32 / 36 us,
-// 10k 45 / 45 / 50, 20k 59 / 60 / 76, 80k 164 / 193 / 275; FP64, jet on a film, 10k 255 /
-// 208 / 202 us, 16k 374 / 331 / 337, 40k 677 / 650 / 737; cube 5k 292 / 332 / 334, 20k
-// 924 / 996 / 1310.  By default 32 up to kStFewRows (jets in FP64 want them there, cubes
-// from 8k on would take 8), 8 beyond.  Film, FP32: 8, which also sets the order of the
-// sums: the Laplacians of a curved film are small differences, and gradients taken
-// through them show every change of rounding.  Film, FP64, 4 / 8 / 16 lanes: 16k 181 / 202 /
-// 287 us, 80k 709 / 869 / 1290.
+// Lanes per particle.  Clouds of more than kStFewRows: the context's stencil3d_group and
+// stencil2d_group, whose default values stand for 8 (3D's 32) and, in FP64, for 4 (film's
+// 8).  More lanes repeat the factorisation and leave part of a row's last gather empty --
+// 3D, FP32, 8 / 16 / 32 lanes: cube of 20k particles 59 / 60 / 76 us, 80k 164 / 193 / 275;
+// FP64, cube 20k 924 / 996 / 1310, jet on a film 40k 677 / 650 / 737; film, FP64, 4 / 8 / 16
+// lanes: 20k 216 / 244 / 348, 80k 709 / 869 / 1290.  Smaller clouds, whose rows do not fill
+// the GPU: 32 lanes in 3D and, in FP64, 8 on film, whatever is asked for (FP32, cube 4852
+// 40 / 32 / 36 us, 10k 45 / 45 / 50; FP64, jet 10k 255 / 208 / 202, cube 5k 292 / 332 / 334);
+// their sums are shorter chains too: with 8 and 4 lanes the FP64 outputs lie 0 to 5 %
+// further from the exact ones (film 6000 particles 6.7e-15 for 6.4e-15).  Film, FP32:
+// always as asked for; the lanes set the order of the sums there, and the Laplacians of a
+// curved film are small differences, whose gradients show every change of rounding.
 template <typename TS, typename C, bool REFINE>
 static int dispatch_stencils(mafp_ctx *ctx, cudaStream_t s, int64_t n, const void *pos_h,
                              const uint8_t *model, const void *frame, const long long *rp,
                              const int32_t *col, void *coef, uint8_t *status, float *cond,
                              const StParams<C> &sp) {
+  const bool few = n <= kStFewRows;
   int g3 = ctx->tune.stencil3d_group, g2 = ctx->tune.stencil2d_group;
-  if (g3 == 32 && n > kStFewRows) g3 = 8;
-  if (sizeof(C) == 8 && g2 == 8 && n > kStFewRows) g2 = 4;
+  if (few) g3 = 32;
+  else if (g3 == 32) g3 = 8;
+  if (sizeof(C) == 8) g2 = few ? 8 : (g2 == 8 ? 4 : g2);
   switch (g3) {
     case 8: launch_stencil<TS, C, 10, 8, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;
     case 16: launch_stencil<TS, C, 10, 16, REFINE>(ctx, s, n, pos_h, model, frame, rp, col, coef, status, cond, sp); break;

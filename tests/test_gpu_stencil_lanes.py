@@ -1,6 +1,7 @@
-"""The lanes per row that a caller asks for are the lanes that the stencil build takes
-(the names of its kernels say them), with the oracle's coefficients; the defaults leave
-them to the library."""
+"""The lanes per row that a caller asks for are the lanes that the stencil build takes in
+clouds of more than 16384 particles (the names of its kernels say them), and on film in
+FP32 always, with the oracle's coefficients; the defaults, and smaller clouds, leave them to
+the library."""
 import numpy as np
 import pytest
 
@@ -22,13 +23,18 @@ def _first(cloud, n):
 
 CLOUDS = {
     "small": lambda: C.config_small(),
-    # 3D rows on either side of the size at which the defaults change
+    # 3D rows on either side of that size
     "16384": lambda: _first(C.jet_on_plate(None, 17_500), 16384),
     "16385": lambda: _first(C.jet_on_plate(None, 17_500), 16385),
 }
-# asked for -> taken below and beyond that size
-DEFAULT = {M.F32_REFINED: {(32, 8): ((32, 8), (8, 8))}, M.F32_PLAIN: {(32, 8): ((32, 8), (8, 8))},
-           M.F64: {(32, 8): ((32, 8), (8, 4))}}
+
+
+def _taken(asked, n, dtype):
+    if n <= 16384:
+        return 32, 8 if dtype == M.F64 else asked[1]
+    return {32: 8}.get(asked[0], asked[0]), 4 if dtype == M.F64 and asked[1] == 8 else asked[1]
+
+
 ASKED = [(8, 4), (16, 16), (16, 4), (8, 16), (32, 8)]
 
 
@@ -45,8 +51,7 @@ def test_lanes_asked_for_are_taken(orc, name, dtype):
         g, *_ = run_gpu(c, dtype, ctx=ctx, cap_nnz=int(rp[-1]) + 8, stages=("nbr", "cls", "st"))
         names = ctx.profile_read()
         ctx.profile(False)
-        taken = DEFAULT[dtype].get(lanes, (lanes, lanes))[c.n > 16384]
-        for model, k in zip((10, 6), taken):
+        for model, k in zip((10, 6), _taken(lanes, c.n, dtype)):
             assert any(f"k_stencil<" in s and f"M={model},G={k}," in s for s in names), (lanes, names)
         assert g["status_block"]["code"] == 0
         np.testing.assert_array_equal(g["status"] == M.STENCIL_DEFICIENT, status != 0)
